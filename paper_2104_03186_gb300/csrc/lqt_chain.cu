@@ -72,7 +72,7 @@ lqt_status fold_slots(const ChainVariant& v, long long* slots) {
                              (int)smem) != cudaSuccess)
         return LQT_ECUDA;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.fold_kernel(),
-                                                      v.fold_groups() * v.n, smem) != cudaSuccess)
+                                                      v.fold_threads(), smem) != cudaSuccess)
         return LQT_ECUDA;
     *slots = (long long)sms * (per_sm > 0 ? per_sm : 1) * v.fold_groups();
     return LQT_OK;

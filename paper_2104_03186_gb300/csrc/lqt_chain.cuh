@@ -46,66 +46,16 @@
 
 #include <cuda_runtime.h>
 
+#include "lqt_chain_args.cuh"
 #include "lqt_lane_step.cuh"
 #include "lqt_refine.cuh"
+#include "lqt_team_chain.cuh"
 #include "lqt_tma.cuh"
 
 namespace lqt {
 namespace chain {
 
 using namespace lanes;
-
-constexpr int kStatusSingular = 8;  // LQT_ESINGULAR
-
-template <typename R>
-struct Item {
-    DescT<R> D;
-    long long B;   // steps per chunk
-    long long c0;  // first chunk in the chunk arrays (a multiple of NC)
-    long long r0;  // first row of the residual kernel's index space (T + 1 rows each)
-    int NC;        // chunks (a power of two)
-    int pad_;
-    R* u_out;      // correction pass: the output u* (holds u^ until then)
-    const R* qh;   // correction pass: U^{-1} h_k (T x M)
-};
-
-template <typename R, typename RT>
-struct Args {
-    const Item<R>* items;  // count items, by decreasing NC (increasing c0)
-    int count;
-    long long C;     // total chunks
-    RT* E;           // C chunk totals (LElem)
-    RT* V;           // C value carries (LValue): the value at each chunk's end
-    RT* FE;          // C chunk affine maps (LAffine)
-    RT* X;           // C chunk start states
-    int* status;
-    int out_mask;    // bit 1: write S; bit 2: write K; bit 4: write v
-    int refine_add;  // 1: correction pass: x <- x^ + dx, u_out <- u^ + w - qh
-};
-
-// The item whose chunks contain chunk c (items sorted by c0).
-template <typename R>
-__device__ __forceinline__ int find_chunk(const Item<R>* items, int count, long long c) {
-    int lo = 0, hi = count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (items[mid].c0 <= c) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-// The item whose residual rows contain row q (items sorted by r0).
-template <typename R>
-__device__ __forceinline__ int find_row(const Item<R>* items, int count, long long q) {
-    int lo = 0, hi = count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (items[mid].r0 <= q) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
 
 // The constant matrices of the Newton correction problem: L = 0, U = I, H = I.
 template <typename R, int N, int M>
@@ -186,15 +136,6 @@ constexpr int groups_for(int bytes_per_group) {
     int g = 256 / N;
     while (g > 1 && g * bytes_per_group > 112 * 1024) --g;
     return g;
-}
-
-template <typename A, typename B>
-__device__ __forceinline__ void copy_in(A* dst, const B* src, int count, int lr, int lanes) {
-    for (int i = lr; i < count; i += lanes) dst[i] = static_cast<A>(src[i]);
-}
-
-__device__ __forceinline__ void flag(int* status, bool ok) {
-    if (!ok) atomicCAS(status, 0, kStatusSingular);
 }
 
 // H_k = I for every step (time-invariant identity with p = N): the step
@@ -314,10 +255,10 @@ __global__ void __launch_bounds__(N) k_cterm(Args<R, RT> a) {
         t += hi * xr[i];
     }
     if (D.etaT) t = static_cast<RT>(D.etaT[r]);
-    RT* val = a.V + it.c0 * LValue<N>::SIZE;
+    RT* val = a.V + it.c0 * GValue<N>::SIZE;
 #pragma unroll
-    for (int j = 0; j < N; ++j) val[LValue<N>::OS + r * LValue<N>::LD + j] = acc[j];
-    val[LValue<N>::OV + r] = t;
+    for (int j = 0; j < N; ++j) val[GValue<N>::OS + r * GValue<N>::LD + j] = acc[j];
+    val[GValue<N>::OV + r] = t;
     a.X[(it.c0 + it.NC - 1) * N + r] = static_cast<RT>(D.x0[r]);
     if (a.out_mask & 1) {
 #pragma unroll
@@ -606,6 +547,34 @@ struct M2Smem {  // P | step | scratch (combine, and the state solve)
     static constexpr int SIZE = SCR_OFF + SCR;
 };
 
+// an element between global memory (GElem) and shared memory (LElem)
+template <int N, typename A, typename B>
+__device__ __forceinline__ void elem_in(A* dst, const B* src, int lr) {
+    using E = LElem<N>;
+    using G = GElem<N>;
+    for (int t = lr; t < N * N; t += N) {
+        const int i = t / N, j = t % N;
+        dst[E::OA + i * E::LD + j] = static_cast<A>(src[G::OA + i * G::LD + j]);
+        dst[E::OC + i * E::LD + j] = static_cast<A>(src[G::OC + i * G::LD + j]);
+        dst[E::OJ + i * E::LD + j] = static_cast<A>(src[G::OJ + i * G::LD + j]);
+    }
+    dst[E::OB + lr] = static_cast<A>(src[G::OB + lr]);
+    dst[E::OE + lr] = static_cast<A>(src[G::OE + lr]);
+}
+template <int N, typename A, typename B>
+__device__ __forceinline__ void elem_out(A* dst, const B* src, int lr) {
+    using E = LElem<N>;
+    using G = GElem<N>;
+    for (int t = lr; t < N * N; t += N) {
+        const int i = t / N, j = t % N;
+        dst[G::OA + i * G::LD + j] = src[E::OA + i * E::LD + j];
+        dst[G::OC + i * G::LD + j] = src[E::OC + i * E::LD + j];
+        dst[G::OJ + i * G::LD + j] = src[E::OJ + i * E::LD + j];
+    }
+    dst[G::OB + lr] = src[E::OB + lr];
+    dst[G::OE + lr] = src[E::OE + lr];
+}
+
 // up-sweep level h: E2[j] <- E2[j - h] (x) E2[j], j = 2h q + 2h - 1
 template <typename RT, int N, int NG>
 __global__ void __launch_bounds__(NG* N) k_m2up(RT* E2, long long active, int h, int* status) {
@@ -619,18 +588,18 @@ __global__ void __launch_bounds__(NG* N) k_m2up(RT* E2, long long active, int h,
     RT* e1 = sh + gi * gstride<N>(UpSmem<N>::SIZE);
     RT* e2 = e1 + E::SIZE;
     RT* scr = e2 + E::SIZE;
-    copy_in(e1, E2 + (j - h) * E::SIZE, E::SIZE, g.lr, N);
-    copy_in(e2, E2 + j * E::SIZE, E::SIZE, g.lr, N);
+    elem_in<N>(e1, E2 + (j - h) * GElem<N>::SIZE, g.lr);
+    elem_in<N>(e2, E2 + j * GElem<N>::SIZE, g.lr);
     g.sync();
     const bool ok = combine<N, N>(e1, e2, e2, scr, g);
-    for (int t = g.lr; t < E::SIZE; t += N) E2[j * E::SIZE + t] = e2[t];
+    elem_out<N>(E2 + j * GElem<N>::SIZE, e2, g.lr);
     flag(status, ok);
 }
 
 // the seed of each problem's prefix sweep: Pref[c0 + NC - 1] <- (0, x_0, 0, 0, 0)
 template <typename R, typename RT, int N>
 __global__ void __launch_bounds__(N) k_m2seed(const Item<R>* items, RT* Pref) {
-    using E = LElem<N>;
+    using E = GElem<N>;
     const Item<R>& it = items[blockIdx.x];
     RT* e = Pref + (it.c0 + it.NC - 1) * E::SIZE;
     const int r = threadIdx.x;
@@ -653,12 +622,13 @@ __global__ void __launch_bounds__(NG* N) k_m2down(const RT* E2, RT* Pref, long l
     RT* e1 = sh + gi * gstride<N>(UpSmem<N>::SIZE);
     RT* e2 = e1 + E::SIZE;
     RT* scr = e2 + E::SIZE;
-    copy_in(e1, Pref + j * E::SIZE, E::SIZE, g.lr, N);
-    copy_in(e2, E2 + (j - h) * E::SIZE, E::SIZE, g.lr, N);
-    for (int t = g.lr; t < E::SIZE; t += N) Pref[(j - h) * E::SIZE + t] = Pref[j * E::SIZE + t];
+    elem_in<N>(e1, Pref + j * GElem<N>::SIZE, g.lr);
+    elem_in<N>(e2, E2 + (j - h) * GElem<N>::SIZE, g.lr);
+    for (int t = g.lr; t < GElem<N>::SIZE; t += N)
+        Pref[(j - h) * GElem<N>::SIZE + t] = Pref[j * GElem<N>::SIZE + t];
     g.sync();
     const bool ok = combine<N, N>(e1, e2, e1, scr, g);
-    for (int t = g.lr; t < E::SIZE; t += N) Pref[j * E::SIZE + t] = e1[t];
+    elem_out<N>(Pref + j * GElem<N>::SIZE, e1, g.lr);
     flag(status, ok);
 }
 
@@ -697,7 +667,6 @@ __device__ bool m2_state(const R* P, const R* S, const R* v, R* xo, R* scr, cons
 template <typename R, typename RT, int N, int M, int NG>
 __global__ void __launch_bounds__(NG* N) k_m2roll(Args<R, RT> a, const RT* Pref) {
     using S = M2Smem<N, M>;
-    using E = LElem<N>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* sh = reinterpret_cast<R*>(smem_raw);
     const Group<N> g;
@@ -715,7 +684,7 @@ __global__ void __launch_bounds__(NG* N) k_m2roll(Args<R, RT> a, const RT* Pref)
     const long long lc = c - it.c0;
     const long long s0 = lc * it.B < T ? lc * it.B : T;
     const long long e0 = s0 + it.B < T ? s0 + it.B : T;
-    copy_in(P, Pref + c * E::SIZE, E::SIZE, r, N);
+    elem_in<N>(P, Pref + c * GElem<N>::SIZE, r);
     g.sync();
     bool ok = true;
     R* xs = scr + combine_scratch<N>() - N;  // the state (end of the scratch)

@@ -49,7 +49,8 @@ struct ChainVariant {
     lqt_status (*run)(const ChainCall& call, cudaStream_t s, Prof* prof);
     const void* (*fold_kernel)();
     size_t (*fold_smem)();
-    int (*fold_groups)();
+    int (*fold_groups)();   // teams or lane groups per CTA
+    int (*fold_threads)();  // threads per CTA
 };
 
 // Variants compiled in lqt_chain_n4.cu, lqt_chain_n8.cu, lqt_chain_n16.cu and

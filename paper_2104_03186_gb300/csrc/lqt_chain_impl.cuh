@@ -62,6 +62,11 @@ static cudaError_t chain_allow_smem(Kernel k, std::atomic<bool>* done, size_t by
     return err;
 }
 
+// Chunk-walk CTAs per SM for a CTA's shared memory (at most five, see NT_WALK).
+constexpr int walk_ctas(int bytes) {
+    return 227 * 1024 / (bytes + 1024) > 5 ? 5 : 227 * 1024 / (bytes + 1024);
+}
+
 template <typename R, typename RT, int N, int M>
 struct Launcher {
     static constexpr int FOLD_B = gstride<N>(FoldSmem<N, M, R>::SIZE) * (int)sizeof(R);
@@ -71,6 +76,24 @@ struct Launcher {
     static constexpr int FUP_B = gstride<N>(FupSmem<N>::SIZE) * (int)sizeof(RT);
     static constexpr int FDOWN_B = gstride<N>(FdownSmem<N>::SIZE) * (int)sizeof(RT);
     static constexpr int ROLL_B = gstride<N>(RollSmem<N, M>::SIZE) * (int)sizeof(R);
+    // n = 8, 16, 32: the team kernels (lqt_team_chain.cuh); n = 4: lane groups
+    static constexpr bool kTeam = N >= 8;
+    static constexpr int LG = N >= 8 ? N * N / 8 : N;  // lanes of a team
+    // chunk walks: CTAs of 128 lanes; as many per SM as the shared memory holds,
+    // five at most, which leaves a lane 96 registers
+    static constexpr int NT_WALK = 128 / LG;
+    static constexpr int TFOLD_B =
+        kTeam ? tstride_of<N, R>(TFoldSmem<N, M>::SIZE) * (int)sizeof(R) : 16;
+    static constexpr int TREFOLD_B =
+        kTeam ? tstride_of<N, R>(TRefoldSmem<N, M>::SIZE) * (int)sizeof(R) : 16;
+    static constexpr int MINB_FOLD = walk_ctas(NT_WALK * TFOLD_B);
+    static constexpr int MINB_REFOLD = walk_ctas(NT_WALK * TREFOLD_B);
+    // tree levels: TT teams per CTA (256 lanes), log2(TT) + 1 levels per launch
+    static constexpr int TT = 256 / LG;
+    static constexpr int TT_LEVELS = TT == 32 ? 6 : TT == 8 ? 4 : 2;
+    static constexpr int TUP_B = tstride_of<N, RT>(team::CombineSmem<N>::SIZE) * (int)sizeof(RT);
+    static constexpr int TDOWN_B = tstride_of<N, RT>(team::ApplySmem<N>::SIZE) * (int)sizeof(RT);
+    static constexpr int TFUP_B = tstride_of<N, RT>(2 * N * N) * (int)sizeof(RT);
     static constexpr int NG_FOLD = groups_for<N>(FOLD_B);
     static constexpr int NG_REFOLD = groups_for<N>(REFOLD_B);
     static constexpr int NG_UP = groups_for<N>(UP_B);
@@ -97,7 +120,19 @@ struct Launcher {
         static std::atomic<bool> d_fold[64], d_refold[64], d_up[64], d_down[64], d_fup[64], d_fdown[64],
             d_roll[64];
         cudaError_t e;
-        if ((e = chain_allow_smem(k_cfold<R, RT, N, M, NG_FOLD>, d_fold,
+        if constexpr (kTeam) {
+            if ((e = chain_allow_smem(k_tfold<R, RT, N, M, NT_WALK, MINB_FOLD>, d_fold,
+                                      (size_t)NT_WALK * TFOLD_B)) != cudaSuccess ||
+                (e = chain_allow_smem(k_trefold<R, RT, N, M, NT_WALK, MINB_REFOLD>, d_refold,
+                                      (size_t)NT_WALK * TREFOLD_B)) != cudaSuccess ||
+                (e = chain_allow_smem(k_tup<RT, N, TT>, d_up, (size_t)TT * TUP_B)) !=
+                    cudaSuccess ||
+                (e = chain_allow_smem(k_tdown<RT, N, TT>, d_down, (size_t)TT * TDOWN_B)) !=
+                    cudaSuccess ||
+                (e = chain_allow_smem(k_tfup<RT, N, TT>, d_fup, (size_t)TT * TFUP_B)) !=
+                    cudaSuccess)
+                return e;
+        } else if ((e = chain_allow_smem(k_cfold<R, RT, N, M, NG_FOLD>, d_fold,
                                   (size_t)NG_FOLD * FOLD_B)) != cudaSuccess ||
             (e = chain_allow_smem(k_crefold<R, RT, N, M, NG_REFOLD>, d_refold,
                                   (size_t)NG_REFOLD * REFOLD_B)) != cudaSuccess ||
@@ -150,15 +185,14 @@ struct Launcher {
 
     static int blocks(long long items, int ng) { return (int)((items + ng - 1) / ng); }
 
-    // The persistent launch (lqt_persist.cuh): groups per CTA from its group
-    // block, as many CTAs as are co-resident (at most one group per chunk).
-    static constexpr int PERSIST_B = persist_group_bytes<R, RT, N, M>();
-    // an even number of groups per CTA (the up-sweep pairs them), at least two
-    static constexpr int NG_PERSIST =
-        (groups_for<N>(PERSIST_B) & ~1) > 2 ? (groups_for<N>(PERSIST_B) & ~1) : 2;
-    // variants whose two groups do not fit one SM (FP64 at n = 32) always take
-    // the per-level launches
-    static constexpr bool kPersistFits = (long long)NG_PERSIST * PERSIST_B <= 227 * 1024;
+    // The persistent launch (lqt_persist.cuh): teams per CTA from its team
+    // block, as many CTAs as are co-resident (at most one team per chunk).
+    static constexpr int PERSIST_B = kTeam ? persist_team_bytes<R, RT, N, M>() : 16;
+    static constexpr int NT_PERSIST = 256 / LG;
+    // variants whose teams do not fit one SM (FP64 at n = 32 and FP64 trees)
+    // always take the per-level launches
+    static constexpr bool kPersistFits =
+        kTeam && (long long)NT_PERSIST * PERSIST_B <= 227 * 1024 - 1024;
 
     // only_if_small: launch nothing and return LQT_EUNSUPPORTED when the grid
     // would need more than half of the co-resident CTAs.  A cooperative launch
@@ -171,19 +205,19 @@ struct Launcher {
             return LQT_EUNSUPPORTED;
         } else {
         if (levels > kMaxLevels) return LQT_EINVAL;
-        auto kern = k_cpersist<R, RT, N, M, NG_PERSIST>;
+        auto kern = k_cpersist<R, RT, N, M, NT_PERSIST>;
         static std::atomic<bool> done[64];
-        const size_t smem = (size_t)NG_PERSIST * PERSIST_B;
+        const size_t smem = (size_t)NT_PERSIST * PERSIST_B;
         if (chain_allow_smem(kern, done, smem) != cudaSuccess) return LQT_ECUDA;
         int dev = 0, sms = 0, per_sm = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NG_PERSIST * N, smem) !=
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT_PERSIST * LG, smem) !=
                 cudaSuccess)
             return LQT_ECUDA;
         if (per_sm < 1) return LQT_ECUDA;
         long long grid = (long long)per_sm * sms;
-        const long long need = (a.C + NG_PERSIST - 1) / NG_PERSIST;
+        const long long need = (a.C + NT_PERSIST - 1) / NT_PERSIST;
         if (only_if_small && 2 * need > grid) return LQT_EUNSUPPORTED;
         if (grid > need) grid = need;
         if (grid < 1) grid = 1;
@@ -196,7 +230,7 @@ struct Launcher {
         long long limit = 1LL << 22;  // polls of 64 ns sleeps: far above any phase's length
         void* args[] = {&aa, &lp, &bar, &limit};
         if (cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kern), dim3((unsigned)grid),
-                                        dim3(NG_PERSIST * N), args, smem, s) != cudaSuccess)
+                                        dim3(NT_PERSIST * LG), args, smem, s) != cudaSuccess)
             return LQT_ECUDA;
         return LQT_OK;
         }
@@ -231,19 +265,19 @@ struct Launcher {
         off += up(sizeof(GridBarrier));
         const size_t nc = (size_t)C;
         L.E = off;
-        off += up(nc * LElem<N>::SIZE * sizeof(RT));
+        off += up(nc * GElem<N>::SIZE * sizeof(RT));
         L.V = off;
-        off += up(nc * LValue<N>::SIZE * sizeof(RT));
+        off += up(nc * GValue<N>::SIZE * sizeof(RT));
         L.FE = off;
-        off += up(nc * LAffine<N>::SIZE * sizeof(RT));
+        off += up(nc * GAffine<N>::SIZE * sizeof(RT));
         L.X = off;
         off += up(nc * N * sizeof(RT));
         L.E2 = L.Pref = 0;
         if (method2) {  // Method 2: a copy of the chunk totals and the prefixes
             L.E2 = off;
-            off += up(nc * LElem<N>::SIZE * sizeof(RT));
+            off += up(nc * GElem<N>::SIZE * sizeof(RT));
             L.Pref = off;
-            off += up(nc * LElem<N>::SIZE * sizeof(RT));
+            off += up(nc * GElem<N>::SIZE * sizeof(RT));
         }
         L.refine0 = off;
         if (refine)
@@ -322,6 +356,73 @@ struct Launcher {
         }
     }
 
+    // Tree levels [l, l + TT_LEVELS) as one launch of the multi-level kernels.
+    static TreeRun tree_run(const long long* active, int levels, int l) {
+        TreeRun tr;
+        memset(&tr, 0, sizeof(tr));
+        tr.h0 = 1 << l;
+        tr.levels = levels - l < TT_LEVELS ? levels - l : TT_LEVELS;
+        for (int i = 0; i < tr.levels; ++i) tr.active[i] = active[l + i];
+        return tr;
+    }
+    static int top_run(int levels) { return levels > 0 ? (levels - 1) / TT_LEVELS * TT_LEVELS : -1; }
+    static int tree_blocks(const TreeRun& tr) {
+        const long long span = 2ll * TT * tr.h0;
+        return (int)((tr.active[0] + span - 1) / span);
+    }
+
+    static void launch_fold(const Args<R, RT>& a, cudaStream_t s) {
+        if constexpr (kTeam)
+            k_tfold<R, RT, N, M, NT_WALK, MINB_FOLD>
+                <<<blocks(a.C, NT_WALK), NT_WALK * LG, (size_t)NT_WALK * TFOLD_B, s>>>(a);
+        else
+            k_cfold<R, RT, N, M, NG_FOLD>
+                <<<blocks(a.C, NG_FOLD), NG_FOLD * N, (size_t)NG_FOLD * FOLD_B, s>>>(a);
+    }
+    static void launch_refold(const Args<R, RT>& a, cudaStream_t s) {
+        if constexpr (kTeam)
+            k_trefold<R, RT, N, M, NT_WALK, MINB_REFOLD>
+                <<<blocks(a.C, NT_WALK), NT_WALK * LG, (size_t)NT_WALK * TREFOLD_B, s>>>(a);
+        else
+            k_crefold<R, RT, N, M, NG_REFOLD>
+                <<<blocks(a.C, NG_REFOLD), NG_REFOLD * N, (size_t)NG_REFOLD * REFOLD_B, s>>>(a);
+    }
+    // up-sweep of the chunk totals
+    static void launch_up(const Args<R, RT>& a, const long long* active, int levels,
+                          cudaStream_t s) {
+        if constexpr (kTeam) {
+            for (int l = 0; l < levels; l += TT_LEVELS) {
+                const TreeRun tr = tree_run(active, levels, l);
+                k_tup<RT, N, TT>
+                    <<<tree_blocks(tr), TT * LG, (size_t)TT * TUP_B, s>>>(a.E, tr, a.status);
+            }
+        } else {
+            for (int l = 0; l < levels; ++l) {
+                const int h = 1 << l;
+                k_cup<RT, N, NG_UP><<<blocks(active[l] / (2 * h), NG_UP), NG_UP * N,
+                                      (size_t)NG_UP * UP_B, s>>>(a.E, active[l], h, a.status);
+            }
+        }
+    }
+    // down-sweep of the value carries
+    static void launch_down(const Args<R, RT>& a, const long long* active, int levels,
+                            cudaStream_t s) {
+        if constexpr (kTeam) {
+            for (int l = top_run(levels); l >= 0; l -= TT_LEVELS) {
+                const TreeRun tr = tree_run(active, levels, l);
+                k_tdown<RT, N, TT>
+                    <<<tree_blocks(tr), TT * LG, (size_t)TT * TDOWN_B, s>>>(a.E, a.V, tr, a.status);
+            }
+        } else {
+            for (int l = levels - 1; l >= 0; --l) {
+                const int h = 1 << l;
+                k_cdown<RT, N, NG_DOWN><<<blocks(active[l] / (2 * h), NG_DOWN), NG_DOWN * N,
+                                          (size_t)NG_DOWN * DOWN_B, s>>>(a.E, a.V, active[l], h,
+                                                                         a.status);
+            }
+        }
+    }
+
     // One pass: backward scan, re-fold, then (unless backward_only) the forward
     // scan and the rollout.  With Method 2 (E2 given) the forward element scan
     // runs on a second stream, forked after the chunk fold and joined before
@@ -337,10 +438,9 @@ struct Launcher {
         bool forked = false, scanned = false;
         if (!sequential) {
             prof_mark(prof, s, pname(kind, 0));
-            k_cfold<R, RT, N, M, NG_FOLD>
-                <<<blocks(C, NG_FOLD), NG_FOLD * N, (size_t)NG_FOLD * FOLD_B, s>>>(a);
+            launch_fold(a, s);
             if (m2) {  // the chunk totals, before the backward up-sweep overwrites them
-                cudaMemcpyAsync(E2, a.E, (size_t)C * LElem<N>::SIZE * sizeof(RT),
+                cudaMemcpyAsync(E2, a.E, (size_t)C * GElem<N>::SIZE * sizeof(RT),
                                 cudaMemcpyDeviceToDevice, s);
                 if (fa && cudaEventRecord(fa->fork, s) == cudaSuccess &&
                     cudaStreamWaitEvent(fa->s, fa->fork, 0) == cudaSuccess) {
@@ -353,23 +453,13 @@ struct Launcher {
                 }
             }
             if (levels > 0) prof_mark(prof, s, pname(kind, 1));
-            for (int l = 0; l < levels; ++l) {
-                const int h = 1 << l;
-                k_cup<RT, N, NG_UP><<<blocks(active[l] / (2 * h), NG_UP), NG_UP * N,
-                                      (size_t)NG_UP * UP_B, s>>>(a.E, active[l], h, a.status);
-            }
+            launch_up(a, active, levels, s);
         }
         prof_mark(prof, s, pname(kind, 2));
         k_cterm<R, RT, N><<<a.count, N, 0, s>>>(a);
-        for (int l = levels - 1; l >= 0; --l) {
-            const int h = 1 << l;
-            k_cdown<RT, N, NG_DOWN><<<blocks(active[l] / (2 * h), NG_DOWN), NG_DOWN * N,
-                                      (size_t)NG_DOWN * DOWN_B, s>>>(a.E, a.V, active[l], h,
-                                                                     a.status);
-        }
+        launch_down(a, active, levels, s);
         prof_mark(prof, s, pname(kind, 3));
-        k_crefold<R, RT, N, M, NG_REFOLD>
-            <<<blocks(C, NG_REFOLD), NG_REFOLD * N, (size_t)NG_REFOLD * REFOLD_B, s>>>(a);
+        launch_refold(a, s);
         if (backward_only) return;
         if (m2) {
             // Method 2: prefix scan of the elements from (0, x_0, 0, 0, 0)
@@ -386,17 +476,7 @@ struct Launcher {
         }
         if (levels > 0) {
             prof_mark(prof, s, pname(kind, 4));
-            for (int l = 0; l < levels; ++l) {
-                const int h = 1 << l;
-                k_cfup<RT, N, NG_FUP><<<blocks(active[l] / (2 * h), NG_FUP), NG_FUP * N,
-                                        (size_t)NG_FUP * FUP_B, s>>>(a.FE, active[l], h);
-            }
-            for (int l = levels - 1; l >= 0; --l) {
-                const int h = 1 << l;
-                k_cfdown<RT, N, NG_FDOWN><<<blocks(active[l] / (2 * h), NG_FDOWN),
-                                            NG_FDOWN * N, (size_t)NG_FDOWN * FDOWN_B, s>>>(
-                    a.FE, a.X, active[l], h);
-            }
+            affine_scan(a.FE, a.X, active, levels, s);
         }
         prof_mark(prof, s, pname(kind, 5));
         k_croll<R, RT, N, M, NG_ROLL>
@@ -406,15 +486,26 @@ struct Launcher {
     // Forward affine scan of the maps FE from the seeds in each problem's top
     // slot of X: afterwards X[c] is the state at the start of chunk c.
     static void affine_scan(RT* FE, RT* X, const long long* active, int levels, cudaStream_t s) {
-        for (int l = 0; l < levels; ++l) {
-            const int h = 1 << l;
-            k_cfup<RT, N, NG_FUP><<<blocks(active[l] / (2 * h), NG_FUP), NG_FUP * N,
-                                    (size_t)NG_FUP * FUP_B, s>>>(FE, active[l], h);
-        }
-        for (int l = levels - 1; l >= 0; --l) {
-            const int h = 1 << l;
-            k_cfdown<RT, N, NG_FDOWN><<<blocks(active[l] / (2 * h), NG_FDOWN), NG_FDOWN * N,
-                                        (size_t)NG_FDOWN * FDOWN_B, s>>>(FE, X, active[l], h);
+        if constexpr (kTeam) {
+            for (int l = 0; l < levels; l += TT_LEVELS) {
+                const TreeRun tr = tree_run(active, levels, l);
+                k_tfup<RT, N, TT><<<tree_blocks(tr), TT * LG, (size_t)TT * TFUP_B, s>>>(FE, tr);
+            }
+            for (int l = top_run(levels); l >= 0; l -= TT_LEVELS) {
+                const TreeRun tr = tree_run(active, levels, l);
+                k_tfdown<RT, N, TT><<<tree_blocks(tr), TT * LG, 0, s>>>(FE, X, tr);
+            }
+        } else {
+            for (int l = 0; l < levels; ++l) {
+                const int h = 1 << l;
+                k_cfup<RT, N, NG_FUP><<<blocks(active[l] / (2 * h), NG_FUP), NG_FUP * N,
+                                        (size_t)NG_FUP * FUP_B, s>>>(FE, active[l], h);
+            }
+            for (int l = levels - 1; l >= 0; --l) {
+                const int h = 1 << l;
+                k_cfdown<RT, N, NG_FDOWN><<<blocks(active[l] / (2 * h), NG_FDOWN), NG_FDOWN * N,
+                                            (size_t)NG_FDOWN * FDOWN_B, s>>>(FE, X, active[l], h);
+            }
         }
     }
 
@@ -467,7 +558,7 @@ struct Launcher {
         a.out_mask = 0;
         a.refine_add = 0;
         // the chunk totals' region holds a copy of each chunk's Psi
-        static_assert(LElem<N>::SIZE >= LAffine<N>::SIZE, "Psi copy fits the element slots");
+        static_assert(GElem<N>::SIZE >= GAffine<N>::SIZE, "Psi copy fits the element slots");
         RT* psi = a.E;
         const long long C = a.C;
         prof_mark(prof, s, "warm_fold");
@@ -682,11 +773,17 @@ struct Launcher {
         return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;
     }
 
-    static int fold_groups_per_cta() { return NG_FOLD; }
+    static int fold_groups_per_cta() { return kTeam ? NT_WALK : NG_FOLD; }
+    static int fold_threads() { return kTeam ? NT_WALK * LG : NG_FOLD * N; }
     static const void* fold_kernel() {
-        return reinterpret_cast<const void*>(k_cfold<R, RT, N, M, NG_FOLD>);
+        if constexpr (kTeam)
+            return reinterpret_cast<const void*>(k_tfold<R, RT, N, M, NT_WALK, MINB_FOLD>);
+        else
+            return reinterpret_cast<const void*>(k_cfold<R, RT, N, M, NG_FOLD>);
     }
-    static size_t fold_smem() { return (size_t)NG_FOLD * FOLD_B; }
+    static size_t fold_smem() {
+        return kTeam ? (size_t)NT_WALK * TFOLD_B : (size_t)NG_FOLD * FOLD_B;
+    }
 };
 
 }  // namespace chain
@@ -696,7 +793,8 @@ struct Launcher {
         sizeof(R) == 8 ? LQT_F64 : LQT_F32, N, M, sizeof(RT) == 8 && sizeof(R) == 4,            \
             &chain::Launcher<R, RT, N, M>::workspace, &chain::Launcher<R, RT, N, M>::run,       \
             &chain::Launcher<R, RT, N, M>::fold_kernel, &chain::Launcher<R, RT, N, M>::fold_smem, \
-            &chain::Launcher<R, RT, N, M>::fold_groups_per_cta                                  \
+            &chain::Launcher<R, RT, N, M>::fold_groups_per_cta,                                 \
+            &chain::Launcher<R, RT, N, M>::fold_threads                                  \
     }
 
 }  // namespace lqt

@@ -6,17 +6,14 @@
 // turn: the chunk folds, the up-sweep levels of Alg. 1, the terminal values,
 // the down-sweep levels of the value carries, the Riccati re-folds, the
 // up- and down-sweep levels of the trajectory maps and the rollouts.  Within
-// a phase the CTAs' lane groups take work items: the chunks of the fold,
-// re-fold and rollout from a counter (whichever group is free takes the next
-// one), the pairs of a tree level by a grid stride; between phases a grid
-// barrier orders the global-memory results.  The per-item work is the same
-// device code as the level kernels' (b_cfold, b_cup, ... in lqt_chain.cuh).
+// a phase the CTAs' teams take work items: the chunks of the fold, re-fold and
+// rollout from a counter (whichever team is free takes the next one), the
+// pairs of a tree level by a grid stride; between phases a grid barrier orders
+// the global-memory results.  The per-item work is the same device code as the
+// level kernels' (lqt_team_chain.cuh, lqt_team.cuh).
 //
-// Each group owns a block sized for the chunk phases (the largest of the
-// fold, re-fold and rollout blocks, and of the level phases other than the
-// up-sweep), so that as many groups share an SM as in the fold launch of the
-// level-by-level pipeline; in the up-sweep levels, whose block is larger, the
-// even groups work on two blocks and the odd ones wait.
+// Each team owns a block sized for the largest phase; the terminal values and
+// the rollouts run on the first N lanes of a team (lane-group code).
 //
 // The barrier is a counter and a generation word in the workspace.  Every
 // wait is bounded: a CTA that waits longer than the limit records
@@ -41,14 +38,17 @@ struct GridBarrier {
     unsigned long long next[3];  // work counters of the fold, re-fold and rollout phases
 };
 
-// The next chunk of a phase for the calling group (lane 0 draws, the group
-// shares it): chunks go to whichever group is free, as the hardware would hand
-// out the CTAs of a launch, so chunks of different lengths balance.
+// The next chunk of a phase for the calling team (lane 0 draws, the team
+// shares it through `slot`): chunks go to whichever team is free, as the
+// hardware would hand out the CTAs of a launch, so chunks of different lengths
+// balance.
 template <int N>
-__device__ __forceinline__ long long next_chunk(unsigned long long* counter, const Group<N>& g) {
-    unsigned long long c = 0;
-    if (g.lr == 0) c = atomicAdd(counter, 1ull);
-    return (long long)__shfl_sync(g.mask, c, (threadIdx.x & 31) - g.lr);
+__device__ __forceinline__ long long next_chunk(unsigned long long* counter,
+                                                unsigned long long* slot, const Team<N>& g) {
+    g.sync();  // the slot's last value has been read
+    if (g.lane == 0) *slot = atomicAdd(counter, 1ull);
+    g.sync();
+    return (long long)*slot;
 }
 
 // Active chunk counts of the tree levels (as in the level-by-level launch).
@@ -127,10 +127,10 @@ __device__ __forceinline__ void b_cterm_group(const Args<R, RT>& a, int q, RT* Y
         t += hi * xr[i];
     }
     if (D.etaT) t = static_cast<RT>(D.etaT[r]);
-    RT* val = a.V + it.c0 * LValue<N>::SIZE;
+    RT* val = a.V + it.c0 * GValue<N>::SIZE;
 #pragma unroll
-    for (int j = 0; j < N; ++j) val[LValue<N>::OS + r * LValue<N>::LD + j] = acc[j];
-    val[LValue<N>::OV + r] = t;
+    for (int j = 0; j < N; ++j) val[GValue<N>::OS + r * GValue<N>::LD + j] = acc[j];
+    val[GValue<N>::OV + r] = t;
     a.X[(it.c0 + it.NC - 1) * N + r] = static_cast<RT>(D.x0[r]);
     if (a.out_mask & 1) {
 #pragma unroll
@@ -141,96 +141,108 @@ __device__ __forceinline__ void b_cterm_group(const Args<R, RT>& a, int q, RT* Y
     g.sync();
 }
 
-// Shared memory of one group of the persistent kernel (bytes, rounded to 16):
-// the largest block of the chunk phases and of the level phases other than
-// the up-sweep, which takes two blocks.
+// Shared memory of one team of the persistent kernel (bytes, a multiple of
+// 16): the largest block of its phases.
 template <typename R, typename RT, int N, int M>
-constexpr int persist_group_bytes() {
-    constexpr int sizes[] = {gstride<N>(FoldSmem<N, M, R>::SIZE) * (int)sizeof(R),
-                             gstride<N>(RefoldSmem<N, M>::SIZE) * (int)sizeof(R),
+constexpr int persist_team_bytes() {
+    constexpr int sizes[] = {tstride_of<N, R>(TFoldSmem<N, M>::SIZE) * (int)sizeof(R),
+                             tstride_of<N, R>(TRefoldSmem<N, M>::SIZE) * (int)sizeof(R),
                              gstride<N>(RollSmem<N, M>::SIZE) * (int)sizeof(R),
-                             gstride<N>(DownSmem<N>::SIZE) * (int)sizeof(RT),
-                             gstride<N>(FupSmem<N>::SIZE) * (int)sizeof(RT),
-                             gstride<N>(FdownSmem<N>::SIZE) * (int)sizeof(RT),
-                             gstride<N>(2 * N * N + 2 * N) * (int)sizeof(RT)};
+                             tstride_of<N, RT>(team::CombineSmem<N>::SIZE) * (int)sizeof(RT),
+                             tstride_of<N, RT>(team::ApplySmem<N>::SIZE) * (int)sizeof(RT),
+                             (2 * N * N + 2 * N) * (int)sizeof(RT)};
     int m = 0;
     for (int s : sizes) m = s > m ? s : m;
     return (m + 15) / 16 * 16;
 }
 
-template <typename R, typename RT, int N, int M>
-constexpr bool persist_up_fits() {
-    return gstride<N>(UpSmem<N>::SIZE) * (int)sizeof(RT) <= 2 * persist_group_bytes<R, RT, N, M>();
-}
-
-// The body of each phase addresses group gi's block at gi * gstride<N>(its own
-// size); the persistent kernel gives each group a block of
-// persist_group_bytes() instead, so it passes the group's own base with gi = 0.
-template <typename R, typename RT, int N, int M, int NG>
-__global__ void __launch_bounds__(NG* N) k_cpersist(Args<R, RT> a, LevelPlan lp,
-                                                    GridBarrier* bar, long long wait_limit) {
+template <typename R, typename RT, int N, int M, int NT>
+__global__ void __launch_bounds__(NT* Team<N>::LG) k_cpersist(Args<R, RT> a, LevelPlan lp,
+                                                              GridBarrier* bar,
+                                                              long long wait_limit) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int GB = persist_group_bytes<R, RT, N, M>();
-    const int gi = threadIdx.x / N;
+    __shared__ unsigned long long slots[NT];
+    constexpr int GB = persist_team_bytes<R, RT, N, M>();
+    const Team<N> g;
+    const Group<N> lanes_g;  // the first N lanes of the team, in the lane-group phases
+    const int gi = threadIdx.x / Team<N>::LG;
+    const bool lead = g.lane < N;
     unsigned char* mine = smem_raw + gi * GB;
-    const Group<N> g;
-    const long long first = (long long)blockIdx.x * NG + gi;
-    const long long stride = (long long)gridDim.x * NG;
+    R* sh = reinterpret_cast<R*>(mine);
+    RT* sht = reinterpret_cast<RT*>(mine);
+    unsigned long long* slot = &slots[gi];
+    const long long first = (long long)blockIdx.x * NT + gi;
+    const long long stride = (long long)gridDim.x * NT;
     const unsigned int nb = gridDim.x;
     const long long C = a.C;
+    bool ok = true;
     // 1. chunk folds
-    for (long long c = next_chunk(&bar->next[0], g); c < C; c = next_chunk(&bar->next[0], g))
-        b_cfold<R, RT, N, M, NG>(a, c, mine, 0);
+    for (long long c = next_chunk(&bar->next[0], slot, g); c < C;
+         c = next_chunk(&bar->next[0], slot, g))
+        b_tfold<R, RT, N, M>(a, c, sh);
     if (!grid_sync(bar, nb, wait_limit, a.status)) return;
     // 2. up-sweep levels
-    static_assert(NG % 2 == 0, "the up-sweep pairs the groups of a CTA");
-    static_assert(persist_up_fits<R, RT, N, M>(), "two blocks hold the up-sweep's");
-    {
-        // even groups only, each on its own block and the next group's
-        const long long ufirst = (long long)blockIdx.x * (NG / 2) + gi / 2;
-        const long long ustride = (long long)gridDim.x * (NG / 2);
-        for (int l = 0; l < lp.levels; ++l) {
-            const int h = 1 << l;
-            const long long pairs = lp.active[l] / (2 * h);
-            if ((gi & 1) == 0)
-                for (long long q = ufirst; q < pairs; q += ustride)
-                    b_cup<RT, N, NG>(a.E, lp.active[l], h, a.status, q * 2 * h, mine, 0);
-            if (!grid_sync(bar, nb, wait_limit, a.status)) return;
+    for (int l = 0; l < lp.levels; ++l) {
+        const long long h = 1ll << l, pairs = lp.active[l] / (2 * h);
+        for (long long q = first; q < pairs; q += stride) {
+            RT* e = a.E + q * 2 * h * DElem<N>::SIZE;
+            ok &= team::combine<N>(e, e + h * DElem<N>::SIZE, e, sht, g);
+            g.sync();
         }
+        if (!grid_sync(bar, nb, wait_limit, a.status)) return;
     }
     // 3. terminal values, then the down-sweep levels of the value carries
-    for (long long q = first; q < a.count; q += stride)
-        b_cterm_group<R, RT, N>(a, (int)q, reinterpret_cast<RT*>(mine), g);
+    if (lead)
+        for (long long q = first; q < a.count; q += stride)
+            b_cterm_group<R, RT, N>(a, (int)q, sht, lanes_g);
     if (!grid_sync(bar, nb, wait_limit, a.status)) return;
     for (int l = lp.levels - 1; l >= 0; --l) {
-        const int h = 1 << l;
-        const long long pairs = lp.active[l] / (2 * h);
-        for (long long q = first; q < pairs; q += stride)
-            b_cdown<RT, N, NG>(a.E, a.V, lp.active[l], h, a.status, q * 2 * h, mine, 0);
+        const long long h = 1ll << l, pairs = lp.active[l] / (2 * h);
+        for (long long q = first; q < pairs; q += stride) {
+            const long long i = q * 2 * h;
+            RT* val = a.V + i * DValue<N>::SIZE;
+            for (int t = g.lane; t < DValue<N>::SIZE; t += Team<N>::LG)
+                val[h * DValue<N>::SIZE + t] = val[t];
+            ok &= team::value_apply<N>(a.E + (i + h) * DElem<N>::SIZE, val, val, sht, g);
+            g.sync();
+        }
         if (!grid_sync(bar, nb, wait_limit, a.status)) return;
     }
     // 4. Riccati re-folds with the outputs and the chunk maps
-    for (long long c = next_chunk(&bar->next[1], g); c < C; c = next_chunk(&bar->next[1], g))
-        b_crefold<R, RT, N, M, NG>(a, c, mine, 0);
+    for (long long c = next_chunk(&bar->next[1], slot, g); c < C;
+         c = next_chunk(&bar->next[1], slot, g))
+        b_trefold<R, RT, N, M>(a, c, sh);
     if (!grid_sync(bar, nb, wait_limit, a.status)) return;
     // 5. trajectory maps: up-sweep, then down-sweep from x_0
     for (int l = 0; l < lp.levels; ++l) {
-        const int h = 1 << l;
-        const long long pairs = lp.active[l] / (2 * h);
-        for (long long q = first; q < pairs; q += stride)
-            b_cfup<RT, N, NG>(a.FE, lp.active[l], h, q * 2 * h + 2 * h - 1, mine, 0);
+        const long long h = 1ll << l, pairs = lp.active[l] / (2 * h);
+        for (long long q = first; q < pairs; q += stride) {
+            RT* f = a.FE + (q * 2 * h + 2 * h - 1) * DAffine<N>::SIZE;
+            team::affine_compose<N>(f - h * DAffine<N>::SIZE, f, f, sht, g);
+            g.sync();
+        }
         if (!grid_sync(bar, nb, wait_limit, a.status)) return;
     }
     for (int l = lp.levels - 1; l >= 0; --l) {
-        const int h = 1 << l;
-        const long long pairs = lp.active[l] / (2 * h);
-        for (long long q = first; q < pairs; q += stride)
-            b_cfdown<RT, N, NG>(a.FE, a.X, lp.active[l], h, q * 2 * h + 2 * h - 1, mine, 0);
+        const long long h = 1ll << l, pairs = lp.active[l] / (2 * h);
+        for (long long q = first; q < pairs; q += stride) {
+            const long long j = q * 2 * h + 2 * h - 1;
+            RT y0, y1;
+            for (int i = g.lane; i < N; i += Team<N>::LG) a.X[(j - h) * N + i] = a.X[j * N + i];
+            team::affine_apply<N>(a.FE + (j - h) * DAffine<N>::SIZE, a.X + j * N, y0, y1, g);
+            g.sync();  // every lane has read X[j]
+            if (g.ci == 0) {
+                a.X[j * N + g.ri] = y0;
+                a.X[j * N + g.ri + N / 2] = y1;
+            }
+        }
         if (!grid_sync(bar, nb, wait_limit, a.status)) return;
     }
     // 6. rollouts
-    for (long long c = next_chunk(&bar->next[2], g); c < C; c = next_chunk(&bar->next[2], g))
-        b_croll<R, RT, N, M, NG>(a, c, mine, 0);
+    for (long long c = next_chunk(&bar->next[2], slot, g); c < C;
+         c = next_chunk(&bar->next[2], slot, g))
+        if (lead) b_croll<R, RT, N, M, NT>(a, c, mine, 0);
+    flag(a.status, ok);
 }
 
 }  // namespace chain

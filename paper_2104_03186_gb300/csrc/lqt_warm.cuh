@@ -135,7 +135,7 @@ __device__ __forceinline__ void warm_ft_column(R* gs, int r) {
 template <typename R, typename RT, int N, int M, int NG>
 __global__ void __launch_bounds__(NG* N) k_wfold(Args<R, RT> a, RT* psi_copy) {
     using W = WarmSmem<N, M>;
-    using A = LAffine<N>;
+    using A = GAffine<N>;
     constexpr int LD = W::LD;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* sh = reinterpret_cast<R*>(smem_raw);
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(N) k_wseed(Args<R, RT> a) {
 template <typename R, typename RT, int N, int M, int NG>
 __global__ void __launch_bounds__(NG* N) k_wrefold(Args<R, RT> a, const RT* psi_copy) {
     using W = WarmSmem<N, M>;
-    using A = LAffine<N>;
+    using A = GAffine<N>;
     constexpr int LD = W::LD, LM = W::LM;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* sh = reinterpret_cast<R*>(smem_raw);
