@@ -141,7 +141,9 @@ lqt_status batch_geometry(const ChainVariant& v, const lqt_batch_item* items, co
         cp.B = T > 0 ? (T + nc - 1) / nc : 1;
     }
     std::stable_sort(out->begin(), out->end(),
-                     [](const ChainProblem& a, const ChainProblem& b) { return a.NC > b.NC; });
+                     [](const ChainProblem& a, const ChainProblem& b) {
+                         return a.NC != b.NC ? a.NC > b.NC : a.B > b.B;
+                     });
     return LQT_OK;
 }
 

@@ -36,6 +36,7 @@ struct Args {
     RT* X;           // C chunk start states
     int* status;
     int out_mask;    // bit 1: write S; bit 2: write K; bit 4: write v
+    int first_total; // 1: the totals of the problems' first chunks are wanted (Method 2)
     int refine_add;  // 1: correction pass: x <- x^ + dx, u_out <- u^ + w - qh
 };
 

@@ -62,9 +62,9 @@ static cudaError_t chain_allow_smem(Kernel k, std::atomic<bool>* done, size_t by
     return err;
 }
 
-// Chunk-walk CTAs per SM for a CTA's shared memory (at most five, see NT_WALK).
+// Chunk-walk CTAs per SM for a CTA's shared memory (at most four, see NT_WALK).
 constexpr int walk_ctas(int bytes) {
-    return 227 * 1024 / (bytes + 1024) > 5 ? 5 : 227 * 1024 / (bytes + 1024);
+    return 227 * 1024 / (bytes + 1024) > 4 ? 4 : 227 * 1024 / (bytes + 1024);
 }
 
 template <typename R, typename RT, int N, int M>
@@ -79,8 +79,16 @@ struct Launcher {
     // n = 8, 16, 32: the team kernels (lqt_team_chain.cuh); n = 4: lane groups
     static constexpr bool kTeam = N >= 8;
     static constexpr int LG = N >= 8 ? N * N / 8 : N;  // lanes of a team
-    // chunk walks: CTAs of 128 lanes; as many per SM as the shared memory holds,
-    // five at most, which leaves a lane 96 registers
+    // Chunk walks: tiles of 2 x 4 entries, at n = 32 in FP32 4 x 4 (LGW lanes a
+    // team).  The walks are bound by shared-memory reads, which cost one
+    // wavefront per 32 words delivered, broadcast or not; a 4 x 4 tile reads a
+    // third less than a 2 x 4 one for the same products but halves the warps.
+    // At n = 32 (T = 65536) it took the refined solve from 8.3 to 7.3 ms; at
+    // n = 16 (ragged batch) 20.3 -> 20.4 ms and at n = 8 it lost 10%.
+    // CTAs of four teams' worth of 32 lanes; at most four per SM, which leaves
+    // a lane 128 registers (five with 96: 20.7 against 20.3 ms on the batch).
+    static constexpr int TR = N == 32 && sizeof(R) == 4 ? 4 : 2;
+    static constexpr int LGW = LG * 2 / TR;
     static constexpr int NT_WALK = 128 / LG;
     static constexpr int TFOLD_B =
         kTeam ? tstride_of<N, R>(TFoldSmem<N, M>::SIZE) * (int)sizeof(R) : 16;
@@ -121,9 +129,9 @@ struct Launcher {
             d_roll[64];
         cudaError_t e;
         if constexpr (kTeam) {
-            if ((e = chain_allow_smem(k_tfold<R, RT, N, M, NT_WALK, MINB_FOLD>, d_fold,
+            if ((e = chain_allow_smem(k_tfold<R, RT, N, M, TR, NT_WALK, MINB_FOLD>, d_fold,
                                       (size_t)NT_WALK * TFOLD_B)) != cudaSuccess ||
-                (e = chain_allow_smem(k_trefold<R, RT, N, M, NT_WALK, MINB_REFOLD>, d_refold,
+                (e = chain_allow_smem(k_trefold<R, RT, N, M, TR, NT_WALK, MINB_REFOLD>, d_refold,
                                       (size_t)NT_WALK * TREFOLD_B)) != cudaSuccess ||
                 (e = chain_allow_smem(k_tup<RT, N, TT>, d_up, (size_t)TT * TUP_B)) !=
                     cudaSuccess ||
@@ -373,16 +381,16 @@ struct Launcher {
 
     static void launch_fold(const Args<R, RT>& a, cudaStream_t s) {
         if constexpr (kTeam)
-            k_tfold<R, RT, N, M, NT_WALK, MINB_FOLD>
-                <<<blocks(a.C, NT_WALK), NT_WALK * LG, (size_t)NT_WALK * TFOLD_B, s>>>(a);
+            k_tfold<R, RT, N, M, TR, NT_WALK, MINB_FOLD>
+                <<<blocks(a.C, NT_WALK), NT_WALK * LGW, (size_t)NT_WALK * TFOLD_B, s>>>(a);
         else
             k_cfold<R, RT, N, M, NG_FOLD>
                 <<<blocks(a.C, NG_FOLD), NG_FOLD * N, (size_t)NG_FOLD * FOLD_B, s>>>(a);
     }
     static void launch_refold(const Args<R, RT>& a, cudaStream_t s) {
         if constexpr (kTeam)
-            k_trefold<R, RT, N, M, NT_WALK, MINB_REFOLD>
-                <<<blocks(a.C, NT_WALK), NT_WALK * LG, (size_t)NT_WALK * TREFOLD_B, s>>>(a);
+            k_trefold<R, RT, N, M, TR, NT_WALK, MINB_REFOLD>
+                <<<blocks(a.C, NT_WALK), NT_WALK * LGW, (size_t)NT_WALK * TREFOLD_B, s>>>(a);
         else
             k_crefold<R, RT, N, M, NG_REFOLD>
                 <<<blocks(a.C, NG_REFOLD), NG_REFOLD * N, (size_t)NG_REFOLD * REFOLD_B, s>>>(a);
@@ -391,8 +399,10 @@ struct Launcher {
     static void launch_up(const Args<R, RT>& a, const long long* active, int levels,
                           cudaStream_t s) {
         if constexpr (kTeam) {
-            for (int l = 0; l < levels; l += TT_LEVELS) {
-                const TreeRun tr = tree_run(active, levels, l);
+            // a problem's root (and every node holding its first chunk) is in no
+            // suffix: level h sweeps the problems with NC >= 4h
+            for (int l = 0; l < levels - 1; l += TT_LEVELS) {
+                const TreeRun tr = tree_run(active + 1, levels - 1, l);
                 k_tup<RT, N, TT>
                     <<<tree_blocks(tr), TT * LG, (size_t)TT * TUP_B, s>>>(a.E, tr, a.status);
             }
@@ -557,6 +567,7 @@ struct Launcher {
         a.status = call.status ? call.status : reinterpret_cast<int*>(base);
         a.out_mask = 0;
         a.refine_add = 0;
+        a.first_total = call.method2 ? 1 : 0;
         // the chunk totals' region holds a copy of each chunk's Psi
         static_assert(GElem<N>::SIZE >= GAffine<N>::SIZE, "Psi copy fits the element slots");
         RT* psi = a.E;
@@ -708,6 +719,7 @@ struct Launcher {
         a.status = call.status ? call.status : reinterpret_cast<int*>(base);
         a.out_mask = 7;
         a.refine_add = 0;
+        a.first_total = call.method2 ? 1 : 0;
         if (kPersistFits && call.persistent && !refine && !method2 && !call.sequential) {
             // one cooperative launch for the whole pass (batches)
             const lqt_status st =
@@ -774,10 +786,10 @@ struct Launcher {
     }
 
     static int fold_groups_per_cta() { return kTeam ? NT_WALK : NG_FOLD; }
-    static int fold_threads() { return kTeam ? NT_WALK * LG : NG_FOLD * N; }
+    static int fold_threads() { return kTeam ? NT_WALK * LGW : NG_FOLD * N; }
     static const void* fold_kernel() {
         if constexpr (kTeam)
-            return reinterpret_cast<const void*>(k_tfold<R, RT, N, M, NT_WALK, MINB_FOLD>);
+            return reinterpret_cast<const void*>(k_tfold<R, RT, N, M, TR, NT_WALK, MINB_FOLD>);
         else
             return reinterpret_cast<const void*>(k_cfold<R, RT, N, M, NG_FOLD>);
     }

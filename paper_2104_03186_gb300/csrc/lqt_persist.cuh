@@ -181,9 +181,10 @@ __global__ void __launch_bounds__(NT* Team<N>::LG) k_cpersist(Args<R, RT> a, Lev
          c = next_chunk(&bar->next[0], slot, g))
         b_tfold<R, RT, N, M>(a, c, sh);
     if (!grid_sync(bar, nb, wait_limit, a.status)) return;
-    // 2. up-sweep levels
-    for (int l = 0; l < lp.levels; ++l) {
-        const long long h = 1ll << l, pairs = lp.active[l] / (2 * h);
+    // 2. up-sweep levels (a problem's root is in no suffix: level h sweeps the
+    // problems with NC >= 4h)
+    for (int l = 0; l + 1 < lp.levels; ++l) {
+        const long long h = 1ll << l, pairs = lp.active[l + 1] / (2 * h);
         for (long long q = first; q < pairs; q += stride) {
             RT* e = a.E + q * 2 * h * DElem<N>::SIZE;
             ok &= team::combine<N>(e, e + h * DElem<N>::SIZE, e, sht, g);

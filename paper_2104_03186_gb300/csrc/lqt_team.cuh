@@ -125,13 +125,14 @@ __device__ __forceinline__ void stg_row(R* m, int row, int col, const R (&o)[CT]
     }
 }
 
-// One team: lane = tile (ri, ci); ri in [0, N/2), ci in [0, N/4).  Left-operand
-// ("NN") tiles hold rows ri and ri + N/2, transposed-left ("TN") tiles rows
-// 2 ri and 2 ri + 1; both hold columns 4 ci .. 4 ci + 3 of N (2 ci, 2 ci + 1 of M).
-template <int N>
+// One team of LG = N^2 / (4 RT) lanes: lane = tile (ri, ci) of RT x 4 entries,
+// ri in [0, N / RT), ci in [0, N / 4).  Left-operand ("NN") tiles hold rows
+// ri + i N / RT, transposed-left ("TN") tiles rows RT ri + i, i < RT; both hold
+// columns 4 ci .. 4 ci + 3 of N (2 ci, 2 ci + 1 of M).
+template <int N, int RT = 2>
 struct Team {
-    static constexpr int LG = N * N / 8;
-    static constexpr int LC = N / 4, LR = N / 2;
+    static constexpr int LC = N / 4, LR = N / RT;
+    static constexpr int LG = LC * LR;
     static constexpr int LW = LG < 32 ? LG : 32;  // lanes in one warp
     static constexpr int NW = LG / LW;            // warps
     int lane, ri, ci;
@@ -149,6 +150,21 @@ struct Team {
         else  // one named barrier per team of the CTA (0 is __syncthreads)
             asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / LG), "n"(LG) : "memory");
     }
+    // whether x holds in every lane of the team
+    __device__ __forceinline__ bool all(bool x) const {
+        if constexpr (LG <= 32) {
+            return __all_sync(mask, x);
+        } else {
+            int r;
+            asm volatile(
+                "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n"
+                " bar.red.and.pred q, %2, %3, p;\n selp.s32 %0, 1, 0, q;\n}"
+                : "=r"(r)
+                : "r"((int)x), "r"(1 + (int)threadIdx.x / LG), "n"(LG)
+                : "memory");
+            return r != 0;
+        }
+    }
     // sum over the LC lanes of a lane row
     template <typename R>
     __device__ __forceinline__ R row_sum(R x) const {
@@ -161,32 +177,31 @@ struct Team {
 // steps of k unrolled together: whole periods of the swizzle, whole loops up to 16
 constexpr int k_unroll(int K) { return K <= 16 ? K : 8; }
 
-// acc{0,1} += sign * A[r0 | r1][0..K) B[0..K)[c0 .. c0 + CT)
-template <int K, int ACOLS, int BCOLS, int CT, bool NEG, typename R>
-__device__ __forceinline__ void nn(R (&acc0)[CT], R (&acc1)[CT], const R* A, const R* B, int r0,
-                                   int r1, int c0) {
+// acc[i] += sign * A[r0 + i step][0..K) B[0..K)[c0 .. c0 + CT)
+template <int K, int ACOLS, int BCOLS, bool NEG, int RT, int CT, typename R>
+__device__ __forceinline__ void nn(R (&acc)[RT][CT], const R* A, const R* B, int r0, int step,
+                                   int c0) {
     constexpr int E = 16 / (int)sizeof(R);
 #pragma unroll(k_unroll(K) / E)
     for (int k = 0; k < K; k += E) {
-        R a0[E], a1[E];
-        ldrow<ACOLS, E>(A, r0, k, a0);
-        ldrow<ACOLS, E>(A, r1, k, a1);
+        R a[RT][E];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) ldrow<ACOLS, E>(A, r0 + i * step, k, a[i]);
 #pragma unroll
         for (int q = 0; q < E; ++q) {
             R b[CT];
             ldrow<BCOLS, CT>(B, k + q, c0, b);
-            const R x0 = NEG ? -a0[q] : a0[q], x1 = NEG ? -a1[q] : a1[q];
 #pragma unroll
-            for (int c = 0; c < CT; ++c) {
-                acc0[c] = fma_(x0, b[c], acc0[c]);
-                acc1[c] = fma_(x1, b[c], acc1[c]);
-            }
+            for (int i = 0; i < RT; ++i)
+#pragma unroll
+                for (int c = 0; c < CT; ++c)
+                    acc[i][c] = fma_(NEG ? -a[i][q] : a[i][q], b[c], acc[i][c]);
         }
     }
 }
 
 // acc[i] += sign * sum_k A[k][r0 + i] B[k][c0 ..), i < RT
-template <int K, int ACOLS, int BCOLS, int RT, int CT, bool NEG, typename R>
+template <int K, int ACOLS, int BCOLS, bool NEG, int RT, int CT, typename R>
 __device__ __forceinline__ void tn(R (&acc)[RT][CT], const R* A, const R* B, int r0, int c0) {
 #pragma unroll(k_unroll(K))
     for (int k = 0; k < K; ++k) {
@@ -210,46 +225,82 @@ __device__ __forceinline__ void zero(R (&a)[RT][CT]) {
 
 // tile <- (tile + transpose) / 2 for a TN tile whose raw values of all lanes
 // are in `raw` (N x N)
-template <int N, typename R>
-__device__ __forceinline__ void symmetrise(R (&t)[2][4], const R* raw, const Team<N>& g) {
+template <int N, int RT, typename R>
+__device__ __forceinline__ void symmetrise(R (&t)[RT][4], const R* raw, const Team<N, RT>& g) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        R x[2];
-        ldrow<N, 2>(raw, 4 * g.ci + c, 2 * g.ri, x);
-        t[0][c] = R(0.5) * (t[0][c] + x[0]);
-        t[1][c] = R(0.5) * (t[1][c] + x[1]);
+        R x[RT];
+        ldrow<N, RT>(raw, 4 * g.ci + c, RT * g.ri, x);
+#pragma unroll
+        for (int i = 0; i < RT; ++i) t[i][c] = R(0.5) * (t[i][c] + x[i]);
     }
 }
 
-// G Z = B for a symmetric positive definite G (M x M) by Gauss-Jordan
-// elimination without pivoting.  Column-per-lane: every warp of the team holds
-// the M columns of G and its share of the NR right sides in registers, the
-// pivot column's entries come from its lane by shuffles, and no sync is needed
-// before the caller's.  get(r, col) fills right side r, put(r, col) takes its
-// solution.
-template <int M, int NR, int N, typename R, typename Get, typename Put>
-__device__ __forceinline__ bool solve_spd(const R* G, const Team<N>& g, Get get, Put put) {
-    using T = Team<N>;
+// RT rows r0 + i step of a swizzled matrix, columns c0 .. c0 + CT
+template <int COLS, int RT, int CT, typename R>
+__device__ __forceinline__ void ldtile(const R* m, int r0, int step, int c0, R (&t)[RT][CT]) {
+#pragma unroll
+    for (int i = 0; i < RT; ++i) ldrow<COLS, CT>(m, r0 + i * step, c0, t[i]);
+}
+template <int COLS, int RT, int CT, typename R>
+__device__ __forceinline__ void sttile(R* m, int r0, int step, int c0, const R (&t)[RT][CT]) {
+#pragma unroll
+    for (int i = 0; i < RT; ++i) strow<COLS, CT>(m, r0 + i * step, c0, t[i]);
+}
+
+// The system [G | B] of an m x m solve in shared memory: M rows, G's M columns
+// and then NR right sides, row stride LD.  A lane reads whole columns, so the
+// solve's loads and stores are one uniform sweep over the rows; LD = 4 mod 16
+// keeps rows 16-byte aligned for the products that read it and spreads the
+// transposed stores of P2 over the banks.
+template <int N, int M, int NR>
+struct Sys {
+    static constexpr int B = M;  // first right side
+    static constexpr int LD = N == 8 ? (M + NR + 3) / 4 * 4 : (M + NR - 4 + 15) / 16 * 16 + 4;
+    static constexpr int SIZE = M * LD;
+    static_assert(LD >= M + NR, "all columns fit");
+};
+template <int LD, int CT, typename R>
+__device__ __forceinline__ void ldsys(const R* t, int row, int col, R (&o)[CT]) {
+    constexpr int E = 16 / (int)sizeof(R), V = CT < E ? CT : E;
+#pragma unroll
+    for (int v = 0; v < CT; v += V) ldv<V>(t + row * LD + col + v, o + v);
+}
+template <int LD, int CT, typename R>
+__device__ __forceinline__ void stsys(R* t, int row, int col, const R (&o)[CT]) {
+    constexpr int E = 16 / (int)sizeof(R), V = CT < E ? CT : E;
+#pragma unroll
+    for (int v = 0; v < CT; v += V) stv<V>(t + row * LD + col + v, o + v);
+}
+
+// 1 / sqrt(x) to within an ulp: the hardware's approximation and one Newton
+// step (FP32; x > 0 and normal), two correctly rounded steps (FP64)
+__device__ __forceinline__ float rsqrt_(float x) {
+    const float y = rsqrtf(x);
+    return fmaf(0.5f * y, fmaf(-x * y, y, 1.0f), y);
+}
+__device__ __forceinline__ double rsqrt_(double x) { return 1.0 / sqrt(x); }
+
+// The M x M systems above by elimination without pivoting (stable for SPD G).
+// Column-per-lane: every warp of the team holds the M columns of G and its
+// share of the right sides in registers; the pivot column's entries come from
+// its lane by shuffles, and no sync is needed before the caller's.  FULL: the
+// right sides become G^{-1} B (Gauss-Jordan); otherwise Rc^{-1} B with
+// G = Rc Rc^T (the forward half of a Cholesky solve, half the work).
+template <bool FULL, int M, int NR, int N, int RT, typename R>
+__device__ __forceinline__ bool solve_spd(R* t, const Team<N, RT>& g) {
+    using T = Team<N, RT>;
+    using S = Sys<N, M, NR>;
     constexpr int NRW = (NR + T::NW - 1) / T::NW;
     constexpr int COLS = M + NRW, SL = (COLS + T::LW - 1) / T::LW;
     const int lw = g.lane % T::LW, wi = g.lane / T::LW;
     R col[SL][M];
 #pragma unroll
     for (int s = 0; s < SL; ++s) {
-        const int j = s * T::LW + lw, r = wi * NRW + (j - M);
+        const int j = s * T::LW + lw, c = j < M ? j : j + wi * NRW;
+        const bool in = j < COLS && c < M + NR;
 #pragma unroll
-        for (int i = 0; i < M; ++i) col[s][i] = R(0);
-        if (j < M) {
-#pragma unroll
-            for (int i = 0; i < M; i += 2) {
-                R x[2];
-                ldrow<M, 2>(G, j, i, x);
-                col[s][i] = x[0];
-                col[s][i + 1] = x[1];
-            }
-        } else if (j < COLS && r < NR) {
-            get(r, col[s]);
-        }
+        for (int i = 0; i < M; ++i) col[s][i] = in ? t[i * S::LD + c] : R(0);
     }
     bool ok = true;
 #pragma unroll
@@ -257,21 +308,27 @@ __device__ __forceinline__ bool solve_spd(const R* G, const Team<N>& g, Get get,
         const int ks = k / T::LW, kl = k % T::LW;
         const R piv = __shfl_sync(g.mask, col[ks][k], kl, T::LW);
         ok = ok && piv > R(0) && isfinite(piv);
-        const R inv = rcp(piv);
+        const R sc = FULL ? rcp(piv) : rsqrt_(piv);
         R f[M];
 #pragma unroll
-        for (int i = 0; i < M; ++i) f[i] = __shfl_sync(g.mask, col[ks][i], kl, T::LW) * inv;
+        for (int i = 0; i < M; ++i)
+            if (i > k || (FULL && i < k)) f[i] = __shfl_sync(g.mask, col[ks][i], kl, T::LW);
 #pragma unroll
         for (int s = 0; s < SL; ++s) {
-            const R pk = col[s][k];
+            const R pk = col[s][k] * sc, fk = FULL ? pk : pk * sc;
 #pragma unroll
-            for (int i = 0; i < M; ++i) col[s][i] = i == k ? pk * inv : fma_(-f[i], pk, col[s][i]);
+            for (int i = 0; i < M; ++i)
+                if (i > k || (FULL && i < k)) col[s][i] = fma_(-f[i], fk, col[s][i]);
+            col[s][k] = pk;
         }
     }
 #pragma unroll
     for (int s = 0; s < SL; ++s) {
-        const int j = s * T::LW + lw, r = wi * NRW + (j - M);
-        if (j >= M && j < COLS && r < NR) put(r, col[s]);
+        const int j = s * T::LW + lw, c = j + wi * NRW;
+        if (j >= M && j < COLS && c < M + NR) {
+#pragma unroll
+            for (int i = 0; i < M; ++i) t[i * S::LD + c] = col[s][i];
+        }
     }
     return ok;
 }
@@ -401,15 +458,14 @@ __device__ bool combine(const R* e1, const R* e2, R* out, R* sh, const Team<N>& 
     g.sync();
     // M = I + C1 J2 ; be = b1 + C1 eta2 ; w = eta2 - J2 b1
     {
-        R a0[4], a1[4];
+        R a[2][4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            a0[c] = ri == 4 * ci + c ? R(1) : R(0);
-            a1[c] = ri + H == 4 * ci + c ? R(1) : R(0);
+            a[0][c] = ri == 4 * ci + c ? R(1) : R(0);
+            a[1][c] = ri + H == 4 * ci + c ? R(1) : R(0);
         }
-        nn<N, N, N, 4, false>(a0, a1, sh + S::C1, sh + S::J2, ri, ri + H, 4 * ci);
-        strow<N, 4>(sh + S::MX, ri, 4 * ci, a0);
-        strow<N, 4>(sh + S::MX, ri + H, 4 * ci, a1);
+        nn<N, N, N, false>(a, sh + S::C1, sh + S::J2, ri, H, 4 * ci);
+        sttile<N>(sh + S::MX, ri, H, 4 * ci, a);
         R s[4] = {R(0), R(0), R(0), R(0)};
         R x0[4], x1[4], y0[4], y1[4];
         ldrow<N, 4>(sh + S::C1, ri, 4 * ci, x0);
@@ -475,9 +531,9 @@ __device__ bool combine(const R* e1, const R* e2, R* out, R* sh, const Team<N>& 
         zero(aa);
         zero(jx);
         zero(t);
-        nn<N, N, N, 4, false>(jx[0], jx[1], sh + S::J2, sh + S::MX, ri, ri + H, 4 * ci);
-        nn<N, N, N, 4, false>(aa[0], aa[1], sh + S::A2, sh + S::MX, ri, ri + H, 4 * ci);
-        nn<N, N, N, 4, false>(t[0], t[1], sh + S::A2, sh + S::X3, ri, ri + H, 4 * ci);
+        nn<N, N, N, false>(jx, sh + S::J2, sh + S::MX, ri, H, 4 * ci);
+        nn<N, N, N, false>(aa, sh + S::A2, sh + S::MX, ri, H, 4 * ci);
+        nn<N, N, N, false>(t, sh + S::A2, sh + S::X3, ri, H, 4 * ci);
         strow<N, 4>(sh + S::JX, ri, 4 * ci, jx[0]);
         strow<N, 4>(sh + S::JX, ri + H, 4 * ci, jx[1]);
         strow<N, 4>(sh + S::T, ri, 4 * ci, t[0]);
@@ -507,7 +563,7 @@ __device__ bool combine(const R* e1, const R* e2, R* out, R* sh, const Team<N>& 
     }
     g.sync();
     // J = J1 + A1^T JX ; C = C2 + T A2^T
-    tn<N, N, N, 2, 4, false>(jj, sh + S::A1, sh + S::JX, 2 * ri, 4 * ci);
+    tn<N, N, N, false>(jj, sh + S::A1, sh + S::JX, 2 * ri, 4 * ci);
     {
         constexpr int EP = 16 / (int)sizeof(R);
 #pragma unroll 1
@@ -571,15 +627,14 @@ __device__ bool value_apply(const R* P, const R* val, R* out, R* sh, const Team<
     const R h0 = P[E::OE + 2 * ri], h1 = P[E::OE + 2 * ri + 1];
     g.sync();
     {
-        R a0[4], a1[4], x0[4], x1[4];
+        R a[2][4], x0[4], x1[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            a0[c] = ri == 4 * ci + c ? R(1) : R(0);
-            a1[c] = ri + H == 4 * ci + c ? R(1) : R(0);
+            a[0][c] = ri == 4 * ci + c ? R(1) : R(0);
+            a[1][c] = ri + H == 4 * ci + c ? R(1) : R(0);
         }
-        nn<N, N, N, 4, false>(a0, a1, sh + S::C, sh + S::S, ri, ri + H, 4 * ci);
-        strow<N, 4>(sh + S::MX, ri, 4 * ci, a0);
-        strow<N, 4>(sh + S::MX, ri + H, 4 * ci, a1);
+        nn<N, N, N, false>(a, sh + S::C, sh + S::S, ri, H, 4 * ci);
+        sttile<N>(sh + S::MX, ri, H, 4 * ci, a);
         ldrow<N, 4>(sh + S::S, ri, 4 * ci, x0);
         ldrow<N, 4>(sh + S::S, ri + H, 4 * ci, x1);
         R s0 = R(0), s1 = R(0);
@@ -627,7 +682,7 @@ __device__ bool value_apply(const R* P, const R* val, R* out, R* sh, const Team<
     {
         R t[2][4];
         zero(t);
-        nn<N, N, N, 4, false>(t[0], t[1], sh + S::S, sh + S::MX, ri, ri + H, 4 * ci);
+        nn<N, N, N, false>(t, sh + S::S, sh + S::MX, ri, H, 4 * ci);
         strow<N, 4>(sh + S::T, ri, 4 * ci, t[0]);
         strow<N, 4>(sh + S::T, ri + H, 4 * ci, t[1]);
         R s0 = R(0), s1 = R(0);
@@ -646,7 +701,7 @@ __device__ bool value_apply(const R* P, const R* val, R* out, R* sh, const Team<
         }
     }
     g.sync();
-    tn<N, N, N, 2, 4, false>(jj, sh + S::A, sh + S::T, 2 * ri, 4 * ci);
+    tn<N, N, N, false>(jj, sh + S::A, sh + S::T, 2 * ri, 4 * ci);
     strow<N, 4>(sh + S::C, 2 * ri, 4 * ci, jj[0]);  // C is no longer read
     strow<N, 4>(sh + S::C, 2 * ri + 1, 4 * ci, jj[1]);
     g.sync();
@@ -670,7 +725,7 @@ __device__ void affine_compose(const R* f1, const R* f2, R* out, R* sh, const Te
     g.sync();
     R t[2][4], x0[4], x1[4];
     zero(t);
-    nn<N, N, N, 4, false>(t[0], t[1], sh, sh + N * N, ri, ri + H, 4 * ci);
+    nn<N, N, N, false>(t, sh, sh + N * N, ri, H, 4 * ci);
     ldrow<N, 4>(sh, ri, 4 * ci, x0);
     ldrow<N, 4>(sh, ri + H, 4 * ci, x1);
     R s0 = R(0), s1 = R(0);
