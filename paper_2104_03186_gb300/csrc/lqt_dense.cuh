@@ -679,6 +679,188 @@ __device__ __forceinline__ void value_replay(const R* fac, int fs, ElemView<R, N
     for (int i = 0; i < N; ++i) v[i] = vn[i];
 }
 
+// ---------------------------------------------------------------------------
+// Column forms of the operators: a team of N neighbouring lanes shares one
+// operator, lane j computing column j of every matrix result and entry j of
+// every vector.  The N x N elimination is repeated by each lane for its own
+// right sides alone, so the lanes exchange nothing: no shuffles, and per lane
+// about half the instructions of the one-thread form.  The C column uses
+//   C e_j = A2 M^{-1} (C1 (A2^T e_j)) + C2 e_j,
+// so that lane j never needs another lane's solves.  Results stay in registers
+// until the team has read its operands (out may alias one of them): the
+// caller separates compute and store by a warp sync.
+// ---------------------------------------------------------------------------
+template <typename R, int N>
+struct ElemCol {  // column j of A, C, J; entry j of b, eta
+    R A[N], C[N], J[N];
+    R b, eta;
+};
+
+template <typename R, int N, bool REC = false>
+__device__ __forceinline__ bool combine_col(ElemView<R, N> e1, ElemView<R, N> e2, int j,
+                                            ElemCol<R, N>& o, R* fac = nullptr, int fs = 1) {
+    constexpr int NR = 3 + (REC ? 2 : 0);
+    R Mx[N][N], B[N][NR];  // A1 e_j | b1 + C1 eta2 | C1 A2^T e_j  (REC: | e_j | C1 e_j)
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+#pragma unroll
+        for (int l = 0; l < N; ++l) Mx[i][l] = (i == l) ? R(1) : R(0);
+        R t = e1.b(i), z = R(0);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const R c = e1.C(i, k);
+#pragma unroll
+            for (int l = 0; l < N; ++l) Mx[i][l] += c * e2.J(k, l);
+            t += c * e2.eta(k);
+            z += c * e2.A(j, k);
+        }
+        B[i][0] = e1.A(i, j);
+        B[i][1] = t;
+        B[i][2] = z;
+        if constexpr (REC) {
+            B[i][3] = (i == j) ? R(1) : R(0);
+            B[i][4] = e1.C(i, j);
+        }
+    }
+    const bool ok = solve_pivoted<R, N, NR>(Mx, B);
+    R x[N], jx[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) x[k] = B[k][0];
+    // eta_j = x . (eta2 - J2 b1) + eta1_j ; jx = J2 x
+    R eta = e1.eta(j);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        R w = e2.eta(i), t = R(0);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            w -= e2.J(i, k) * e1.b(k);
+            t += e2.J(i, k) * x[k];
+        }
+        jx[i] = t;
+        eta += x[i] * w;
+    }
+    o.eta = eta;
+    R b = e2.b(j);
+#pragma unroll
+    for (int k = 0; k < N; ++k) b += e2.A(j, k) * B[k][1];
+    o.b = b;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        R a = R(0), c = e2.C(i, j), jj = e1.J(i, j);
+        R g1 = R(0), g2 = R(0);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const R a2 = e2.A(i, k);
+            a += a2 * x[k];
+            c += a2 * B[k][2];
+            jj += e1.A(k, i) * jx[k];
+            if constexpr (REC) {
+                g1 += a2 * B[k][3];
+                g2 += a2 * B[k][4];
+            }
+        }
+        o.A[i] = a;
+        o.C[i] = c;
+        o.J[i] = jj;
+        if constexpr (REC) {
+            fac[(i * N + j) * fs] = g1;
+            fac[(N * N + i * N + j) * fs] = g2;
+            fac[(2 * N * N + j * N + i) * fs] = x[i];
+            fac[(3 * N * N + j * N + i) * fs] = -jx[i];
+        }
+    }
+    return ok;
+}
+
+// Column j of an element; the upper triangle of C and J is stored.
+template <typename R, int N>
+__device__ __forceinline__ void store_col(const ElemCol<R, N>& o, int j, ElemView<R, N> out) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        out.A(i, j) = o.A[i];
+        if (i <= j) {
+            out.C(i, j) = o.C[i];
+            out.J(i, j) = o.J[i];
+        }
+    }
+    out.b(j) = o.b;
+    out.eta(j) = o.eta;
+}
+
+// combine_replay's entry j of (b, eta).
+template <typename R, int N>
+__device__ __forceinline__ void combine_replay_row(const R* fac, int fs, ElemView<R, N> e1,
+                                                   ElemView<R, N> e2, int j, R& b, R& h) {
+    b = e2.b(j);
+    h = e1.eta(j);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const R b1 = e1.b(k), h2 = e2.eta(k);
+        b += fac[(j * N + k) * fs] * b1 + fac[(N * N + j * N + k) * fs] * h2;
+        h += fac[(2 * N * N + j * N + k) * fs] * h2 + fac[(3 * N * N + j * N + k) * fs] * b1;
+    }
+}
+
+// value_apply's column j of S and entry j of v, for the value in view `in`.
+template <typename R, int N, bool REC = false>
+__device__ __forceinline__ bool value_apply_col(ElemView<R, N> P, ValueView<R, N> in, int j,
+                                                R (&Sc)[N], R& vj, R* fac = nullptr, int fs = 1) {
+    R Mx[N][N], X[N][1];
+    R S[Dims<N>::SYM];
+#pragma unroll
+    for (int k = 0; k < Dims<N>::SYM; ++k) S[k] = in.p[k * in.s];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+#pragma unroll
+        for (int l = 0; l < N; ++l) Mx[i][l] = (i == l) ? R(1) : R(0);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const R c = P.C(i, k);
+#pragma unroll
+            for (int l = 0; l < N; ++l) Mx[i][l] += c * S[sym<N>(k, l)];
+        }
+        X[i][0] = P.A(i, j);
+    }
+    const bool ok = solve_pivoted<R, N, 1>(Mx, X);
+    R sx[N];
+    R v = P.eta(j);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        R e = in.v(i), t = R(0);
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            e -= S[sym<N>(i, k)] * P.b(k);
+            t += S[sym<N>(i, k)] * X[k][0];
+        }
+        sx[i] = t;
+        v += X[i][0] * e;
+    }
+    vj = v;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        R t = P.J(i, j);
+#pragma unroll
+        for (int k = 0; k < N; ++k) t += P.A(k, i) * sx[k];
+        Sc[i] = t;
+        if constexpr (REC) {
+            fac[(j * N + i) * fs] = X[i][0];
+            fac[(N * N + j * N + i) * fs] = -sx[i];
+        }
+    }
+    return ok;
+}
+
+// value_replay's entry j of v.
+template <typename R, int N>
+__device__ __forceinline__ R value_replay_row(const R* fac, int fs, ElemView<R, N> P,
+                                              ValueView<R, N> in, int j) {
+    R t = P.eta(j);
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        t += fac[(j * N + k) * fs] * in.v(k) + fac[(N * N + j * N + k) * fs] * P.b(k);
+    return t;
+}
+
 template <typename R, int N>
 __device__ __forceinline__ void load_value(Value<R, N>& val, ValueView<R, N> in) {
 #pragma unroll

@@ -426,6 +426,72 @@ constexpr int tile_threads() {
     return tile_smem_bytes_max<R, N, M, w>() <= 227 * 1024 ? w : w / 2;
 }
 
+// Teams of N lanes share one operator (the column forms of lqt_dense.cuh) in
+// the tree levels with few pairs; the levels with more run one thread per pair.
+// FP64 levels are bound by the FP64 pipe (a warp instruction takes 16 cycles of
+// an SM): a team's warp issues about half the instructions of a
+// thread-per-pair warp but holds a quarter of the pairs, so teams win up to one
+// warp of them (n = 4, T = 30011: 655 -> 536 us).  FP32 levels are bound by the
+// operator's latency: a team level of up to four warps (one per scheduler)
+// takes about 1350 cycles against 2300 for a thread per pair, one of 16 warps
+// 4100.  ONE_CTA: the kernels whose trees are the whole grid's critical path
+// (k_bwd_top, k_solo).  The per-tile kernels of a larger FP32 problem, where
+// 152 CTAs fetch the code of both forms, lost (T = 100003, time-varying model:
+// 249 -> 254 us) and keep the thread form.
+template <typename R, int N, bool ONE_CTA>
+__host__ __device__ constexpr bool team_level(int pairs) {
+    return N == 4 && (ONE_CTA || sizeof(R) == 8) && pairs * N <= (sizeof(R) == 4 ? 128 : 32);
+}
+
+// One up-sweep level by teams: slots i = 2h t and i + h into i.
+template <typename R, int N>
+__device__ __forceinline__ bool team_combine_level(R* tree, int ts, int h, int pairs, int tid) {
+    const int t = tid / N, j = tid % N, i = 2 * h * t;
+    const bool act = t < pairs;
+    ElemCol<R, N> o;
+    bool ok = true;
+    const ElemView<R, N> e1{tree + tslot<R>(i), ts}, e2{tree + tslot<R>(i + h), ts};
+    if (act) ok = combine_col<R, N>(e1, e2, j, o);
+    __syncwarp();
+    if (act) store_col(o, j, e1);
+    return ok;
+}
+
+// One value down-sweep level by teams: carry[i + h] <- carry[i], then carry[i]
+// through the element of slot i + h.
+template <typename R, int N>
+__device__ __forceinline__ void team_store_value(ValueView<R, N> in, ValueView<R, N> out, int j,
+                                                 const R (&Sc)[N], R v) {
+    R So[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (i <= j) So[i] = in.S(i, j);
+    const R vo = in.v(j);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (i <= j) {
+            out.S(i, j) = So[i];
+            in.S(i, j) = Sc[i];
+        }
+    out.v(j) = vo;
+    in.v(j) = v;
+}
+
+template <typename R, int N>
+__device__ __forceinline__ bool team_apply_level(R* tree, R* carry, int ts, int h, int pairs,
+                                                 int tid) {
+    const int t = tid / N, j = tid % N, i = 2 * h * t;
+    const bool act = t < pairs;
+    bool ok = true;
+    R Sc[N], v = R(0);
+    const ValueView<R, N> ci{carry + tslot<R>(i), ts}, ch{carry + tslot<R>(i + h), ts};
+    if (act)
+        ok = value_apply_col<R, N>(ElemView<R, N>{tree + tslot<R>(i + h), ts}, ci, j, Sc, v);
+    __syncwarp();
+    if (act) team_store_value<R, N>(ci, ch, j, Sc, v);
+    return ok;
+}
+
 // ===========================================================================
 // bwd_up: chunk fold + in-tile up-sweep (left-anchored: after level d, slot
 // i = j * 2^{d+1} holds the total of chunks [i, i + 2^{d+1}); slot i + 2^d
@@ -460,7 +526,9 @@ __device__ __forceinline__ void bwd_up_body(const Params<R>& P, unsigned tile, R
 #pragma unroll 1
     for (int h = 1; h < Weff; h <<= 1) {
         const int i = tid * 2 * h;
-        if (i < Weff)
+        if (team_level<R, N, SOLO>(Weff / (2 * h)))
+            ok2 &= team_combine_level<R, N>(tree, WS, h, Weff / (2 * h), tid);
+        else if (i < Weff)
             ok2 &= combine_view<R, N>(ElemView<R, N>{tree + tslot<R>(i), WS},
                                       ElemView<R, N>{tree + tslot<R>(i + h), WS},
                                       ElemView<R, N>{tree + tslot<R>(i), WS});
@@ -630,7 +698,26 @@ __global__ void __launch_bounds__(TP, 1) k_bwd_top(const Params<R> P) {
 #pragma unroll 1
     for (int h = 1; h < Teff; h <<= 1) {
         const int i = tid * 2 * h;
-        if (i < Teff) {
+        if (team_level<R, N, true>(Teff / (2 * h))) {
+            const int t = tid / N, j = tid % N, it = 2 * h * t;
+            const bool act = t < Teff / (2 * h);
+            const ElemView<R, N> e1{tree + tslot<R>(it), TS}, e2{tree + tslot<R>(it + h), TS};
+            if (mode == 2) {
+                R b = R(0), eta = R(0);
+                if (act) combine_replay_row<R, N>(sfac + node + t, TP, e1, e2, j, b, eta);
+                __syncwarp();
+                if (act) {
+                    e1.b(j) = b;
+                    e1.eta(j) = eta;
+                }
+            } else {
+                ElemCol<R, N> o;
+                if (act)
+                    ok &= combine_col<R, N, mode == 1>(e1, e2, j, o, P.top_fac + node + t, TP);
+                __syncwarp();
+                if (act) store_col(o, j, e1);
+            }
+        } else if (i < Teff) {
             const ElemView<R, N> e1{tree + tslot<R>(i), TS}, e2{tree + tslot<R>(i + h), TS};
             if (mode == 2)
                 combine_replay<R, N>(sfac + node + tid, TP, e1, e2, e1);
@@ -649,7 +736,30 @@ __global__ void __launch_bounds__(TP, 1) k_bwd_top(const Params<R> P) {
 #pragma unroll 1
     for (int h = Teff / 2; h >= 1; h >>= 1) {
         const int i = tid * 2 * h;
-        if (i < Teff) {
+        if (team_level<R, N, true>(Teff / (2 * h))) {
+            const int t = tid / N, j = tid % N, it = 2 * h * t;
+            const bool act = t < Teff / (2 * h);
+            const ValueView<R, N> ci{carry + tslot<R>(it), TS}, ch{carry + tslot<R>(it + h), TS};
+            const ElemView<R, N> el{tree + tslot<R>(it + h), TS};
+            R v = R(0), vo = R(0);
+            if (mode == 2) {
+                if (act) {
+                    v = value_replay_row<R, N>(sdn + node + t, TP, el, ci, j);
+                    vo = ci.v(j);
+                }
+                __syncwarp();
+                if (act) {
+                    ch.v(j) = vo;
+                    ci.v(j) = v;
+                }
+            } else {
+                R Sc[N];
+                if (act)
+                    ok &= value_apply_col<R, N, mode == 1>(el, ci, j, Sc, v, gdn + node + t, TP);
+                __syncwarp();
+                if (act) team_store_value<R, N>(ci, ch, j, Sc, v);
+            }
+        } else if (i < Teff) {
             const ValueView<R, N> ci{carry + tslot<R>(i), TS}, ch{carry + tslot<R>(i + h), TS};
             const ElemView<R, N> el{tree + tslot<R>(i + h), TS};
             if (mode == 2) {
@@ -776,7 +886,9 @@ __device__ __forceinline__ void bwd_down_body(const Params<R>& P, unsigned tile,
 #pragma unroll 1
     for (int h = Weff / 2; h >= 1; h >>= 1) {
         const int i = tid * 2 * h;
-        if (i < Weff) {
+        if (team_level<R, N, SOLO>(Weff / (2 * h))) {
+            ok_sing &= team_apply_level<R, N>(tree, carry, WS, h, Weff / (2 * h), tid);
+        } else if (i < Weff) {
             Value<R, N> c;
             load_value(c, ValueView<R, N>{carry + tslot<R>(i), WS});
             store_value(c, ValueView<R, N>{carry + tslot<R>(i + h), WS});
