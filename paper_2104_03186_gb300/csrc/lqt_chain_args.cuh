@@ -23,6 +23,7 @@ struct Item {
     int pad_;
     R* u_out;      // correction pass: the output u* (holds u^ until then)
     const R* qh;   // correction pass: U^{-1} h_k (T x M)
+    R* gi;         // refinement: G_k^{-1} of the first pass (T x M x M), or nullptr
 };
 
 template <typename R, typename RT>
@@ -36,6 +37,7 @@ struct Args {
     RT* X;           // C chunk start states
     int* status;
     int out_mask;    // bit 1: write S; bit 2: write K; bit 4: write v
+    RT* maps;        // refinement: a copy of every chunk map, or nullptr
     int first_total; // 1: the totals of the problems' first chunks are wanted (Method 2)
     int refine_add;  // 1: correction pass: x <- x^ + dx, u_out <- u^ + w - qh
 };

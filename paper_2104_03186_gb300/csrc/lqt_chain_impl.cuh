@@ -12,6 +12,7 @@
 #include "lqt_chain.cuh"
 #include "lqt_chain_api.h"
 #include "lqt_persist.cuh"
+#include "lqt_vector_walk.cuh"
 #include "lqt_warm.cuh"
 #include "lqt_launch.cuh"
 #include "lqt_upload.cuh"
@@ -102,6 +103,9 @@ struct Launcher {
     static constexpr int TUP_B = tstride_of<N, RT>(team::CombineSmem<N>::SIZE) * (int)sizeof(RT);
     static constexpr int TDOWN_B = tstride_of<N, RT>(team::ApplySmem<N>::SIZE) * (int)sizeof(RT);
     static constexpr int TFUP_B = tstride_of<N, RT>(2 * N * N) * (int)sizeof(RT);
+    using VW = VWalk<N, M>;
+    static constexpr int VFWD_B = VW::NT * VW::FWD_SIZE * (int)sizeof(R);
+    static constexpr int VBACK_B = VW::NT * VW::BACK_SIZE * (int)sizeof(R);
     static constexpr int NG_FOLD = groups_for<N>(FOLD_B);
     static constexpr int NG_REFOLD = groups_for<N>(REFOLD_B);
     static constexpr int NG_UP = groups_for<N>(UP_B);
@@ -140,6 +144,13 @@ struct Launcher {
                 (e = chain_allow_smem(k_tfup<RT, N, TT>, d_fup, (size_t)TT * TFUP_B)) !=
                     cudaSuccess)
                 return e;
+            static std::atomic<bool> d_vf[64], d_vfm[64], d_vb[64], d_vbm[64];
+            if ((e = chain_allow_smem(k_vfwd<R, RT, N, M, false>, d_vf, VFWD_B)) != cudaSuccess ||
+                (e = chain_allow_smem(k_vfwd<R, RT, N, M, true>, d_vfm, VFWD_B)) != cudaSuccess ||
+                (e = chain_allow_smem(k_vback<R, RT, N, M, false>, d_vb, VBACK_B)) !=
+                    cudaSuccess ||
+                (e = chain_allow_smem(k_vback<R, RT, N, M, true>, d_vbm, VBACK_B)) != cudaSuccess)
+                return e;
         } else if ((e = chain_allow_smem(k_cfold<R, RT, N, M, NG_FOLD>, d_fold,
                                   (size_t)NG_FOLD * FOLD_B)) != cudaSuccess ||
             (e = chain_allow_smem(k_crefold<R, RT, N, M, NG_REFOLD>, d_refold,
@@ -177,7 +188,10 @@ struct Launcher {
             (e = chain_allow_smem(k_ngains<R, N, M, NG_NEWTON>, d_ngain,
                                   (size_t)NG_NEWTON * NEWTON_B)) != cudaSuccess)
             return e;
-        return chain_allow_smem(k_croll<R, RT, N, M, NG_ROLL>, d_roll, (size_t)NG_ROLL * ROLL_B);
+        if constexpr (!kTeam)
+            return chain_allow_smem(k_croll<R, RT, N, M, NG_ROLL>, d_roll,
+                                    (size_t)NG_ROLL * ROLL_B);
+        return cudaSuccess;
     }
 
     static cudaError_t prepare_warm() {
@@ -247,7 +261,7 @@ struct Launcher {
 
     // Workspace layout of a call (bytes from the start of the workspace).
     struct Layout {
-        size_t items1, items2, items3, consts, bar, E, V, FE, X, E2, Pref, refine0, total;
+        size_t items1, items2, items3, consts, bar, E, V, FE, X, maps, E2, Pref, refine0, total;
         long long C;
     };
 
@@ -280,6 +294,8 @@ struct Launcher {
         off += up(nc * GAffine<N>::SIZE * sizeof(RT));
         L.X = off;
         off += up(nc * N * sizeof(RT));
+        L.maps = off;  // the first pass's chunk maps, for the correction pass
+        if (refine && kTeam) off += up(nc * GAffine<N>::SIZE * sizeof(RT));
         L.E2 = L.Pref = 0;
         if (method2) {  // Method 2: a copy of the chunk totals and the prefixes
             L.E2 = off;
@@ -302,7 +318,8 @@ struct Launcher {
     static size_t kkt_bytes(long long T) {
         const size_t t = (size_t)T;
         return 2 * up(t * N * sizeof(R)) + 2 * up(t * M * sizeof(R)) + 2 * up(N * sizeof(R)) +
-               up((t + 1) * N * sizeof(R)) /* v' of the correction pass (Method 2) */;
+               up((t + 1) * N * sizeof(R)) /* v' of the correction pass (Method 2) */ +
+               (kTeam ? up(t * M * M * sizeof(R)) : 0) /* G^{-1} of the first pass */;
     }
     static size_t newton_bytes(long long T) {
         const size_t t = (size_t)T;
@@ -394,6 +411,15 @@ struct Launcher {
         else
             k_crefold<R, RT, N, M, NG_REFOLD>
                 <<<blocks(a.C, NG_REFOLD), NG_REFOLD * N, (size_t)NG_REFOLD * REFOLD_B, s>>>(a);
+    }
+    // rollout
+    static void launch_roll(const Args<R, RT>& a, cudaStream_t s) {
+        if constexpr (kTeam)
+            k_vfwd<R, RT, N, M, false>
+                <<<blocks(a.C, VW::NT), 32 * VW::NT, VFWD_B, s>>>(a, nullptr);
+        else
+            k_croll<R, RT, N, M, NG_ROLL>
+                <<<blocks(a.C, NG_ROLL), NG_ROLL * N, (size_t)NG_ROLL * ROLL_B, s>>>(a);
     }
     // up-sweep of the chunk totals
     static void launch_up(const Args<R, RT>& a, const long long* active, int levels,
@@ -489,8 +515,7 @@ struct Launcher {
             affine_scan(a.FE, a.X, active, levels, s);
         }
         prof_mark(prof, s, pname(kind, 5));
-        k_croll<R, RT, N, M, NG_ROLL>
-            <<<blocks(C, NG_ROLL), NG_ROLL * N, (size_t)NG_ROLL * ROLL_B, s>>>(a);
+        launch_roll(a, s);
     }
 
     // Forward affine scan of the maps FE from the seeds in each problem's top
@@ -516,6 +541,31 @@ struct Launcher {
                 k_cfdown<RT, N, NG_FDOWN><<<blocks(active[l] / (2 * h), NG_FDOWN), NG_FDOWN * N,
                                             (size_t)NG_FDOWN * FDOWN_B, s>>>(FE, X, active[l], h);
             }
+        }
+    }
+
+    // The correction pass by vector walks (lqt_vector_walk.cuh): Method 1 of the
+    // parallel solve at the team sizes.  Method 2 and the sequential recursion
+    // solve the correction problem with their own passes.
+    static bool vector_correction(const ChainCall& call) {
+        return kTeam && call.refine && !call.method2 && !call.sequential;
+    }
+    static void correct(const Args<R, RT>& b, const RT* maps, const long long* active, int levels,
+                        cudaStream_t s, Prof* prof) {
+        if constexpr (kTeam) {
+            const unsigned grid = (unsigned)blocks(b.C, VW::NT), block = 32 * VW::NT;
+            prof_mark(prof, s, "chain_vback.refine");
+            if (levels > 0)
+                k_vback<R, RT, N, M, true><<<grid, block, VBACK_B, s>>>(b, maps);
+            k_vseed<R, RT, N, true><<<b.count, N, 0, s>>>(b);
+            affine_scan(b.FE, b.X, active, levels, s);
+            k_vback<R, RT, N, M, false><<<grid, block, VBACK_B, s>>>(b, maps);
+            prof_mark(prof, s, "chain_vfwd.refine");
+            if (levels > 0)
+                k_vfwd<R, RT, N, M, true><<<grid, block, VFWD_B, s>>>(b, maps);
+            k_vseed<R, RT, N, false><<<b.count, N, 0, s>>>(b);
+            affine_scan(b.FE, b.X, active, levels, s);
+            launch_roll(b, s);
         }
     }
 
@@ -567,7 +617,8 @@ struct Launcher {
         a.status = call.status ? call.status : reinterpret_cast<int*>(base);
         a.out_mask = 0;
         a.refine_add = 0;
-        a.first_total = call.method2 ? 1 : 0;
+        a.first_total = 0;
+        a.maps = nullptr;
         // the chunk totals' region holds a copy of each chunk's Psi
         static_assert(GElem<N>::SIZE >= GAffine<N>::SIZE, "Psi copy fits the element slots");
         RT* psi = a.E;
@@ -585,8 +636,7 @@ struct Launcher {
         k_wseed<R, RT, N><<<count, N, 0, s>>>(a);
         affine_scan(a.FE, a.X, active.data(), levels, s);
         prof_mark(prof, s, "warm_roll");
-        k_croll<R, RT, N, M, NG_ROLL>
-            <<<blocks(C, NG_ROLL), NG_ROLL * N, (size_t)NG_ROLL * ROLL_B, s>>>(a);
+        launch_roll(a, s);
         prof_end(prof, s);
         return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;
     }
@@ -636,6 +686,7 @@ struct Launcher {
                                                2 * up(t * M * sizeof(R)));
                 R* x0p = etaT + up(N * sizeof(R)) / sizeof(R);
                 R* vcorr = x0p + up(N * sizeof(R)) / sizeof(R);
+                if (vector_correction(call)) a.gi = vcorr + up((t + 1) * N * sizeof(R)) / sizeof(R);
                 char* nb = base + roff + kkt_bytes(cp.problem->T);
                 roff += kkt_bytes(cp.problem->T) + (newton ? newton_bytes(cp.problem->T) : 0);
                 set_correction(it2[(size_t)i], a, eta, ctil, etaT, qh, dbuf, x0p);
@@ -651,6 +702,7 @@ struct Launcher {
                 // the Newton correction of (S, v) as an LQT problem (k_nresid)
                 Item<R>& c3 = it3[(size_t)i];
                 c3 = a;
+                c3.gi = nullptr;
                 DescT<R>& D3 = c3.D;
                 D3.p = N;
                 D3.pT = N;
@@ -720,6 +772,7 @@ struct Launcher {
         a.out_mask = 7;
         a.refine_add = 0;
         a.first_total = call.method2 ? 1 : 0;
+        a.maps = vector_correction(call) ? reinterpret_cast<RT*>(base + L.maps) : nullptr;
         if (kPersistFits && call.persistent && !refine && !method2 && !call.sequential) {
             // one cooperative launch for the whole pass (batches)
             const lqt_status st =
@@ -749,6 +802,7 @@ struct Launcher {
                                                                                 a.status);
             Args<R, RT> c = a;
             c.items = d3;
+            c.maps = nullptr;
             c.out_mask = 5;
             pass(c, active.data(), levels, call.sequential, 2, true, s, prof);
             prof_mark(prof, s, "chain_newton_gains");
@@ -779,7 +833,11 @@ struct Launcher {
             // the pass's own v', kept in a workspace buffer
             b.out_mask = method2 ? 4 : 0;
             b.refine_add = 1;
-            pass(b, active.data(), levels, call.sequential, 1, false, s, prof, E2, Pref);
+            b.maps = nullptr;
+            if (vector_correction(call))
+                correct(b, a.maps, active.data(), levels, s, prof);
+            else
+                pass(b, active.data(), levels, call.sequential, 1, false, s, prof, E2, Pref);
         }
         prof_end(prof, s);
         return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;

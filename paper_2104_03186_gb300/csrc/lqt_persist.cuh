@@ -12,8 +12,8 @@
 // the global-memory results.  The per-item work is the same device code as the
 // level kernels' (lqt_team_chain.cuh, lqt_team.cuh).
 //
-// Each team owns a block sized for the largest phase; the terminal values and
-// the rollouts run on the first N lanes of a team (lane-group code).
+// Each team owns a block sized for the largest phase; the terminal values run on
+// the first N lanes of a team (lane-group code), the rollouts one warp a chunk.
 //
 // The barrier is a counter and a generation word in the workspace.  Every
 // wait is bounded: a CTA that waits longer than the limit records
@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include "lqt_chain.cuh"
+#include "lqt_vector_walk.cuh"
 
 namespace lqt {
 namespace chain {
@@ -147,7 +148,7 @@ template <typename R, typename RT, int N, int M>
 constexpr int persist_team_bytes() {
     constexpr int sizes[] = {tstride_of<N, R>(TFoldSmem<N, M>::SIZE) * (int)sizeof(R),
                              tstride_of<N, R>(TRefoldSmem<N, M>::SIZE) * (int)sizeof(R),
-                             gstride<N>(RollSmem<N, M>::SIZE) * (int)sizeof(R),
+                             VWalk<N, M>::FWD_SIZE * (int)sizeof(R) / (N == 8 ? 4 : 1),
                              tstride_of<N, RT>(team::CombineSmem<N>::SIZE) * (int)sizeof(RT),
                              tstride_of<N, RT>(team::ApplySmem<N>::SIZE) * (int)sizeof(RT),
                              (2 * N * N + 2 * N) * (int)sizeof(RT)};
@@ -239,10 +240,22 @@ __global__ void __launch_bounds__(NT* Team<N>::LG) k_cpersist(Args<R, RT> a, Lev
         }
         if (!grid_sync(bar, nb, wait_limit, a.status)) return;
     }
-    // 6. rollouts
-    for (long long c = next_chunk(&bar->next[2], slot, g); c < C;
-         c = next_chunk(&bar->next[2], slot, g))
-        if (lead) b_croll<R, RT, N, M, NT>(a, c, mine, 0);
+    // 6. rollouts, one warp per chunk: the first warp of a team, or (n = 8) every
+    // warp in the blocks of its four teams
+    constexpr int LG = Team<N>::LG, TW = LG < 32 ? 32 / LG : 1;  // teams per warp
+    static_assert(VWalk<N, M>::FWD_SIZE * (int)sizeof(R) <= TW * GB, "a rollout's ring fits");
+    if (g.lane < 32) {
+        const int lane = threadIdx.x & 31;
+        R* ring = reinterpret_cast<R*>(smem_raw + gi / TW * TW * GB);
+        for (;;) {
+            unsigned long long c = 0;
+            if (lane == 0) c = atomicAdd(&bar->next[2], 1ull);
+            c = __shfl_sync(0xffffffffu, c, 0);
+            if ((long long)c >= C) break;
+            b_vfwd<R, RT, N, M, false>(a, (long long)c, nullptr, ring);
+            __syncwarp();
+        }
+    }
     flag(a.status, ok);
 }
 

@@ -286,9 +286,11 @@ __device__ __forceinline__ double rsqrt_(double x) { return 1.0 / sqrt(x); }
 // share of the right sides in registers; the pivot column's entries come from
 // its lane by shuffles, and no sync is needed before the caller's.  FULL: the
 // right sides become G^{-1} B (Gauss-Jordan); otherwise Rc^{-1} B with
-// G = Rc Rc^T (the forward half of a Cholesky solve, half the work).
+// G = Rc Rc^T (the forward half of a Cholesky solve, half the work).  With inv
+// (FULL) G^{-1} replaces G: a pivot's own column takes its inverse column
+// instead of the unit column.
 template <bool FULL, int M, int NR, int N, int RT, typename R>
-__device__ __forceinline__ bool solve_spd(R* t, const Team<N, RT>& g) {
+__device__ __forceinline__ bool solve_spd(R* t, const Team<N, RT>& g, bool inv = false) {
     using T = Team<N, RT>;
     using S = Sys<N, M, NR>;
     constexpr int NRW = (NR + T::NW - 1) / T::NW;
@@ -302,6 +304,7 @@ __device__ __forceinline__ bool solve_spd(R* t, const Team<N, RT>& g) {
 #pragma unroll
         for (int i = 0; i < M; ++i) col[s][i] = in ? t[i * S::LD + c] : R(0);
     }
+    if (FULL && T::NW > 1 && inv) g.sync();  // every warp has read G
     bool ok = true;
 #pragma unroll
     for (int k = 0; k < M; ++k) {
@@ -315,17 +318,19 @@ __device__ __forceinline__ bool solve_spd(R* t, const Team<N, RT>& g) {
             if (i > k || (FULL && i < k)) f[i] = __shfl_sync(g.mask, col[ks][i], kl, T::LW);
 #pragma unroll
         for (int s = 0; s < SL; ++s) {
-            const R pk = col[s][k] * sc, fk = FULL ? pk : pk * sc;
+            const bool own = FULL && s == ks && inv && lw == kl;
+            const R pk = own ? sc : col[s][k] * sc, fk = FULL ? pk : pk * sc;
 #pragma unroll
             for (int i = 0; i < M; ++i)
-                if (i > k || (FULL && i < k)) col[s][i] = fma_(-f[i], fk, col[s][i]);
+                if (i > k || (FULL && i < k))
+                    col[s][i] = fma_(-f[i], fk, own ? R(0) : col[s][i]);
             col[s][k] = pk;
         }
     }
 #pragma unroll
     for (int s = 0; s < SL; ++s) {
-        const int j = s * T::LW + lw, c = j + wi * NRW;
-        if (j >= M && j < COLS && c < M + NR) {
+        const int j = s * T::LW + lw, c = j < M ? j : j + wi * NRW;
+        if ((j >= M || (FULL && inv && wi == 0)) && j < COLS && c < M + NR) {
 #pragma unroll
             for (int i = 0; i < M; ++i) t[i * S::LD + c] = col[s][i];
         }

@@ -533,8 +533,10 @@ __device__ __forceinline__ void b_trefold(const Args<R, RT>& a, long long c, R* 
     const long long e0 = s0 + B < T ? s0 + B : T;
     const TeamWalk<R, N, M, TR> wk(D, g);
     const bool vS = vec_ok(D.S, 0), vK = vec_ok(D.K, 0);
-    // no prefix holds a problem's last chunk: its map is left neutral
-    const bool map = lc + 1 < it.NC;
+    // no prefix holds a problem's last chunk: its map is left neutral, unless the
+    // refinement keeps it (the value scan runs the other way)
+    const bool map = lc + 1 < it.NC || a.maps;
+    R* gi = it.gi;
     if (s0 < e0) wk.stage(D, e0 - 1, sh + S::IN, 0, true, g);
     {
         const RT* val = a.V + c * DValue<N>::SIZE;
@@ -652,7 +654,7 @@ __device__ __forceinline__ void b_trefold(const Args<R, RT>& a, long long c, R* 
         g.sync();
         if (wk.hid) cost_prefetch<N, M>(cost, D, k, wk, g);
         // [K | d] = G^{-1} [W | L^T ev] in place
-        ok &= team::solve_spd<true, M, N + 1>(sy, g);
+        ok &= team::solve_spd<true, M, N + 1>(sy, g, gi != nullptr);
         g.sync();
         // Ft = F - L K, S Ft = S F - SL K, ct = c + L d; K_k and d_k out
         {
@@ -699,6 +701,11 @@ __device__ __forceinline__ void b_trefold(const Args<R, RT>& a, long long c, R* 
                     R y[4];
                     team::ldsys<LD>(sy, row, CK + 4 * ci, y);
                     team::stg_row<N, 4>(D.K + k * M * N, row, 4 * ci, y, vK);
+                }
+                if (gi) {
+                    R y[2];
+                    team::ldsys<LD>(sy, row, 2 * ci, y);
+                    team::stg_row<M, 2>(gi + k * M * M, row, 2 * ci, y, true);
                 }
             }
         }
@@ -757,8 +764,11 @@ __device__ __forceinline__ void b_trefold(const Args<R, RT>& a, long long c, R* 
     }
     g.sync();
     RT* out = a.FE + c * DAffine<N>::SIZE;
-    for (int t = g.lane; t < N * N; t += LG)
-        out[DAffine<N>::OF + t] = static_cast<RT>(Phi[Sw<R, N>::at(t / N, t % N)]);
+    for (int t = g.lane; t < N * N; t += LG) {
+        const RT x = static_cast<RT>(Phi[Sw<R, N>::at(t / N, t % N)]);
+        out[DAffine<N>::OF + t] = x;
+        if (a.maps) a.maps[c * DAffine<N>::SIZE + DAffine<N>::OF + t] = x;
+    }
     for (int i = g.lane; i < N; i += LG) out[DAffine<N>::OC + i] = static_cast<RT>(gm[i]);
     flag(a.status, ok);
 }
