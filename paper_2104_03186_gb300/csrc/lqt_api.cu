@@ -310,6 +310,13 @@ void fill_params(Params<R>& K, const lqt_problem* P, const lqt_solution* sol, vo
     K.dyn_invariant =
         P->F.step_stride == 0 && P->L.step_stride == 0 && P->U.step_stride == 0 ? 1 : 0;
     K.c_invariant = (P->c.ptr == nullptr || P->c.step_stride == 0) ? 1 : 0;
+    const auto vec = [](const lqt_in& in) {
+        return in.ptr && reinterpret_cast<uintptr_t>(in.ptr) % 16 == 0 &&
+               (in.step_stride * (int64_t)sizeof(R)) % 16 == 0;
+    };
+    // (a row of H is N values: 16-byte rows only where N fills them)
+    K.vec = (vec(P->F) ? VEC_F : 0) | (vec(P->L) ? VEC_L : 0) | (vec(P->U) ? VEC_U : 0) |
+            (vec(P->c) ? VEC_C : 0) | (vec(P->H) ? VEC_H : 0);
     K.out_mask = OUT_ALL;
     K.wait_limit = kWaitLimit;
     K.wait_probe = 0;

@@ -46,6 +46,8 @@ enum : int {
 
 enum : int { OUT_S = 1, OUT_V = 2, OUT_K = 4, OUT_ALL = 7 };
 
+enum : int { VEC_F = 1, VEC_L = 2, VEC_U = 4, VEC_C = 8, VEC_H = 16 };
+
 constexpr int kStageG = 2;  // steps per warp-staged group
 
 template <typename R>
@@ -72,6 +74,7 @@ struct Params {
     int cost_invariant;  // H and X time-invariant: H^T X and H^T X H precomputed
     int dyn_invariant;   // F, L, U time-invariant: kept in shared memory
     int c_invariant;     // c time-invariant (or absent): kept in shared memory
+    int vec;             // VEC_*: arrays whose every step starts on 16 bytes
     int out_mask;        // OUT_S | OUT_V | OUT_K: which of S, v, K this pass writes
     int refine_emit;     // first pass of a refined solve: write r', c', r'_T, x'_0
     int refine_add;      // second pass: x <- x + xi instead of x <- xi
@@ -194,43 +197,40 @@ __device__ __forceinline__ void load_row(const R* src, R* vals) {
     }
 }
 
-// Step k of the model: F, c, L, U and the cost element Q = H^T X H, q = H^T X r,
-// from the shared model area where the input is time-invariant.
-template <typename R, int N, int M>
-__device__ __forceinline__ void load_step(const Params<R>& P, long long k, const R* sm,
-                                          const R* r_staged, Step<R, N, M>& st,
-                                          int r_stride = 1) {
-    using ML = ModelLayout<N, M>;
-    if (P.dyn_invariant) {
-        load_row<R, N * N>(sm + ML::OF, &st.F[0][0]);
-        load_row<R, N * M>(sm + ML::OL, &st.L[0][0]);
-        load_row<R, M * M>(sm + ML::OU, &st.U[0][0]);
-    } else {
-        const R* F = P.F + k * P.sF;
-        const R* L = P.L + k * P.sL;
-        const R* U = P.U + k * P.sU;
+// COUNT consecutive values of a per-step input.  Each thread reads its own
+// chunk's steps, so a load instruction touches a line per lane and the L1 tag
+// stage serves one line a cycle: a record is read in as few instructions as its
+// alignment allows (vec: 16-byte loads).  Scalar reads of a time-varying n = 4,
+// p = 3 model took 88 instructions a step, vector reads 25: T = 100003 refined
+// 248 -> 165 us.
+template <typename R, int COUNT>
+__device__ __forceinline__ void ldg_vals(const R* src, bool vec, R* vals) {
+    constexpr int E = 16 / (int)sizeof(R);
+    if (COUNT % E == 0 && vec) {
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-#pragma unroll
-            for (int j = 0; j < N; ++j) st.F[i][j] = __ldg(F + i * N + j);
-#pragma unroll
-            for (int a = 0; a < M; ++a) st.L[i][a] = __ldg(L + i * M + a);
+        for (int i = 0; i < COUNT; i += E) {
+            if constexpr (sizeof(R) == 4) {
+                const float4 t = __ldg(reinterpret_cast<const float4*>(src + i));
+                vals[i] = t.x; vals[i + 1] = t.y; vals[i + 2] = t.z; vals[i + 3] = t.w;
+            } else {
+                const double2 t = __ldg(reinterpret_cast<const double2*>(src + i));
+                vals[i] = t.x; vals[i + 1] = t.y;
+            }
         }
-#pragma unroll
-        for (int a = 0; a < M; ++a)
-#pragma unroll
-            for (int b = 0; b < M; ++b) st.U[a][b] = __ldg(U + a * M + b);
-    }
-    if (P.c_invariant) {
-        load_row<R, N>(sm + ML::OC, st.c);
     } else {
-        const R* c = P.c + k * P.sc;
 #pragma unroll
-        for (int i = 0; i < N; ++i) st.c[i] = __ldg(c + i);
+        for (int i = 0; i < COUNT; ++i) vals[i] = __ldg(src + i);
     }
+}
+
+// The cost element of step k: Q = H^T X H, q = H^T X r.
+template <typename R, int N, int M, bool INV = false>
+__device__ __forceinline__ void load_cost(const Params<R>& P, long long k, const R* sm,
+                                          const R* r_staged, Step<R, N, M>& st, int r_stride) {
+    using ML = ModelLayout<N, M>;
     const int p = P.p;
     const R* r = P.r ? P.r + k * P.sr : nullptr;
-    if (P.cost_invariant) {
+    if (INV || P.cost_invariant) {
         const R* sHX = sm + ML::OHX;
         load_row<R, Dims<N>::SYM>(sm + ML::OQ, st.Q);
 #pragma unroll
@@ -252,6 +252,37 @@ __device__ __forceinline__ void load_step(const Params<R>& P, long long k, const
         for (int k2 = 0; k2 < Dims<N>::SYM; ++k2) st.Q[k2] = R(0);
 #pragma unroll
         for (int i = 0; i < N; ++i) st.q[i] = R(0);
+        if (p <= 4) {  // H's rows read once
+            R h[4][N], rr[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+                if (a < p) {
+                    ldg_vals<R, N>(H + a * N, P.vec & VEC_H, h[a]);
+                    rr[a] = r ? __ldg(r + a) : R(0);
+                }
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+                if (a < p) {
+                    R y[N], xr = R(0);
+#pragma unroll
+                    for (int j = 0; j < N; ++j) y[j] = R(0);
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        if (b < p) {
+                            const R xab = __ldg(X + a * p + b);
+#pragma unroll
+                            for (int j = 0; j < N; ++j) y[j] += xab * h[b][j];
+                            xr += xab * rr[b];
+                        }
+#pragma unroll
+                    for (int i = 0; i < N; ++i) {
+                        st.q[i] += h[a][i] * xr;
+#pragma unroll
+                        for (int j = i; j < N; ++j) st.Q[sym<N>(i, j)] += h[a][i] * y[j];
+                    }
+                }
+            return;
+        }
         for (int a = 0; a < p; ++a) {
             R y[N];
 #pragma unroll
@@ -273,6 +304,33 @@ __device__ __forceinline__ void load_step(const Params<R>& P, long long k, const
                 for (int j = i; j < N; ++j) st.Q[sym<N>(i, j)] += h[i] * y[j];
             }
         }
+    }
+}
+
+// Step k of the model: F, c, L, U and the cost element Q = H^T X H, q = H^T X r,
+// from the shared model area where the input is time-invariant.
+template <typename R, int N, int M, bool INV = false>
+__device__ __forceinline__ void load_step(const Params<R>& P, long long k, const R* sm,
+                                          const R* r_staged, Step<R, N, M>& st,
+                                          int r_stride = 1) {
+    using ML = ModelLayout<N, M>;
+    load_cost<R, N, M, INV>(P, k, sm, r_staged, st, r_stride);  // first: its temporaries die here
+    if (INV || P.dyn_invariant) {
+        load_row<R, N * N>(sm + ML::OF, &st.F[0][0]);
+        load_row<R, N * M>(sm + ML::OL, &st.L[0][0]);
+        load_row<R, M * M>(sm + ML::OU, &st.U[0][0]);
+    } else {
+        const R* F = P.F + k * P.sF;
+        const R* L = P.L + k * P.sL;
+        const R* U = P.U + k * P.sU;
+        ldg_vals<R, N * N>(F, P.vec & VEC_F, &st.F[0][0]);
+        ldg_vals<R, N * M>(L, P.vec & VEC_L, &st.L[0][0]);
+        ldg_vals<R, M * M>(U, P.vec & VEC_U, &st.U[0][0]);
+    }
+    if (P.c_invariant) {
+        load_row<R, N>(sm + ML::OC, st.c);
+    } else {
+        ldg_vals<R, N>(P.c + k * P.sc, P.vec & VEC_C, st.c);
     }
 }
 
@@ -498,11 +556,15 @@ __device__ __forceinline__ bool team_apply_level(R* tree, R* carry, int ts, int 
 // keeps the total of [i + 2^d, i + 2^{d+1}) for the down-sweep).  Only the
 // chunks that hold steps are swept (the rest are neutral).
 // ===========================================================================
+// INV: F, L, U, H and X are time-invariant (the model area holds them), so the
+// per-step loads of a time-varying model, their registers and their code are
+// left out: with both in one kernel the vehicle at T = 1e6 took 345 us, 320
+// without the vector loads, 310 split.
 // The body of each per-tile kernel is a device function over one tile, so
 // that the single-tile solve (k_solo) runs the same code back to back with
 // its trees left in shared memory.  SOLO: the only tile of the problem; the
 // tree is not stored for another kernel.  The model area `sm` is filled.
-template <typename R, int N, int M, int W, bool SOLO>
+template <typename R, int N, int M, int W, bool SOLO, bool INV>
 __device__ __forceinline__ void bwd_up_body(const Params<R>& P, unsigned tile, R* tree,
                                             const R* sm) {
     using SM = Smem<R, N, M, W>;
@@ -517,7 +579,7 @@ __device__ __forceinline__ void bwd_up_body(const Params<R>& P, unsigned tile, R
     bool ok = true;
     for (long long k = e - 1; k >= s; --k) {
         Step<R, N, M> st;
-        load_step<R, N, M>(P, k, sm, nullptr, st);
+        load_step<R, N, M, INV>(P, k, sm, nullptr, st);
         ok &= fold_step<R, N, M>(st, P.has_c != 0, acc);
     }
     store_elem(acc, ElemView<R, N>{tree + tslot<R>(tid), WS});
@@ -543,7 +605,7 @@ __device__ __forceinline__ void bwd_up_body(const Params<R>& P, unsigned tile, R
     if (!ok2) set_status(P.status, ST_SINGULAR);
 }
 
-template <typename R, int N, int M, int W>
+template <typename R, int N, int M, int W, bool INV>
 __global__ void __launch_bounds__(W, 1) k_bwd_up(const Params<R> P) {
     griddep_launch_dependents();
     griddep_wait();
@@ -552,7 +614,7 @@ __global__ void __launch_bounds__(W, 1) k_bwd_up(const Params<R> P) {
     R* tree = reinterpret_cast<R*>(smem_raw + kSmemHead);  // [ELEM][WS]
     R* sm = tree + SM::UP_BIG + SM::RBUF;
     model_prologue<R, N, M>(P, sm);
-    bwd_up_body<R, N, M, W, false>(P, blockIdx.x, tree, sm);
+    bwd_up_body<R, N, M, W, false, INV>(P, blockIdx.x, tree, sm);
 }
 
 // Terminal value S_T = H_T^T X_T H_T, v_T = H_T^T X_T r_T.
@@ -830,7 +892,7 @@ __device__ __forceinline__ void terminal_outputs(const Params<R>& P, const Value
 // W); sm: the model area, filled here unless SOLO (the caller filled it).
 // SOLO: the up-sweep's tree is already in `big`, and the value carried into
 // the tile is the terminal value (Lemma LQT_assoc), formed here.
-template <typename R, int N, int M, int W, bool SOLO>
+template <typename R, int N, int M, int W, bool SOLO, bool INV>
 __device__ __forceinline__ void bwd_down_body(const Params<R>& P, unsigned tile,
                                               unsigned char* smem_raw, R* rbuf, R* sm) {
     using SM = Smem<R, N, M, W>;
@@ -932,7 +994,7 @@ __device__ __forceinline__ void bwd_down_body(const Params<R>& P, unsigned tile,
         for (int jj = cnt - 1; jj >= 0; --jj) {
             const long long k = lo + jj;
             Step<R, N, M> st;
-            load_step<R, N, M>(P, k, sm, staged ? rg + jj * kRStage * W : nullptr, st, W);
+            load_step<R, N, M, INV>(P, k, sm, staged ? rg + jj * kRStage * W : nullptr, st, W);
             R K[M][N], d[M], Ft[N][N], ct[N], Rc[M][M], Rinv[M];
             ok &= riccati_step<R, N, M>(st, P.has_c != 0, val.S, val.v, K, d, Ft, ct, Rc, Rinv);
             // records of step k into this lane's staging row
@@ -1022,14 +1084,14 @@ __device__ __forceinline__ void bwd_down_body(const Params<R>& P, unsigned tile,
     if (!ok_load) set_status(P.status, ST_TIMEOUT);
 }
 
-template <typename R, int N, int M, int W>
+template <typename R, int N, int M, int W, bool INV>
 __global__ void __launch_bounds__(W, 1) k_bwd_down(const Params<R> P) {
     griddep_launch_dependents();
     griddep_wait();
     using SM = Smem<R, N, M, W>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* big = reinterpret_cast<R*>(smem_raw + kSmemHead);
-    bwd_down_body<R, N, M, W, false>(P, blockIdx.x, smem_raw, big + SM::DOWN_BIG + threadIdx.x,
+    bwd_down_body<R, N, M, W, false, INV>(P, blockIdx.x, smem_raw, big + SM::DOWN_BIG + threadIdx.x,
                                      big + SM::DOWN_BIG + SM::RBUF);
 }
 
@@ -1117,7 +1179,7 @@ __global__ void __launch_bounds__(TP, 1) k_fwd_top(const Params<R> P) {
 // fwd_down over one tile; sm: the model area, filled here unless SOLO.
 // SOLO: the forward tree is already in `big` and the tile starts at x_0
 // (Lemma lqt_fwd_init).
-template <typename R, int N, int M, int W, bool SOLO>
+template <typename R, int N, int M, int W, bool SOLO, bool INV>
 __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
                                               unsigned char* smem_raw, R* sm) {
     using SM = Smem<R, N, M, W>;
@@ -1186,13 +1248,14 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
     long long s, e;
     geo.chunk(tid, s, e);
     const long long tbase = geo.chunk0 * P.B;
+    const bool dyn = INV || P.dyn_invariant, cost = INV || P.cost_invariant;
     const int p = P.p;
     const R* sHm = sm + ML::OH(p);
     const int groups = (P.B + kStageG - 1) / kStageG;
     const bool stage_rp = P.refine_emit && p <= kRStage;  // r' kept with 4 floats per step
     // a time-invariant F, L stays in registers for the whole chunk
     R Fr[N][N], Lr[N][M];
-    if (P.dyn_invariant) {
+    if (dyn) {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
 #pragma unroll
@@ -1233,18 +1296,17 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
             R Kk[M * N], d[M];
             load_row<R, M * N>(in + SM::FIK + jj * M * N, Kk);
             load_row<R, M>(in + SM::FID + jj * M, d);
-            if (!P.dyn_invariant) {
+            if (!dyn) {
                 const R* Fg = P.F + k * P.sF;
                 const R* Lg = P.L + k * P.sL;
-#pragma unroll
-                for (int i = 0; i < N; ++i) {
-#pragma unroll
-                    for (int j = 0; j < N; ++j) Fr[i][j] = __ldg(Fg + i * N + j);
-#pragma unroll
-                    for (int a = 0; a < M; ++a) Lr[i][a] = __ldg(Lg + i * M + a);
-                }
+                ldg_vals<R, N * N>(Fg, P.vec & VEC_F, &Fr[0][0]);
+                ldg_vals<R, N * M>(Lg, P.vec & VEC_L, &Lr[0][0]);
             }
-            const R* c = P.has_c ? (P.c_invariant ? sm + ML::OC : P.c + k * P.sc) : nullptr;
+            R c[N];
+            if (!P.c_invariant)
+                ldg_vals<R, N>(P.c + k * P.sc, P.vec & VEC_C, c);
+            else
+                load_row<R, N>(sm + ML::OC, c);  // zeros when there is none
             R uk[M];
 #pragma unroll
             for (int a = 0; a < M; ++a) {
@@ -1256,7 +1318,7 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
             R xn[N];
 #pragma unroll
             for (int i = 0; i < N; ++i) {
-                R t = c ? c[i] : R(0);
+                R t = c[i];
 #pragma unroll
                 for (int j = 0; j < N; ++j) t += Fr[i][j] * x[j];
 #pragma unroll
@@ -1271,12 +1333,17 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
             if (P.refine_emit) {
                 // shifted data of the second pass, each a compensated dot product
                 const R* rk = P.r ? P.r + k * P.sr : nullptr;
-                const R* Hk = P.cost_invariant ? sHm : P.H + k * P.sH;
+                const R* Hk = cost ? sHm : P.H + k * P.sH;
                 R* rrow = myrow + SM::FR + jj * kRStage;
                 for (int a = 0; a < p; ++a) {
+                    R h[N];
+                    if (cost)
+                        load_row<R, N>(Hk + a * N, h);
+                    else
+                        ldg_vals<R, N>(Hk + a * N, P.vec & VEC_H, h);
                     Dot2<R> acc(rk ? rk[a] : R(0));
 #pragma unroll
-                    for (int j = 0; j < N; ++j) acc.add_prod(-Hk[a * N + j], x[j]);
+                    for (int j = 0; j < N; ++j) acc.add_prod(-h[j], x[j]);
                     if (stage_rp)
                         rrow[a] = acc.value();
                     else
@@ -1287,7 +1354,7 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
                 R cpk[N];
 #pragma unroll
                 for (int i = 0; i < N; ++i) {
-                    Dot2<R> acc(c ? c[i] : R(0));
+                    Dot2<R> acc(c[i]);
 #pragma unroll
                     for (int j = 0; j < N; ++j) acc.add_prod(Fr[i][j], x[j]);
                     acc.add(-xn[i]);
@@ -1341,14 +1408,14 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
     if (!ok_load) set_status(P.status, ST_TIMEOUT);
 }
 
-template <typename R, int N, int M, int W>
+template <typename R, int N, int M, int W, bool INV>
 __global__ void __launch_bounds__(W, 1) k_fwd_down(const Params<R> P) {
     griddep_launch_dependents();
     griddep_wait();
     using SM = Smem<R, N, M, W>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* big = reinterpret_cast<R*>(smem_raw + kSmemHead);
-    fwd_down_body<R, N, M, W, false>(P, blockIdx.x, smem_raw, big + SM::FDOWN_BIG + SM::RBUF);
+    fwd_down_body<R, N, M, W, false, INV>(P, blockIdx.x, smem_raw, big + SM::FDOWN_BIG + SM::RBUF);
 }
 
 // ===========================================================================
@@ -1366,7 +1433,7 @@ struct SoloSmem {
     static size_t bytes(int p) { return SM::bytes(BIG, p); }
 };
 
-template <typename R, int N, int M, int W>
+template <typename R, int N, int M, int W, bool INV>
 __global__ void __launch_bounds__(W, 1) k_solo(const Params<R> P) {
     griddep_launch_dependents();
     griddep_wait();
@@ -1376,11 +1443,11 @@ __global__ void __launch_bounds__(W, 1) k_solo(const Params<R> P) {
     R* big = reinterpret_cast<R*>(smem_raw + kSmemHead);
     R* sm = big + BIG + SM::RBUF;
     model_prologue<R, N, M>(P, sm);  // ends with __syncthreads
-    bwd_up_body<R, N, M, W, true>(P, 0, big, sm);
+    bwd_up_body<R, N, M, W, true, INV>(P, 0, big, sm);
     __syncthreads();
-    bwd_down_body<R, N, M, W, true>(P, 0, smem_raw, big + BIG + threadIdx.x, sm);
+    bwd_down_body<R, N, M, W, true, INV>(P, 0, smem_raw, big + BIG + threadIdx.x, sm);
     __syncthreads();
-    fwd_down_body<R, N, M, W, true>(P, 0, smem_raw, sm);
+    fwd_down_body<R, N, M, W, true, INV>(P, 0, smem_raw, sm);
 }
 
 // ===========================================================================

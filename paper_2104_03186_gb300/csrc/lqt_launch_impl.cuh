@@ -49,9 +49,9 @@ static cudaError_t launch_pdl(void (*kernel)(const Params<R>), unsigned grid, un
     return cudaLaunchKernelEx(&cfg, kernel, P);
 }
 
-template <typename R, int N, int M>
-lqt_status launch_solve(const Params<R>& P, const Plan& plan, cudaStream_t stream, Prof* prof,
-                        cudaEvent_t bwd_done) {
+template <typename R, int N, int M, bool INV>
+static lqt_status launch_solve_inv(const Params<R>& P, const Plan& plan, cudaStream_t stream,
+                                   Prof* prof, cudaEvent_t bwd_done) {
     constexpr int W = tile_threads<R, N, M>();
     constexpr int TP = top_threads();
     using SM = Smem<R, N, M, W>;
@@ -60,10 +60,10 @@ lqt_status launch_solve(const Params<R>& P, const Plan& plan, cudaStream_t strea
     if (plan.solo) {
         // one tile: the whole pass in one CTA
         const size_t smem = SoloSmem<R, N, M, W>::bytes(P.p);
-        if (plan.tiles != 1 || allow_smem(k_solo<R, N, M, W>, done_solo, smem) != cudaSuccess)
+        if (plan.tiles != 1 || allow_smem(k_solo<R, N, M, W, INV>, done_solo, smem) != cudaSuccess)
             return plan.tiles != 1 ? LQT_EINVAL : LQT_ECUDA;
         prof_mark(prof, stream, P.refine_add ? "solo.refine" : "solo");
-        if (launch_pdl<R>(k_solo<R, N, M, W>, 1, W, smem, stream, P, true) != cudaSuccess)
+        if (launch_pdl<R>(k_solo<R, N, M, W, INV>, 1, W, smem, stream, P, true) != cudaSuccess)
             return LQT_ECUDA;
         if (bwd_done && cudaEventRecord(bwd_done, stream) != cudaSuccess) return LQT_ECUDA;
         return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;
@@ -82,19 +82,19 @@ lqt_status launch_solve(const Params<R>& P, const Plan& plan, cudaStream_t strea
     const size_t smem_ftop = (size_t)(Dims<N>::AFFINE + N) * tstride(TP, (int)sizeof(R)) * sizeof(R);
     const size_t smem_fdown = SM::bytes(SM::FDOWN_BIG, P.p);
     cudaError_t err;
-    if ((err = allow_smem(k_bwd_up<R, N, M, W>, done_up, smem_up)) != cudaSuccess ||
+    if ((err = allow_smem(k_bwd_up<R, N, M, W, INV>, done_up, smem_up)) != cudaSuccess ||
         (err = allow_smem(k_bwd_top<R, N, TP, 0>, done_top, smem_top_full)) != cudaSuccess ||
         (err = allow_smem(k_bwd_top<R, N, TP, 1>, done_top1, smem_top_full)) != cudaSuccess ||
         (err = allow_smem(k_bwd_top<R, N, TP, 2>, done_top2, smem_top_max)) != cudaSuccess ||
-        (err = allow_smem(k_bwd_down<R, N, M, W>, done_down, smem_down)) != cudaSuccess ||
+        (err = allow_smem(k_bwd_down<R, N, M, W, INV>, done_down, smem_down)) != cudaSuccess ||
         (err = allow_smem(k_fwd_top<R, N, TP>, done_ftop, smem_ftop)) != cudaSuccess ||
-        (err = allow_smem(k_fwd_down<R, N, M, W>, done_fdown, smem_fdown)) != cudaSuccess)
+        (err = allow_smem(k_fwd_down<R, N, M, W, INV>, done_fdown, smem_fdown)) != cudaSuccess)
         return LQT_ECUDA;
     const int tiles = plan.tiles;
     const bool pdl = plan.B <= kPdlMaxChunk;
     if (tiles > 0) {
         prof_mark(prof, stream, P.refine_add ? "bwd_up.refine" : "bwd_up");
-        err = launch_pdl<R>(k_bwd_up<R, N, M, W>, tiles, W, smem_up, stream, P, pdl);
+        err = launch_pdl<R>(k_bwd_up<R, N, M, W, INV>, tiles, W, smem_up, stream, P, pdl);
         if (err != cudaSuccess) return LQT_ECUDA;
     }
     prof_mark(prof, stream, P.refine_add ? "bwd_top.refine" : "bwd_top");
@@ -105,7 +105,7 @@ lqt_status launch_solve(const Params<R>& P, const Plan& plan, cudaStream_t strea
     if (err != cudaSuccess) return LQT_ECUDA;
     if (tiles > 0) {
         prof_mark(prof, stream, P.refine_add ? "bwd_down.refine" : "bwd_down");
-        err = launch_pdl<R>(k_bwd_down<R, N, M, W>, tiles, W, smem_down, stream, P, pdl);
+        err = launch_pdl<R>(k_bwd_down<R, N, M, W, INV>, tiles, W, smem_down, stream, P, pdl);
         if (err != cudaSuccess) return LQT_ECUDA;
     }
     // S, v and K are final here (a second refinement pass does not write them)
@@ -115,10 +115,19 @@ lqt_status launch_solve(const Params<R>& P, const Plan& plan, cudaStream_t strea
     if (err != cudaSuccess) return LQT_ECUDA;
     if (tiles > 0) {
         prof_mark(prof, stream, P.refine_add ? "fwd_down.refine" : "fwd_down");
-        err = launch_pdl<R>(k_fwd_down<R, N, M, W>, tiles, W, smem_fdown, stream, P, pdl);
+        err = launch_pdl<R>(k_fwd_down<R, N, M, W, INV>, tiles, W, smem_fdown, stream, P, pdl);
         if (err != cudaSuccess) return LQT_ECUDA;
     }
     return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;
+}
+
+template <typename R, int N, int M>
+lqt_status launch_solve(const Params<R>& P, const Plan& plan, cudaStream_t stream, Prof* prof,
+                        cudaEvent_t bwd_done) {
+    // the time-invariant model's kernels, or those that load it step by step
+    return P.dyn_invariant && P.cost_invariant
+               ? launch_solve_inv<R, N, M, true>(P, plan, stream, prof, bwd_done)
+               : launch_solve_inv<R, N, M, false>(P, plan, stream, prof, bwd_done);
 }
 
 template <typename R, int N, int M>
