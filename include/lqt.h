@@ -274,13 +274,10 @@ lqt_status lqt_solve_batched(const lqt_batch_item *items, int32_t count, void *w
  * resident group; `persistent` selects the launch mode: one launch per tree
  * level (LQT_BATCH_PER_LEVEL), one cooperative launch per state size that
  * runs every tree level with grid barriers (LQT_BATCH_PERSISTENT), or
- * (LQT_BATCH_AUTO, the default) the cooperative launch when its grid (one lane
- * group per chunk) needs at most half of the CTAs the device holds at once,
- * per-level launches otherwise.  The persistent launch saves the launch gaps
- * that dominate small batches; a larger cooperative launch waits until its
- * whole grid is resident, which serialises it with the work of other
- * streams, and with many waves of chunks the per-level kernels, whose blocks
- * are sized per phase, keep more groups busy.  count = 0
+ * (LQT_BATCH_AUTO, the default) the library's choice, the per-level launches: a
+ * launch covers several tree levels and the sizes of a batch run side by side,
+ * which the cooperative launches, each waiting for its whole grid, hold up.
+ * count = 0
  * clears the table.  The settings are process-wide; calls already launched
  * are not affected.  Returns LQT_EINVAL for more than 64 entries, a
  * non-positive n or chunk length, or another launch mode.  The Python binding

@@ -12,6 +12,7 @@
 #include "lqt.h"
 #include "lqt_batch_launch.cuh"
 #include "lqt_chain_api.h"
+#include "lqt_fork.h"
 #include "lqt_upload.cuh"
 
 namespace lqt {
@@ -128,45 +129,13 @@ static size_t head_bytes(int32_t count) {
     return up(256) + up(64 * sizeof(int)) + up((size_t)count * sizeof(BatchDesc));
 }
 
-// The lane sizes of a batch with at least kForkSteps steps run side by side,
-// each on an auxiliary stream forked from the caller's stream after the
-// workspace head is cleared and joined back to it (events; a CUDA graph
-// captures them as parallel branches), beside the n = 4 launch on the caller's
+// The lane sizes of a batch run side by side, each on an auxiliary stream
+// (lqt_fork.h) forked from the caller's stream after the workspace head is
+// cleared and joined back to it, beside the n = 4 launch on the caller's
 // stream: the sizes are independent, and one size's tree levels and last wave
-// leave most SMs idle.  Smaller batches (a server's) keep the caller's stream:
-// the auxiliary streams belong to the host thread, so a thread's small batches
-// on several streams would otherwise queue on them.
-constexpr long long kForkSteps = 1LL << 20;
-constexpr int kMaxAux = 4;
-
-struct BatchAux {
-    cudaStream_t s[kMaxAux] = {};
-    cudaEvent_t fork = nullptr, join[kMaxAux] = {};
-    bool ready = false;
-};
-
-// This host thread's auxiliary streams and events on the current device,
-// created on its first large batch there and kept until the process exits;
-// nullptr if they cannot be created (the batch then runs on one stream).
-static BatchAux* batch_aux() {
-    thread_local BatchAux aux[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    BatchAux& a = aux[dev];
-    if (!a.ready) {
-        // handles made by an earlier, failed attempt are kept and not made again
-        if (!a.fork && cudaEventCreateWithFlags(&a.fork, cudaEventDisableTiming) != cudaSuccess)
-            return nullptr;
-        for (int i = 0; i < kMaxAux; ++i)
-            if ((!a.s[i] && cudaStreamCreateWithFlags(&a.s[i], cudaStreamNonBlocking) !=
-                                cudaSuccess) ||
-                (!a.join[i] &&
-                 cudaEventCreateWithFlags(&a.join[i], cudaEventDisableTiming) != cudaSuccess))
-                return nullptr;
-        a.ready = true;
-    }
-    return &a;
-}
+// leave most SMs idle.  Batches of fewer steps than this stay on one stream:
+// the fork and joins cost about what they save.
+constexpr long long kForkSteps = 1024;
 
 // Workspace bytes of each lane group (its own region, so that the groups may
 // run at once); false if a group is invalid.
@@ -227,10 +196,10 @@ extern "C" lqt_status lqt_solve_batched(const lqt_batch_item* items, int32_t cou
     long long total_steps = 0;
     for (int i = 0; i < count; ++i) total_steps += items[i].problem.T;
     const int lanes_running = (int)groups.size();
-    BatchAux* aux = nullptr;
-    if (lanes_running >= 1 && lanes_running <= kMaxAux &&
+    ForkSet* aux = nullptr;
+    if (lanes_running >= 1 && lanes_running <= kForkStreams &&
         lanes_running + (descs.empty() ? 0 : 1) >= 2 && total_steps >= kForkSteps)
-        aux = batch_aux();
+        aux = next_fork_set();
     if (aux && cudaEventRecord(aux->fork, s) != cudaSuccess) return LQT_ECUDA;
     if (!descs.empty()) {
         // through kernel parameters (lqt_upload.cuh): a pageable copy would

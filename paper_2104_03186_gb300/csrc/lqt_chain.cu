@@ -17,18 +17,14 @@ namespace {
 // smallest chunk the planner makes, in steps
 constexpr long long kMinChunk = 4;
 
-// Batches of the lane sizes: one launch per tree level, one persistent
-// launch, or (the default) the persistent launch where its grid needs at most
-// half of the CTAs the device holds at once, per-level launches otherwise
-// (lqt_batch_set_tuning).  Measured on one GB300 (time-varying random
-// problems, p = n, chunk lengths as planned): the persistent launch took
-// 5-20% off single problems and batches of 16 at n = 8, 16, 32 and
-// T = 128..2048, and lost where its chunks were many waves of the device's
-// groups (n = 32, 16 problems of T = 2048 in 4-step chunks: 7.5 against
-// 6.1 ms; the 4096-problem benchmark batch: 47.3 against 45.8 ms).  A server
-// running batches on several streams at once lost twice its latency at
-// 20 000 requests/s when every batch took a cooperative launch: a launch whose
-// grid covers the device waits for the other streams' kernels to leave.
+// Batches of the lane sizes: launches per run of tree levels, one persistent
+// launch, or (the default) the per-level launches everywhere
+// (lqt_batch_set_tuning).  Measured on one GB300 with the sizes side by side,
+// per-level against persistent against the persistent launch only for grids of
+// at most half the device: 8 mixed requests 335 / 345 / 345 us, 48 658 / 1142 /
+// 696, 200 1.53 / 2.56 / 1.63 ms, 512 problems of T <= 1024 1.01 / 1.48 / 1.01,
+// the 4096-problem batch 19.8 / 21.5 / 19.8 ms.  A cooperative launch waits
+// until its whole grid is resident, so it holds up the other sizes.
 std::atomic<int> g_batch_mode{LQT_BATCH_AUTO};
 
 // Tuned chunk lengths of batches (lqt_batch_set_tuning): entry e applies to
@@ -228,9 +224,7 @@ lqt_status chain_batch_solve(const lqt_batch_item* items, const int* idx, int co
     const lqt_status st = batch_geometry(*v, items, idx, count, &probs);
     if (st != LQT_OK) return st;
     ChainCall call{probs.data(), count, false, false, false, false, ws, ws_bytes, status};
-    const int mode = g_batch_mode.load();
-    call.persistent = mode != LQT_BATCH_PER_LEVEL;
-    call.persistent_if_small = mode == LQT_BATCH_AUTO;
+    call.persistent = g_batch_mode.load() == LQT_BATCH_PERSISTENT;
     return v->run(call, s, nullptr);
 }
 

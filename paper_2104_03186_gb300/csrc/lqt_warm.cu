@@ -1,8 +1,9 @@
 // C ABI of the warm solve (include/lqt.h: lqt_solve_warm): problems whose S_k
 // and K_k are known (a receding horizon over an earlier solve's model), solved
 // for v, x* and u* by the vector scans of lqt_warm.cuh.  Problems are grouped
-// by (dtype, n, m); each group is one chain call, the groups run one after
-// another on the stream.
+// by (dtype, n, m); each group is one chain call with its own part of the
+// workspace, and the groups run side by side: the first on the caller's stream,
+// the others on auxiliary streams forked from it and joined back (lqt_fork.h).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -12,6 +13,7 @@
 
 #include "lqt.h"
 #include "lqt_chain_api.h"
+#include "lqt_fork.h"
 
 namespace lqt {
 namespace {
@@ -78,13 +80,13 @@ extern "C" size_t lqt_warm_workspace_bytes(const lqt_batch_item* items, int32_t 
     if (count < 0 || (count > 0 && !items)) return 0;
     for (int i = 0; i < count; ++i)
         if (check_warm_item(items[i]) != LQT_OK) return 0;
-    size_t most = 0;
+    size_t sum = 0;
     for (const std::vector<int>& g : warm_groups(items, count)) {
         size_t b = 0;
         if (chain_warm_workspace(items, g.data(), (int)g.size(), &b) != LQT_OK) return 0;
-        most = std::max(most, b);
+        sum += up(b);
     }
-    return up(256) + up(most);
+    return up(256) + sum;
 }
 
 extern "C" lqt_status lqt_solve_warm(const lqt_batch_item* items, int32_t count, void* workspace,
@@ -102,11 +104,36 @@ extern "C" lqt_status lqt_solve_warm(const lqt_batch_item* items, int32_t count,
     int* status = reinterpret_cast<int*>(base);
     if (cudaMemsetAsync(base, 0, sizeof(int), s) != cudaSuccess) return LQT_ECUDA;
     char* ws = base + up(256);
-    const size_t ws_bytes = workspace_bytes - up(256);
-    for (const std::vector<int>& g : warm_groups(items, count)) {
-        const lqt_status st = chain_warm_solve(items, g.data(), (int)g.size(), ws, ws_bytes,
-                                               status, s);
-        if (st != LQT_OK) return st;
+    const std::vector<std::vector<int>> groups = warm_groups(items, count);
+    ForkSet* aux = groups.size() > 1 ? next_fork_set() : nullptr;
+    if (aux && cudaEventRecord(aux->fork, s) != cudaSuccess) return LQT_ECUDA;
+    // the auxiliary streams in use rejoin the caller's stream on every return
+    // (their work uses the workspace, and a capture must end joined)
+    int forked = 0;
+    auto rejoin = [&](lqt_status st) {
+        for (int i = 0; i < forked; ++i)
+            if (cudaEventRecord(aux->join[i], aux->s[i]) != cudaSuccess ||
+                cudaStreamWaitEvent(s, aux->join[i], 0) != cudaSuccess)
+                st = st == LQT_OK ? LQT_ECUDA : st;
+        return st;
+    };
+    for (size_t i = 0; i < groups.size(); ++i) {
+        const std::vector<int>& g = groups[i];
+        size_t bytes = 0;
+        lqt_status st = chain_warm_workspace(items, g.data(), (int)g.size(), &bytes);
+        if (st != LQT_OK) return rejoin(st);
+        cudaStream_t gs = s;
+        if (aux && i > 0) {  // group i on set stream (i - 1) mod kForkStreams
+            const int q = (int)((i - 1) % kForkStreams);
+            gs = aux->s[q];
+            if (q >= forked) {
+                if (cudaStreamWaitEvent(gs, aux->fork, 0) != cudaSuccess) return rejoin(LQT_ECUDA);
+                forked = q + 1;
+            }
+        }
+        st = chain_warm_solve(items, g.data(), (int)g.size(), ws, up(bytes), status, gs);
+        if (st != LQT_OK) return rejoin(st);
+        ws += up(bytes);
     }
-    return LQT_OK;
+    return rejoin(LQT_OK);
 }
