@@ -198,20 +198,10 @@ int refine_r_stride(int p) { return p <= kRStage ? kRStage : p; }
 
 struct Layout {
     size_t tree, tile_agg, tile_carry, ftree, ftile_agg, ftile_x;
-    // refinement: maps recorded by the first pass's top-level scan (0: none)
-    size_t top_fac;
     // refinement: shifted references and offsets, zero initial state
     size_t rp, rTp, cp, x0p;
     size_t total;
 };
-
-// The second pass of a refined solve replays the first pass's top-level
-// backward scan from recorded maps when every top-scan thread holds one tile
-// and the staged maps fit the CTA's shared memory.
-bool top_replay(const Variant& var, const Plan& plan, size_t es) {
-    return plan.tiles > 0 && plan.tiles <= var.TP &&
-           top_smem_bytes(var.elem, var.value, var.n, var.TP, (int)es, true) <= kTopSmemMax;
-}
 
 Layout layout(const Variant& var, const Plan& plan, size_t es, const lqt_problem* P,
               bool refine) {
@@ -231,11 +221,6 @@ Layout layout(const Variant& var, const Plan& plan, size_t es, const lqt_problem
     L.ftile_x = off;
     off += align_up(t * var.n * es);
     L.rp = L.rTp = L.cp = L.x0p = 0;
-    L.top_fac = 0;
-    if (refine && top_replay(var, plan, es)) {
-        L.top_fac = off;
-        off += align_up((size_t)top_fac_elems(var.n, var.TP) * es);
-    }
     if (refine) {
         const size_t T = (size_t)P->T, n = (size_t)P->n;
         L.rp = off;
@@ -292,7 +277,6 @@ void fill_params(Params<R>& K, const lqt_problem* P, const lqt_solution* sol, vo
         K.ftree = reinterpret_cast<R*>(base + L->ftree);
         K.ftile_agg = reinterpret_cast<R*>(base + L->ftile_agg);
         K.ftile_x = reinterpret_cast<R*>(base + L->ftile_x);
-        if (L->top_fac) K.top_fac = reinterpret_cast<R*>(base + L->top_fac);
         if (L->rp | L->rTp | L->cp | L->x0p) {
             K.rp = reinterpret_cast<R*>(base + L->rp);
             K.rTp = reinterpret_cast<R*>(base + L->rTp);
@@ -316,7 +300,15 @@ void fill_params(Params<R>& K, const lqt_problem* P, const lqt_solution* sol, vo
     };
     // (a row of H is N values: 16-byte rows only where N fills them)
     K.vec = (vec(P->F) ? VEC_F : 0) | (vec(P->L) ? VEC_L : 0) | (vec(P->U) ? VEC_U : 0) |
-            (vec(P->c) ? VEC_C : 0) | (vec(P->H) ? VEC_H : 0);
+            (vec(P->c) ? VEC_C : 0) | (vec(P->H) ? VEC_H : 0) | (vec(P->r) ? VEC_R : 0);
+    const auto vec_out = [](const void* p, int64_t per_step) {
+        return p && reinterpret_cast<uintptr_t>(p) % 16 == 0 &&
+               (per_step * (int64_t)sizeof(R)) % 16 == 0;
+    };
+    const int64_t n = P->n, m = P->m;
+    K.vec |= vec_out(sol->S, n * n) ? VEC_S : 0;
+    // (d_k is stored beside K_k's reads: u 8-byte aligned as well)
+    K.vec |= vec_out(sol->K, m * n) && reinterpret_cast<uintptr_t>(sol->u) % 8 == 0 ? VEC_K : 0;
     K.out_mask = OUT_ALL;
     K.wait_limit = kWaitLimit;
     K.wait_probe = 0;
@@ -385,7 +377,7 @@ lqt_status lqt_plan(const lqt_problem* prob, const lqt_options* opts, int32_t* c
     if (chain) {
         int NC = 0, nk = 0;
         long long B = 0;
-        if ((st = chain_workspace(prob, refine, newton, false, method2, nullptr, &NC, &B, &nk)) !=
+        if ((st = chain_workspace(prob, refine, newton, false, method2, false, nullptr, &NC, &B, &nk)) !=
             LQT_OK)
             return st;
         if (B > INT32_MAX) return LQT_EINVAL;
@@ -406,6 +398,14 @@ lqt_status lqt_plan(const lqt_problem* prob, const lqt_options* opts, int32_t* c
 }
 
 size_t lqt_workspace_bytes(const lqt_problem* prob, const lqt_options* opts) {
+    return lqt::workspace_bytes(prob, opts, false);
+}
+
+}  // extern "C"
+
+namespace lqt {
+
+size_t workspace_bytes(const lqt_problem* prob, const lqt_options* opts, bool lean) {
     if (validate(prob, nullptr) != LQT_OK) return 0;
     bool refine = false, newton = false, method2 = false;
     if (resolve_refine(prob, opts, &refine, &newton, &method2) != LQT_OK) return 0;
@@ -415,7 +415,7 @@ size_t lqt_workspace_bytes(const lqt_problem* prob, const lqt_options* opts) {
     if (unsupported) return 0;
     if (chain) {
         size_t bytes = 0;
-        if (chain_workspace(prob, refine, newton, false, method2, &bytes, nullptr, nullptr,
+        if (chain_workspace(prob, refine, newton, false, method2, lean, &bytes, nullptr, nullptr,
                             nullptr) != LQT_OK)
             return 0;
         return bytes;
@@ -425,9 +425,6 @@ size_t lqt_workspace_bytes(const lqt_problem* prob, const lqt_options* opts) {
     return layout(*var, plan, elem_bytes(prob->dtype), prob, refine).total;
 }
 
-}  // extern "C"
-
-namespace lqt {
 namespace {
 
 // One pass of the parallel solve or of the sequential baseline.
@@ -442,9 +439,10 @@ lqt_status run_pass(const Variant& var, const lqt_problem* P, const lqt_solution
     K.out_mask = out_mask;
     K.refine_emit = refine_emit;
     K.refine_add = refine_add;
-    // the first pass of a refined solve records the top scan's maps, the
-    // second (same matrices) replays them
-    K.top_mode = K.top_fac ? (refine_add ? 2 : (refine_emit ? 1 : 0)) : 0;
+    // the second pass of a refined solve scans vectors through the first pass's
+    // chunk maps
+    K.keep_maps = refine_emit && !sequential;
+    K.vector_pass = refine_add && !sequential;
     if (sequential) {
         if (prof) prof_mark(prof, s, refine_add ? "riccati_seq.refine" : "riccati_seq");
         return var.seq(&K, s);
@@ -466,9 +464,8 @@ lqt_status run_solve(const Variant& var, const lqt_problem* P, const lqt_solutio
     }
     // pass 2: the problem shifted by the first trajectory, x = x^ + xi, with
     // the same matrices, small references and offsets, and x'_0 = 0.  Its S
-    // and K equal those of pass 1 bit for bit (they do not depend on r or c):
-    // the pass does not write S, v, K again, reads K back, writes u* and adds
-    // xi into x.
+    // and K are those of pass 1 (they do not depend on r or c): the pass scans
+    // vectors alone, reads S and K back, writes u* and adds xi into x.
     char* base = static_cast<char*>(ws);
     lqt_problem P2 = *P;
     P2.r.ptr = P->p > 0 ? base + L.rp : nullptr;
@@ -486,7 +483,8 @@ lqt_status run_solve(const Variant& var, const lqt_problem* P, const lqt_solutio
 // where the path can tell (the thread-per-chunk kernels); *recorded says so.
 lqt_status solve_common(const lqt_problem* prob, const lqt_solution* sol, const lqt_options* opts,
                         void* workspace, size_t workspace_bytes, void* stream, bool sequential,
-                        cudaEvent_t bwd_done = nullptr, bool* recorded = nullptr) {
+                        cudaEvent_t bwd_done = nullptr, bool* recorded = nullptr,
+                        bool lean = false) {
     if (recorded) *recorded = false;
     lqt_status st = validate(prob, sol);
     if (st != LQT_OK) return st;
@@ -504,7 +502,7 @@ lqt_status solve_common(const lqt_problem* prob, const lqt_solution* sol, const 
     if (chain) {
         // the chunked pipeline (one chunk when sequential)
         size_t need = 0;
-        if ((st = chain_workspace(prob, refine, newton, sequential, method2, &need, nullptr,
+        if ((st = chain_workspace(prob, refine, newton, sequential, method2, lean, &need, nullptr,
                                   nullptr, nullptr)) != LQT_OK)
             return st;
         if (workspace_bytes < need) return LQT_ENOMEM;
@@ -512,7 +510,7 @@ lqt_status solve_common(const lqt_problem* prob, const lqt_solution* sol, const 
         if (cudaMemsetAsync(workspace, 0, sizeof(int), s) != cudaSuccess) return LQT_ECUDA;
         Prof* prof = nullptr;
         if ((st = prof_begin(&prof)) != LQT_OK) return st;
-        return chain_solve(prob, sol, refine, newton, sequential, method2, workspace,
+        return chain_solve(prob, sol, refine, newton, sequential, method2, lean, workspace,
                            workspace_bytes, s, prof);
     }
     Plan plan;
@@ -532,6 +530,16 @@ lqt_status solve_common(const lqt_problem* prob, const lqt_solution* sol, const 
 }
 
 }  // namespace
+}  // namespace lqt
+
+namespace lqt {
+
+lqt_status solve_lean(const lqt_problem* prob, const lqt_solution* sol, const lqt_options* opts,
+                      void* workspace, size_t workspace_bytes, void* stream) {
+    return solve_common(prob, sol, opts, workspace, workspace_bytes, stream, false, nullptr,
+                        nullptr, true);
+}
+
 }  // namespace lqt
 
 extern "C" {

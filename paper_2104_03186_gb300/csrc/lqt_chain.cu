@@ -95,12 +95,6 @@ lqt_status geometry(const ChainVariant& v, const lqt_problem* P, bool sequential
     return LQT_OK;
 }
 
-int levels(int NC) {
-    int l = 0;
-    while ((1 << l) < NC) ++l;
-    return l;
-}
-
 // Chunk geometry of a batch of one variant: a chunk length B* from the
 // total work over the resident fold groups, clamped to [kMinChunk,
 // kMaxBatchChunk] so that no problem's latency grows with the batch, or the
@@ -154,7 +148,8 @@ bool chain_small_supported(int dtype, int n, int m) {
 }
 
 lqt_status chain_workspace(const lqt_problem* P, bool refine, bool newton, bool sequential,
-                           bool method2, size_t* bytes, int* NC, long long* B, int* kernels) {
+                           bool method2, bool lean, size_t* bytes, int* NC, long long* B,
+                           int* kernels) {
     if (P->p > 2 * P->n || P->pT > 2 * P->n) return LQT_EUNSUPPORTED;
     // FP64 tree levels with the FULL refinement (the Newton step); FP32 otherwise
     const bool mixed = refine && newton && P->dtype == LQT_F32;
@@ -166,26 +161,17 @@ lqt_status chain_workspace(const lqt_problem* P, bool refine, bool newton, bool 
     if (st != LQT_OK) return st;
     ChainProblem cp{P, nullptr, nc, b};
     const bool rf = refine && P->T > 0;
-    if (bytes) *bytes = v->workspace(&cp, 1, rf, rf && newton, method2);
+    const bool vector = rf && !method2 && !sequential && !lean;
+    if (bytes) *bytes = v->workspace(&cp, 1, rf, rf && newton, method2, vector);
     if (NC) *NC = nc;
     if (B) *B = b;
-    if (kernels) {
-        const int l = levels(nc);
-        // Method 2: the element copy, 2 l sweep levels, the seeds, the walk
-        const int fwd = method2 ? 2 * l + 2 : (sequential ? 0 : 2 * l);
-        const int per_pass = (sequential ? 2 : 3 + 2 * l) + fwd + (method2 ? 0 : 1);
-        const int bwd = sequential ? 2 : 3 + 2 * l;
-        int k = 1 + per_pass;  // the item upload, the solve
-        if (rf) k += 1 + 1 + per_pass;  // item upload, KKT residuals, correction solve
-        if (rf && newton) k += 2 + bwd + 2;  // constants, residuals, dS/dv scan, gains, add
-        *kernels = k;
-    }
+    if (kernels) *kernels = v->kernels(nc, rf, rf && newton, sequential, method2, vector);
     return LQT_OK;
 }
 
 lqt_status chain_solve(const lqt_problem* P, const lqt_solution* sol, bool refine, bool newton,
-                       bool sequential, bool method2, void* ws, size_t ws_bytes, cudaStream_t s,
-                       Prof* prof) {
+                       bool sequential, bool method2, bool lean, void* ws, size_t ws_bytes,
+                       cudaStream_t s, Prof* prof) {
     if (P->p > 2 * P->n || P->pT > 2 * P->n) return LQT_EUNSUPPORTED;
     const bool mixed = refine && newton && P->dtype == LQT_F32;
     const ChainVariant* v = find_chain(P->dtype, P->n, P->m, mixed);
@@ -197,6 +183,7 @@ lqt_status chain_solve(const lqt_problem* P, const lqt_solution* sol, bool refin
     ChainProblem cp{P, sol, NC, B};
     const bool rf = refine && P->T > 0;
     ChainCall call{&cp, 1, rf, rf && newton, sequential, method2, ws, ws_bytes, nullptr};
+    call.vector = rf && !method2 && !sequential && !lean;
     return v->run(call, s, prof);
 }
 
@@ -210,7 +197,7 @@ lqt_status chain_batch_workspace(const lqt_batch_item* items, const int* idx, in
     std::vector<ChainProblem> probs;
     const lqt_status st = batch_geometry(*v, items, idx, count, &probs);
     if (st != LQT_OK) return st;
-    *bytes = v->workspace(probs.data(), count, false, false, false);
+    *bytes = v->workspace(probs.data(), count, false, false, false, false);
     return LQT_OK;
 }
 
@@ -262,7 +249,7 @@ lqt_status chain_warm_workspace(const lqt_batch_item* items, const int* idx, int
     std::vector<ChainProblem> probs;
     const lqt_status st = warm_geometry(*v, items, idx, count, &probs);
     if (st != LQT_OK) return st;
-    *bytes = v->workspace(probs.data(), count, false, false, false);
+    *bytes = v->workspace(probs.data(), count, false, false, false, false);
     return LQT_OK;
 }
 

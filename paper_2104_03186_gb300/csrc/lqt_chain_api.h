@@ -36,18 +36,22 @@ struct ChainCall {
     // one persistent cooperative launch instead of one launch per tree level
     // (no refinement, Method 1 only)
     bool persistent = false;
+    // the refinement's correction pass by vector walks (lqt_vector_walk.cuh)
+    bool vector = false;
 };
 
 struct ChainVariant {
     int dtype, n, m;
     int mixed;         // FP32 chunk work with FP64 tree levels
     size_t (*workspace)(const ChainProblem* probs, int count, bool refine, bool newton,
-                        bool method2);
+                        bool method2, bool vector);
     lqt_status (*run)(const ChainCall& call, cudaStream_t s, Prof* prof);
     const void* (*fold_kernel)();
     size_t (*fold_smem)();
     int (*fold_groups)();   // teams or lane groups per CTA
     int (*fold_threads)();  // threads per CTA
+    // kernel launches of one problem of nc chunks
+    int (*kernels)(int nc, bool refine, bool newton, bool sequential, bool method2, bool vector);
 };
 
 // Variants compiled in lqt_chain_n4.cu, lqt_chain_n8.cu, lqt_chain_n16.cu and
@@ -100,12 +104,14 @@ bool chain_supported(int dtype, int n, int m);
 // n <= 4 sizes with a compiled chain variant: used for Method 2 and the FULL
 // refinement, which the thread-per-step kernels do not provide.
 bool chain_small_supported(int dtype, int n, int m);
-// Single problem: workspace bytes, chunk geometry and kernel launches.
+// Single problem: workspace bytes, chunk geometry and kernel launches.  lean: the
+// least workspace, without what the vector form of the correction pass keeps.
 lqt_status chain_workspace(const lqt_problem* P, bool refine, bool newton, bool sequential,
-                           bool method2, size_t* bytes, int* NC, long long* B, int* kernels);
+                           bool method2, bool lean, size_t* bytes, int* NC, long long* B,
+                           int* kernels);
 lqt_status chain_solve(const lqt_problem* P, const lqt_solution* sol, bool refine, bool newton,
-                       bool sequential, bool method2, void* ws, size_t ws_bytes, cudaStream_t s,
-                       Prof* prof);
+                       bool sequential, bool method2, bool lean, void* ws, size_t ws_bytes,
+                       cudaStream_t s, Prof* prof);
 // Batch of problems of one FP32 (n, m), no refinement: items[idx[0..count)].
 lqt_status chain_batch_workspace(const lqt_batch_item* items, const int* idx, int count,
                                  size_t* bytes);
@@ -117,5 +123,11 @@ lqt_status chain_warm_workspace(const lqt_batch_item* items, const int* idx, int
                                 size_t* bytes);
 lqt_status chain_warm_solve(const lqt_batch_item* items, const int* idx, int count, void* ws,
                             size_t ws_bytes, int* status, cudaStream_t s);
+
+// lqt_workspace_bytes, and with lean the least that solve_lean takes (lqt_api.cu).
+size_t workspace_bytes(const lqt_problem* prob, const lqt_options* opts, bool lean);
+// lqt_solve in the least workspace.
+lqt_status solve_lean(const lqt_problem* prob, const lqt_solution* sol, const lqt_options* opts,
+                      void* workspace, size_t workspace_bytes, void* stream);
 
 }  // namespace lqt

@@ -262,7 +262,7 @@ struct Launcher {
     static size_t up(size_t x) { return (x + 255) / 256 * 256; }
 
     static Layout layout(const ChainProblem* probs, int count, bool refine, bool newton,
-                         bool method2 = false) {
+                         bool method2, bool vector) {
         Layout L;
         long long C = 0;
         for (int i = 0; i < count; ++i) C += probs[i].NC;
@@ -289,7 +289,7 @@ struct Launcher {
         L.X = off;
         off += up(nc * N * sizeof(RT));
         L.maps = off;  // the first pass's chunk maps, for the correction pass
-        if (refine && kTeam) off += up(nc * GAffine<N>::SIZE * sizeof(RT));
+        if (vector) off += up(nc * GAffine<N>::SIZE * sizeof(RT));
         L.E2 = L.Pref = 0;
         if (method2) {  // Method 2: a copy of the chunk totals and the prefixes
             L.E2 = off;
@@ -300,7 +300,7 @@ struct Launcher {
         L.refine0 = off;
         if (refine)
             for (int i = 0; i < count; ++i)
-                off += kkt_bytes(probs[i].problem->T) +
+                off += kkt_bytes(probs[i].problem->T, vector) +
                        (newton ? newton_bytes(probs[i].problem->T) : 0);
         L.total = off;
         return L;
@@ -309,11 +309,11 @@ struct Launcher {
     // per problem, KKT correction: eta T x N, c~ T x N, U^{-1} h T x M,
     // feedforward T x M, eta_T N, x'_0 N; Newton correction: Phi T x N x N,
     // ct T x N, R (T + 1) x N x N, rho (T + 1) x N, dS (T + 1) x N x N, dv (T + 1) x N
-    static size_t kkt_bytes(long long T) {
+    static size_t kkt_bytes(long long T, bool vector) {
         const size_t t = (size_t)T;
         return 2 * up(t * N * sizeof(R)) + 2 * up(t * M * sizeof(R)) + 2 * up(N * sizeof(R)) +
                up((t + 1) * N * sizeof(R)) /* v' of the correction pass (Method 2) */ +
-               (kTeam ? up(t * M * M * sizeof(R)) : 0) /* G^{-1} of the first pass */;
+               (vector ? up(t * M * M * sizeof(R)) : 0) /* G^{-1} of the first pass */;
     }
     static size_t newton_bytes(long long T) {
         const size_t t = (size_t)T;
@@ -340,8 +340,8 @@ struct Launcher {
     }
 
     static size_t workspace(const ChainProblem* probs, int count, bool refine, bool newton,
-                            bool method2) {
-        return layout(probs, count, refine, newton, method2).total;
+                            bool method2, bool vector) {
+        return layout(probs, count, refine, newton, method2, vector && kTeam).total;
     }
 
     // Kernel names for the profile, by pass: the solve, the correction pass of
@@ -539,11 +539,10 @@ struct Launcher {
     }
 
     // The correction pass by vector walks (lqt_vector_walk.cuh): Method 1 of the
-    // parallel solve at the team sizes.  Method 2 and the sequential recursion
-    // solve the correction problem with their own passes.
-    static bool vector_correction(const ChainCall& call) {
-        return kTeam && call.refine && !call.method2 && !call.sequential;
-    }
+    // parallel solve at the team sizes.  Method 2, the sequential recursion and
+    // calls whose workspace has no room for the maps and G^{-1} solve the
+    // correction problem with their own passes.
+    static bool vector_correction(const ChainCall& call) { return kTeam && call.vector; }
     static void correct(const Args<R, RT>& b, const RT* maps, const long long* active, int levels,
                         cudaStream_t s, Prof* prof) {
         if constexpr (kTeam) {
@@ -570,7 +569,7 @@ struct Launcher {
         if (prepare_warm() != cudaSuccess) return LQT_ECUDA;
         const int count = call.count;
         if (count <= 0) return LQT_OK;
-        const Layout L = layout(call.probs, count, false, false, false);
+        const Layout L = layout(call.probs, count, false, false, false, false);
         if (call.ws_bytes < L.total) return LQT_ENOMEM;
         char* base = static_cast<char*>(call.ws);
         std::vector<Item<R>> it1((size_t)count);
@@ -643,7 +642,7 @@ struct Launcher {
         const bool refine = call.refine;
         const bool newton = refine && call.newton;
         const bool method2 = call.method2;
-        const Layout L = layout(call.probs, count, refine, newton, method2);
+        const Layout L = layout(call.probs, count, refine, newton, method2, vector_correction(call));
         RT* E2 = method2 ? reinterpret_cast<RT*>(base_of(call) + L.E2) : nullptr;
         RT* Pref = method2 ? reinterpret_cast<RT*>(base_of(call) + L.Pref) : nullptr;
         if (call.ws_bytes < L.total) return LQT_ENOMEM;
@@ -681,8 +680,9 @@ struct Launcher {
                 R* x0p = etaT + up(N * sizeof(R)) / sizeof(R);
                 R* vcorr = x0p + up(N * sizeof(R)) / sizeof(R);
                 if (vector_correction(call)) a.gi = vcorr + up((t + 1) * N * sizeof(R)) / sizeof(R);
-                char* nb = base + roff + kkt_bytes(cp.problem->T);
-                roff += kkt_bytes(cp.problem->T) + (newton ? newton_bytes(cp.problem->T) : 0);
+                char* nb = base + roff + kkt_bytes(cp.problem->T, vector_correction(call));
+                roff += kkt_bytes(cp.problem->T, vector_correction(call)) +
+                        (newton ? newton_bytes(cp.problem->T) : 0);
                 set_correction(it2[(size_t)i], a, eta, ctil, etaT, qh, dbuf, x0p);
                 if (method2) it2[(size_t)i].D.v = vcorr;
                 if (!newton) continue;
@@ -832,6 +832,26 @@ struct Launcher {
         return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;
     }
 
+    // Kernel launches of one problem of nc chunks (lqt_plan).
+    static int kernels(int nc, bool refine, bool newton, bool sequential, bool method2,
+                       bool vector) {
+        int l = 0;
+        while ((1 << l) < nc) ++l;
+        const int per = kTeam ? TT_LEVELS : 1;  // levels per launch
+        const auto runs = [&](int levels) { return (levels + per - 1) / per; };
+        const int up = sequential ? 0 : 1 + runs(kTeam && l > 0 ? l - 1 : l);  // fold, up-sweep
+        const int back = up + 1 + runs(l) + 1;         // terminal value, down-sweep, re-fold
+        const int scan = 2 * runs(l);                  // affine up- and down-sweep
+        // Method 2: the element copy, 2 l sweep levels, the seeds, the walk
+        const int fwd = method2 ? 2 * l + 3 : scan + 1;
+        int k = 1 + back + fwd;  // the item upload, the solve
+        if (refine) {            // residuals; the correction by walks or by a pass
+            const bool vec = kTeam && vector;
+            k += 1 + (vec ? 2 * (scan + 2) + (l > 0 ? 2 : 0) : back + fwd);
+        }
+        if (refine && newton) k += 2 + back + 3;  // upload, constants, residuals, scan, gains, add
+        return k;
+    }
     static int fold_groups_per_cta() { return kTeam ? NT_WALK : NG_FOLD; }
     static int fold_threads() { return kTeam ? NT_WALK * LGW : NG_FOLD * N; }
     static const void* fold_kernel() {
@@ -853,7 +873,8 @@ struct Launcher {
             &chain::Launcher<R, RT, N, M>::workspace, &chain::Launcher<R, RT, N, M>::run,       \
             &chain::Launcher<R, RT, N, M>::fold_kernel, &chain::Launcher<R, RT, N, M>::fold_smem, \
             &chain::Launcher<R, RT, N, M>::fold_groups_per_cta,                                 \
-            &chain::Launcher<R, RT, N, M>::fold_threads                                  \
+            &chain::Launcher<R, RT, N, M>::fold_threads,                                        \
+            &chain::Launcher<R, RT, N, M>::kernels                                              \
     }
 
 }  // namespace lqt

@@ -431,20 +431,11 @@ __device__ __forceinline__ bool solve_pivoted(R (&Mx)[N][N], R (&B)[N][NR]) {
 //   eta = X1^T (eta2 - J2 b1) + eta1,  J = A1^T J2 X1 + J1
 // using (I + J2 C1)^{-1} = M^{-T} and M^{-T} J2 = J2 M^{-1} (C, J symmetric).
 // `out` may alias e1 (in-place up-sweep); it must not alias e2.
-//
-// The vector parts are linear in the operands' vectors,
-//   b = b2 + G1 b1 + G2 eta2,   eta = eta1 + H1 eta2 + H2 b1,
-// with G1 = A2 M^{-1}, G2 = A2 M^{-1} C1, H1 = X1^T, H2 = -(J2 X1)^T.  With REC
-// the elimination also carries I (for M^{-1}) and the four maps are written
-// to fac (4 N^2 values, row-major G1 | G2 | H1 | H2), so that a problem with
-// the same matrices and other vectors can be combined by combine_replay.
-// Entry e of the maps is stored at fac[e * fs].
 // ---------------------------------------------------------------------------
-template <typename R, int N, bool REC = false>
+template <typename R, int N>
 __device__ __forceinline__ bool combine_view(ElemView<R, N> e1, ElemView<R, N> e2,
-                                             ElemView<R, N> out, R* fac = nullptr, int fs = 1) {
-    constexpr int NI = 2 * N + 1;  // first column of I when recording
-    constexpr int NR = NI + (REC ? N : 0);
+                                             ElemView<R, N> out) {
+    constexpr int NR = 2 * N + 1;
     R Mx[N][N];
     R B[N][NR];
 #pragma unroll
@@ -457,7 +448,6 @@ __device__ __forceinline__ bool combine_view(ElemView<R, N> e1, ElemView<R, N> e
             Mx[i][j] = t;
             B[i][j] = e1.A(i, j);
             B[i][N + 1 + j] = e1.C(i, j);
-            if constexpr (REC) B[i][NI + j] = (i == j) ? R(1) : R(0);
         }
         R t = e1.b(i);
 #pragma unroll
@@ -533,21 +523,6 @@ __device__ __forceinline__ bool combine_view(ElemView<R, N> e1, ElemView<R, N> e
             for (int k = 0; k < N; ++k) t += T3[i][k] * e2.A(j, k);
             Cn[sym<N>(i, j)] = t;
         }
-    if constexpr (REC) {
-        // T3 = A2 M^{-1} C1 is G2; e2 is not aliased by out
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                R g = R(0);
-#pragma unroll
-                for (int k = 0; k < N; ++k) g += e2.A(i, k) * B[k][NI + j];
-                fac[(i * N + j) * fs] = g;
-                fac[(N * N + i * N + j) * fs] = T3[i][j];
-                fac[(2 * N * N + i * N + j) * fs] = B[j][i];
-                fac[(3 * N * N + i * N + j) * fs] = -JX[j][i];
-            }
-    }
 #pragma unroll
     for (int i = 0; i < N; ++i) {
 #pragma unroll
@@ -563,45 +538,14 @@ __device__ __forceinline__ bool combine_view(ElemView<R, N> e1, ElemView<R, N> e
     return ok;
 }
 
-// The vector parts of e1 (x) e2 from the maps combine_view<REC> recorded for
-// operands with the same matrices: out.b, out.eta (out may alias e1).
-template <typename R, int N>
-__device__ __forceinline__ void combine_replay(const R* fac, int fs, ElemView<R, N> e1,
-                                               ElemView<R, N> e2, ElemView<R, N> out) {
-    R b1[N], h1[N], b2[N], h2[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        b1[i] = e1.b(i);
-        h1[i] = e1.eta(i);
-        b2[i] = e2.b(i);
-        h2[i] = e2.eta(i);
-    }
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        R b = b2[i], h = h1[i];
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            b += fac[(i * N + k) * fs] * b1[k] + fac[(N * N + i * N + k) * fs] * h2[k];
-            h += fac[(2 * N * N + i * N + k) * fs] * h2[k] +
-                 fac[(3 * N * N + i * N + k) * fs] * b1[k];
-        }
-        out.b(i) = b;
-        out.eta(i) = h;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Value carry through an element: (S, v) <- value part of P (x) (0, 0, 0, v, S)
 // (eq. lqt_comb with A2 = b2 = C2 = 0, as in the proof of Lemma LQT_assoc):
 //   X1 = (I + C_P S)^{-1} A_P
 //   S <- A_P^T S X1 + J_P,   v <- X1^T (v - S b_P) + eta_P
-// With REC the maps of the vector part, v <- eta_P + V1 v + V2 b_P with
-// V1 = X1^T and V2 = -(S X1)^T, are written to fac (2 N^2 values, V1 | V2)
-// for value_replay (entry e at fac[e * fs]).
 // ---------------------------------------------------------------------------
-template <typename R, int N, bool REC = false>
-__device__ __forceinline__ bool value_apply(ElemView<R, N> P, Value<R, N>& val,
-                                            R* fac = nullptr, int fs = 1) {
+template <typename R, int N>
+__device__ __forceinline__ bool value_apply(ElemView<R, N> P, Value<R, N>& val) {
     R Mx[N][N];
     R X[N][N];
 #pragma unroll
@@ -640,15 +584,6 @@ __device__ __forceinline__ bool value_apply(ElemView<R, N> P, Value<R, N>& val,
         for (int k = 0; k < N; ++k) t += X[k][i] * e[k];
         val.v[i] = t;
     }
-    if constexpr (REC) {
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                fac[(i * N + j) * fs] = X[j][i];
-                fac[(N * N + i * N + j) * fs] = -SX[j][i];
-            }
-    }
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
@@ -659,24 +594,6 @@ __device__ __forceinline__ bool value_apply(ElemView<R, N> P, Value<R, N>& val,
             val.S[sym<N>(i, j)] = t;
         }
     return ok;
-}
-
-// The vector part of value_apply from the maps value_apply<REC> recorded
-// for an element and a value with the same matrices: v <- eta_P + V1 v + V2 b_P.
-template <typename R, int N>
-__device__ __forceinline__ void value_replay(const R* fac, int fs, ElemView<R, N> P,
-                                             R (&v)[N]) {
-    R vn[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        R t = P.eta(i);
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-            t += fac[(i * N + k) * fs] * v[k] + fac[(N * N + i * N + k) * fs] * P.b(k);
-        vn[i] = t;
-    }
-#pragma unroll
-    for (int i = 0; i < N; ++i) v[i] = vn[i];
 }
 
 // ---------------------------------------------------------------------------
@@ -696,11 +613,11 @@ struct ElemCol {  // column j of A, C, J; entry j of b, eta
     R b, eta;
 };
 
-template <typename R, int N, bool REC = false>
+template <typename R, int N>
 __device__ __forceinline__ bool combine_col(ElemView<R, N> e1, ElemView<R, N> e2, int j,
-                                            ElemCol<R, N>& o, R* fac = nullptr, int fs = 1) {
-    constexpr int NR = 3 + (REC ? 2 : 0);
-    R Mx[N][N], B[N][NR];  // A1 e_j | b1 + C1 eta2 | C1 A2^T e_j  (REC: | e_j | C1 e_j)
+                                            ElemCol<R, N>& o) {
+    constexpr int NR = 3;
+    R Mx[N][N], B[N][NR];  // A1 e_j | b1 + C1 eta2 | C1 A2^T e_j
 #pragma unroll
     for (int i = 0; i < N; ++i) {
 #pragma unroll
@@ -717,10 +634,6 @@ __device__ __forceinline__ bool combine_col(ElemView<R, N> e1, ElemView<R, N> e2
         B[i][0] = e1.A(i, j);
         B[i][1] = t;
         B[i][2] = z;
-        if constexpr (REC) {
-            B[i][3] = (i == j) ? R(1) : R(0);
-            B[i][4] = e1.C(i, j);
-        }
     }
     const bool ok = solve_pivoted<R, N, NR>(Mx, B);
     R x[N], jx[N];
@@ -747,27 +660,16 @@ __device__ __forceinline__ bool combine_col(ElemView<R, N> e1, ElemView<R, N> e2
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         R a = R(0), c = e2.C(i, j), jj = e1.J(i, j);
-        R g1 = R(0), g2 = R(0);
 #pragma unroll
         for (int k = 0; k < N; ++k) {
             const R a2 = e2.A(i, k);
             a += a2 * x[k];
             c += a2 * B[k][2];
             jj += e1.A(k, i) * jx[k];
-            if constexpr (REC) {
-                g1 += a2 * B[k][3];
-                g2 += a2 * B[k][4];
-            }
         }
         o.A[i] = a;
         o.C[i] = c;
         o.J[i] = jj;
-        if constexpr (REC) {
-            fac[(i * N + j) * fs] = g1;
-            fac[(N * N + i * N + j) * fs] = g2;
-            fac[(2 * N * N + j * N + i) * fs] = x[i];
-            fac[(3 * N * N + j * N + i) * fs] = -jx[i];
-        }
     }
     return ok;
 }
@@ -787,24 +689,10 @@ __device__ __forceinline__ void store_col(const ElemCol<R, N>& o, int j, ElemVie
     out.eta(j) = o.eta;
 }
 
-// combine_replay's entry j of (b, eta).
-template <typename R, int N>
-__device__ __forceinline__ void combine_replay_row(const R* fac, int fs, ElemView<R, N> e1,
-                                                   ElemView<R, N> e2, int j, R& b, R& h) {
-    b = e2.b(j);
-    h = e1.eta(j);
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-        const R b1 = e1.b(k), h2 = e2.eta(k);
-        b += fac[(j * N + k) * fs] * b1 + fac[(N * N + j * N + k) * fs] * h2;
-        h += fac[(2 * N * N + j * N + k) * fs] * h2 + fac[(3 * N * N + j * N + k) * fs] * b1;
-    }
-}
-
 // value_apply's column j of S and entry j of v, for the value in view `in`.
-template <typename R, int N, bool REC = false>
+template <typename R, int N>
 __device__ __forceinline__ bool value_apply_col(ElemView<R, N> P, ValueView<R, N> in, int j,
-                                                R (&Sc)[N], R& vj, R* fac = nullptr, int fs = 1) {
+                                                R (&Sc)[N], R& vj) {
     R Mx[N][N], X[N][1];
     R S[Dims<N>::SYM];
 #pragma unroll
@@ -842,23 +730,8 @@ __device__ __forceinline__ bool value_apply_col(ElemView<R, N> P, ValueView<R, N
 #pragma unroll
         for (int k = 0; k < N; ++k) t += P.A(k, i) * sx[k];
         Sc[i] = t;
-        if constexpr (REC) {
-            fac[(j * N + i) * fs] = X[i][0];
-            fac[(N * N + j * N + i) * fs] = -sx[i];
-        }
     }
     return ok;
-}
-
-// value_replay's entry j of v.
-template <typename R, int N>
-__device__ __forceinline__ R value_replay_row(const R* fac, int fs, ElemView<R, N> P,
-                                              ValueView<R, N> in, int j) {
-    R t = P.eta(j);
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-        t += fac[(j * N + k) * fs] * in.v(k) + fac[(N * N + j * N + k) * fs] * P.b(k);
-    return t;
 }
 
 template <typename R, int N>

@@ -46,7 +46,9 @@ enum : int {
 
 enum : int { OUT_S = 1, OUT_V = 2, OUT_K = 4, OUT_ALL = 7 };
 
-enum : int { VEC_F = 1, VEC_L = 2, VEC_U = 4, VEC_C = 8, VEC_H = 16 };
+enum : int {
+    VEC_F = 1, VEC_L = 2, VEC_U = 4, VEC_C = 8, VEC_H = 16, VEC_S = 32, VEC_K = 64, VEC_R = 128
+};
 
 constexpr int kStageG = 2;  // steps per warp-staged group
 
@@ -78,11 +80,8 @@ struct Params {
     int out_mask;        // OUT_S | OUT_V | OUT_K: which of S, v, K this pass writes
     int refine_emit;     // first pass of a refined solve: write r', c', r'_T, x'_0
     int refine_add;      // second pass: x <- x + xi instead of x <- xi
-    // top-level backward scan: 0 full operators; 1 full operators that also
-    // record the maps of their vector parts in top_fac; 2 the vector parts
-    // alone from top_fac (a pass whose matrices equal the recording pass's)
-    int top_mode;
-    R* top_fac;
+    int keep_maps;       // first pass: keep the chunk maps for the second (kept_map)
+    int vector_pass;     // second pass: vector recursions from S, K and those maps
     long long wait_limit;  // polls of each bounded mbarrier wait
     int wait_probe;        // > 0: k_bwd_down also waits this many polls on a barrier
                            // nothing completes (diagnostic of the timeout path)
@@ -652,58 +651,38 @@ __device__ __forceinline__ void terminal_value(const Params<R>& P, Value<R, N>& 
 // CTA sweeps the partial totals, and the value carries flow back from the
 // terminal value (S_T, v_T) of Lemma LQT_assoc.
 // ===========================================================================
-// MODE (the pass's Params::top_mode) selects the kernel: 0 full operators,
-// 1 full operators recording their maps, 2 replay.  One kernel per mode keeps
-// each one's code small: the single warp that works at the upper levels
-// otherwise stalls on instruction fetch.  Modes 1 and 2 need one tile per
-// thread (tiles <= TP), which the host checks.
-template <typename R, int N, int TP, int MODE>
+template <typename R, int N, int TP>
 __global__ void __launch_bounds__(TP, 1) k_bwd_top(const Params<R> P) {
     griddep_launch_dependents();
     griddep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int TS = tstride(TP, (int)sizeof(R));      // tree slots per field
-    constexpr int FU = top_fac_up(N), FD = top_fac_dn(N);
     R* tree = reinterpret_cast<R*>(smem_raw);            // [ELEM][TS]
     R* carry = tree + (size_t)Dims<N>::ELEM * TS;        // [VALUE][TS]
-    R* sfac = carry + (size_t)Dims<N>::VALUE * TS;       // mode 2: staged factor store
+    R* stg = carry + (size_t)Dims<N>::VALUE * TS;        // staged tile totals
     const int tid = threadIdx.x;
     const int tiles = P.tiles;
     const int g = tiles > 0 ? (tiles + TP - 1) / TP : 1;
     const int used = tiles > 0 ? (tiles + g - 1) / g : 1;
     const int Teff = next_pow2(used);
     const int t0 = min(tid * g, tiles), t1 = min(t0 + g, tiles);
-    constexpr int mode = MODE;
-    if (mode != 0 && g != 1) {
-        // the factor store covers one tile per thread; the host rejects other
-        // plans before launching, so this only guards against a bad caller
-        if (tid == 0) set_status(P.status, ST_SINGULAR);
-        return;
-    }
     bool ok = true;
 
-    // Shared memory after the carries: [mode 2: the recorded maps of both
-    // sweeps] | the tile totals as stored ([tiles][ELEM], one tile per thread)
-    // | the mbarrier of the bulk copies that bring both in.
+    // Shared memory after the carries: the tile totals as stored ([tiles][ELEM],
+    // one tile per thread) | the mbarrier of the bulk copy that brings them in.
     constexpr int E = Dims<N>::ELEM;
-    constexpr long long kFacElems = mode == 2 ? top_fac_elems(N, TP) : 0;
-    constexpr uint32_t kFacBytes = (uint32_t)(kFacElems * sizeof(R));
-    static_assert(kFacBytes % 16 == 0, "bulk copy of 16-byte multiples");
-    R* stg = sfac + kFacElems;
     uint64_t* bar = reinterpret_cast<uint64_t*>(stg + top_stage_elems(E, TP, (int)sizeof(R)));
     const bool bulk = g == 1 && tiles > 0;  // tile totals by bulk copy
-    const bool stage = mode == 2 && Teff > 1;
     // the copy may round up past the last tile into the buffer's alignment padding
     const uint32_t agg_bytes = (uint32_t)(((size_t)tiles * E * sizeof(R) + 15) / 16 * 16);
-    if ((bulk || stage) && tid == 0) {
+    if (bulk && tid == 0) {
         mbar_init(bar, 1);
-        mbar_expect_tx(bar, (stage ? kFacBytes : 0u) + (bulk ? agg_bytes : 0u));
-        if (stage) bulk_g2s(sfac, P.top_fac, kFacBytes, bar);
-        if (bulk) bulk_g2s(stg, P.tile_agg, agg_bytes, bar);
+        mbar_expect_tx(bar, agg_bytes);
+        bulk_g2s(stg, P.tile_agg, agg_bytes, bar);
     }
     // thread partial: tile totals t0..t1-1 folded right to left (neutral if empty)
     ElemView<R, N> mine{tree + tslot<R>(tid), TS};
-    if (mode == 0 && !bulk && t1 > t0) {  // several tiles per thread (mode 0 only)
+    if (!bulk && t1 > t0) {  // several tiles per thread
         const R* src = P.tile_agg + (size_t)(t1 - 1) * E;
         for (int k = 0; k < E; ++k) mine.p[k * TS] = src[k];
         for (int t = t1 - 2; t >= t0; --t)
@@ -732,7 +711,7 @@ __global__ void __launch_bounds__(TP, 1) k_bwd_top(const Params<R> P) {
         }
     }
     __syncthreads();  // the mbarrier is initialised before anyone waits on it
-    if (bulk || stage) {
+    if (bulk) {
         const bool ok_load = mbar_wait(bar, 0, P.wait_limit);
         if (!ok_load) {
             mbar_wait(bar, 0, P.wait_limit);  // one more bounded wait for the copies in flight
@@ -740,131 +719,49 @@ __global__ void __launch_bounds__(TP, 1) k_bwd_top(const Params<R> P) {
         }
     }
     if (bulk && t1 > t0) {
-        // this thread's tile total into its tree slot (mode 2: the vectors alone)
+        // this thread's tile total into its tree slot
         const R* row = stg + (size_t)tid * E;
-        if (mode == 2) {
-#pragma unroll
-            for (int k = 0; k < N; ++k) {
-                mine.b(k) = row[Dims<N>::OB + k];
-                mine.eta(k) = row[Dims<N>::OE + k];
-            }
-        } else {
 #pragma unroll 4
-            for (int k = 0; k < E; ++k) mine.p[k * TS] = row[k];
-        }
+        for (int k = 0; k < E; ++k) mine.p[k * TS] = row[k];
     }
     __syncthreads();
-    // up-sweep; the combines of level h are numbered after those of the lower
-    // levels (Teff / 2h of them), thread order within a level
-    int node = 0;
+    // up-sweep
 #pragma unroll 1
     for (int h = 1; h < Teff; h <<= 1) {
         const int i = tid * 2 * h;
-        if (team_level<R, N, true>(Teff / (2 * h))) {
-            const int t = tid / N, j = tid % N, it = 2 * h * t;
-            const bool act = t < Teff / (2 * h);
-            const ElemView<R, N> e1{tree + tslot<R>(it), TS}, e2{tree + tslot<R>(it + h), TS};
-            if (mode == 2) {
-                R b = R(0), eta = R(0);
-                if (act) combine_replay_row<R, N>(sfac + node + t, TP, e1, e2, j, b, eta);
-                __syncwarp();
-                if (act) {
-                    e1.b(j) = b;
-                    e1.eta(j) = eta;
-                }
-            } else {
-                ElemCol<R, N> o;
-                if (act)
-                    ok &= combine_col<R, N, mode == 1>(e1, e2, j, o, P.top_fac + node + t, TP);
-                __syncwarp();
-                if (act) store_col(o, j, e1);
-            }
-        } else if (i < Teff) {
-            const ElemView<R, N> e1{tree + tslot<R>(i), TS}, e2{tree + tslot<R>(i + h), TS};
-            if (mode == 2)
-                combine_replay<R, N>(sfac + node + tid, TP, e1, e2, e1);
-            else if (mode == 1)
-                ok &= combine_view<R, N, true>(e1, e2, e1, P.top_fac + node + tid, TP);
-            else
-                ok &= combine_view<R, N>(e1, e2, e1);
-        }
-        node += Teff / (2 * h);
+        if (team_level<R, N, true>(Teff / (2 * h)))
+            ok &= team_combine_level<R, N>(tree, TS, h, Teff / (2 * h), tid);
+        else if (i < Teff)
+            ok &= combine_view<R, N>(ElemView<R, N>{tree + tslot<R>(i), TS},
+                                     ElemView<R, N>{tree + tslot<R>(i + h), TS},
+                                     ElemView<R, N>{tree + tslot<R>(i), TS});
         __syncthreads();
     }
-    // down-sweep, applies numbered the same way from the top level
-    R* gdn = P.top_fac + (long long)TP * FU;
-    const R* sdn = sfac + (long long)TP * FU;
-    node = 0;
+    // down-sweep
 #pragma unroll 1
     for (int h = Teff / 2; h >= 1; h >>= 1) {
         const int i = tid * 2 * h;
         if (team_level<R, N, true>(Teff / (2 * h))) {
-            const int t = tid / N, j = tid % N, it = 2 * h * t;
-            const bool act = t < Teff / (2 * h);
-            const ValueView<R, N> ci{carry + tslot<R>(it), TS}, ch{carry + tslot<R>(it + h), TS};
-            const ElemView<R, N> el{tree + tslot<R>(it + h), TS};
-            R v = R(0), vo = R(0);
-            if (mode == 2) {
-                if (act) {
-                    v = value_replay_row<R, N>(sdn + node + t, TP, el, ci, j);
-                    vo = ci.v(j);
-                }
-                __syncwarp();
-                if (act) {
-                    ch.v(j) = vo;
-                    ci.v(j) = v;
-                }
-            } else {
-                R Sc[N];
-                if (act)
-                    ok &= value_apply_col<R, N, mode == 1>(el, ci, j, Sc, v, gdn + node + t, TP);
-                __syncwarp();
-                if (act) team_store_value<R, N>(ci, ch, j, Sc, v);
-            }
+            ok &= team_apply_level<R, N>(tree, carry, TS, h, Teff / (2 * h), tid);
         } else if (i < Teff) {
             const ValueView<R, N> ci{carry + tslot<R>(i), TS}, ch{carry + tslot<R>(i + h), TS};
-            const ElemView<R, N> el{tree + tslot<R>(i + h), TS};
-            if (mode == 2) {
-                // the values' S equal the recording pass's: only v moves
-                R v[N];
-#pragma unroll
-                for (int k = 0; k < N; ++k) v[k] = ci.v(k);
-#pragma unroll
-                for (int k = 0; k < N; ++k) ch.v(k) = v[k];
-                value_replay<R, N>(sdn + node + tid, TP, el, v);
-#pragma unroll
-                for (int k = 0; k < N; ++k) ci.v(k) = v[k];
-            } else {
-                Value<R, N> c;
-                load_value(c, ci);
-                store_value(c, ch);
-                if (mode == 1)
-                    ok &= value_apply<R, N, true>(el, c, gdn + node + tid, TP);
-                else
-                    ok &= value_apply<R, N>(el, c);
-                store_value(c, ci);
-            }
+            Value<R, N> c;
+            load_value(c, ci);
+            store_value(c, ch);
+            ok &= value_apply<R, N>(ElemView<R, N>{tree + tslot<R>(i + h), TS}, c);
+            store_value(c, ci);
         }
-        node += Teff / (2 * h);
         __syncthreads();
     }
     // per-tile carries for this thread's tiles
     if (t1 > t0) {
-        if (mode == 2) {
-            // S of the carries stays as the recording pass wrote it
-            R* dst = P.tile_carry + (size_t)t0 * Dims<N>::VALUE + Dims<N>::SYM;
-#pragma unroll
-            for (int k = 0; k < N; ++k) dst[k] = carry[(Dims<N>::SYM + k) * TS + tslot<R>(tid)];
-        } else {
-            Value<R, N> c;
-            load_value(c, ValueView<R, N>{carry + tslot<R>(tid), TS});
-            for (int t = t1 - 1; t >= t0; --t) {
-                store_value(c, ValueView<R, N>{P.tile_carry + (size_t)t * Dims<N>::VALUE, 1});
-                if (t > t0)
-                    ok &= value_apply<R, N>(
-                        ElemView<R, N>{const_cast<R*>(P.tile_agg) + (size_t)t * Dims<N>::ELEM, 1},
-                        c);
-            }
+        Value<R, N> c;
+        load_value(c, ValueView<R, N>{carry + tslot<R>(tid), TS});
+        for (int t = t1 - 1; t >= t0; --t) {
+            store_value(c, ValueView<R, N>{P.tile_carry + (size_t)t * Dims<N>::VALUE, 1});
+            if (t > t0)
+                ok &= value_apply<R, N>(
+                    ElemView<R, N>{const_cast<R*>(P.tile_agg) + (size_t)t * Dims<N>::ELEM, 1}, c);
         }
     }
     if (!ok) set_status(P.status, ST_SINGULAR);
@@ -885,6 +782,79 @@ __device__ __forceinline__ void terminal_outputs(const Params<R>& P, const Value
             for (int j = 0; j < N; ++j) ST[i * N + j] = z.S[sym<N>(i, j)];
         }
         if (P.out_mask & OUT_V) P.v[(size_t)P.T * N + i] = z.v[i];
+    }
+}
+
+// A tile's block of the backward tree ([ELEM][WS]) is free once its CTA has
+// loaded it: the second pass's value tree takes its first AFFINE fields, the
+// first pass's chunk maps ([N*N][W]) the place behind them.
+template <typename R, int N, int W>
+__device__ __forceinline__ R* kept_maps(R* tree, unsigned tile) {
+    constexpr int WS = tstride(W, (int)sizeof(R));
+    static_assert((Dims<N>::ELEM - Dims<N>::AFFINE) * WS >= N * N * W, "the maps fit");
+    return tree + (size_t)tile * Dims<N>::ELEM * WS + Dims<N>::AFFINE * WS;
+}
+
+// The forward tree of a tile in shared memory ([AFFINE][WS]): the map (Phi, gam)
+// at slot `slot`, then the right-anchored up-sweep: after level d, slot
+// j = i + 2^{d+1} - 1 holds the composite of slots [i, i + 2^{d+1}), slot
+// i + 2^d - 1 keeps [i, i + 2^d).  Unless SOLO the tree and the tile's total go
+// to global memory.
+template <typename R, int N, int W, bool SOLO>
+__device__ __forceinline__ void affine_sweep(R* ftree, const R (&Phi)[N][N], const R (&gam)[N],
+                                             int slot, int Weff, R* tree_out, size_t tree_stride,
+                                             R* agg_out, unsigned tile) {
+    constexpr int WS = tstride(W, (int)sizeof(R));
+    const int tid = threadIdx.x;
+    if (slot >= 0) {
+        AffineView<R, N> mine{ftree + tslot<R>(slot), WS};
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) mine.F(i, j) = Phi[i][j];
+            mine.c(i) = gam[i];
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int h = 1; h < Weff; h <<= 1) {
+        const int j = tid * 2 * h + 2 * h - 1;
+        if (j < Weff)
+            affine_compose_view<R, N>(AffineView<R, N>{ftree + tslot<R>(j - h), WS},
+                                      AffineView<R, N>{ftree + tslot<R>(j), WS},
+                                      AffineView<R, N>{ftree + tslot<R>(j), WS});
+        __syncthreads();
+    }
+    if (!SOLO) {
+        if (tid < Dims<N>::AFFINE)
+            agg_out[(size_t)tile * Dims<N>::AFFINE + tid] = ftree[tid * WS + tslot<R>(Weff - 1)];
+        cta_bulk_store(tree_out + tile * tree_stride, ftree,
+                       (uint32_t)(Dims<N>::AFFINE * WS * sizeof(R)));
+    }
+}
+
+// The down-sweep of the states through that tree: slot Weff - 1 of xs ([N][WS])
+// holds the state at the tile's start on entry, slot i the state at the start
+// of slot i's map on return.
+template <typename R, int N, int W>
+__device__ __forceinline__ void affine_descend(const R* ftree, R* xs, int Weff) {
+    constexpr int WS = tstride(W, (int)sizeof(R));
+    const int tid = threadIdx.x;
+#pragma unroll 1
+    for (int h = Weff / 2; h >= 1; h >>= 1) {
+        const int j = tid * 2 * h + 2 * h - 1;
+        if (j < Weff) {
+            R xv[N];
+#pragma unroll
+            for (int i = 0; i < N; ++i) xv[i] = xs[i * WS + tslot<R>(j)];
+#pragma unroll
+            for (int i = 0; i < N; ++i) xs[i * WS + tslot<R>(j - h)] = xv[i];
+            affine_apply_view<R, N>(AffineView<R, N>{const_cast<R*>(ftree) + tslot<R>(j - h), WS},
+                                    xv);
+#pragma unroll
+            for (int i = 0; i < N; ++i) xs[i * WS + tslot<R>(j)] = xv[i];
+        }
+        __syncthreads();
     }
 }
 
@@ -1048,36 +1018,14 @@ __device__ __forceinline__ void bwd_down_body(const Params<R>& P, unsigned tile,
         WarpRows<R, M, kStageG>::store(P.u, tbase, rows + SM::DD, SM::DROW, lrel, cnt);
         __syncwarp();
     }
+    if (P.keep_maps) {
+        R* keep = kept_maps<R, N, W>(P.tree, tile);
+#pragma unroll
+        for (int i = 0; i < N * N; ++i) keep[i * W + tid] = Phi[i / N][i % N];
+    }
     __syncthreads();  // the big area becomes the forward tree
-    // forward up-sweep (right-anchored): after level d, slot j = i + 2^{d+1} - 1
-    // holds the composite of chunks [i, i + 2^{d+1}); slot i + 2^d - 1 keeps [i, i + 2^d)
-    R* ftree = big;  // [AFFINE][WS]
-    {
-        AffineView<R, N> mine{ftree + tslot<R>(tid), WS};
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-#pragma unroll
-            for (int j = 0; j < N; ++j) mine.F(i, j) = Phi[i][j];
-            mine.c(i) = gam[i];
-        }
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int h = 1; h < Weff; h <<= 1) {
-        const int j = tid * 2 * h + 2 * h - 1;
-        if (j < Weff)
-            affine_compose_view<R, N>(AffineView<R, N>{ftree + tslot<R>(j - h), WS},
-                                      AffineView<R, N>{ftree + tslot<R>(j), WS},
-                                      AffineView<R, N>{ftree + tslot<R>(j), WS});
-        __syncthreads();
-    }
-    if (!SOLO) {
-        if (tid < Dims<N>::AFFINE)
-            P.ftile_agg[(size_t)tile * Dims<N>::AFFINE + tid] =
-                ftree[tid * WS + tslot<R>(Weff - 1)];
-        cta_bulk_store(P.ftree + (size_t)tile * Dims<N>::AFFINE * WS, ftree,
-                       (uint32_t)(Dims<N>::AFFINE * WS * sizeof(R)));
-    }
+    affine_sweep<R, N, W, SOLO>(big, Phi, gam, tid, Weff, P.ftree, Dims<N>::AFFINE * WS,
+                                P.ftile_agg, tile);
     if (!ok) set_status(P.status, ST_NOTSPD);
     if (!finite) set_status(P.status, ST_NONFINITE);
     if (!ok_sing) set_status(P.status, ST_SINGULAR);
@@ -1099,7 +1047,9 @@ __global__ void __launch_bounds__(W, 1) k_bwd_down(const Params<R> P) {
 // fwd_top: one CTA of TP threads; prefix scan of tile affine maps seeded with
 // x_0 (Lemma lqt_fwd_init: the first element maps everything to the state).
 // ===========================================================================
-template <typename R, int N, int TP>
+// VALUE: the scan of the second pass's value maps instead (k_vec_up; tiles from
+// the last to the first), seeded with v_T.
+template <typename R, int N, int TP, bool VALUE>
 __global__ void __launch_bounds__(TP, 1) k_fwd_top(const Params<R> P) {
     griddep_launch_dependents();
     griddep_wait();
@@ -1108,6 +1058,8 @@ __global__ void __launch_bounds__(TP, 1) k_fwd_top(const Params<R> P) {
     R* tree = reinterpret_cast<R*>(smem_raw);      // [AFFINE][TS]
     R* xs = tree + (size_t)Dims<N>::AFFINE * TS;   // [N][TS]
     const int tid = threadIdx.x;
+    R* const agg = VALUE ? P.tile_agg : P.ftile_agg;
+    R* const ends = VALUE ? P.tile_carry : P.ftile_x;
     const int tiles = P.tiles;
     const int g = tiles > 0 ? (tiles + TP - 1) / TP : 1;
     const int used = tiles > 0 ? (tiles + g - 1) / g : 1;
@@ -1123,7 +1075,7 @@ __global__ void __launch_bounds__(TP, 1) k_fwd_top(const Params<R> P) {
         }
         for (int t = t0; t < t1; ++t)
             affine_compose_view<R, N>(
-                mine, AffineView<R, N>{P.ftile_agg + (size_t)t * Dims<N>::AFFINE, 1}, mine);
+                mine, AffineView<R, N>{agg + (size_t)t * Dims<N>::AFFINE, 1}, mine);
     }
     __syncthreads();
 #pragma unroll 1
@@ -1135,7 +1087,14 @@ __global__ void __launch_bounds__(TP, 1) k_fwd_top(const Params<R> P) {
                                       AffineView<R, N>{tree + tslot<R>(j), TS});
         __syncthreads();
     }
-    if (tid == 0) {
+    if (VALUE) {
+        if (tid == 0) {
+            Value<R, N> z;
+            terminal_value<R, N>(P, z);
+#pragma unroll
+            for (int i = 0; i < N; ++i) xs[i * TS + tslot<R>(Teff - 1)] = z.v[i];
+        }
+    } else if (tid == 0) {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             const R x0 = P.x0[i];
@@ -1165,8 +1124,8 @@ __global__ void __launch_bounds__(TP, 1) k_fwd_top(const Params<R> P) {
         for (int i = 0; i < N; ++i) xv[i] = xs[i * TS + tslot<R>(tid)];
         for (int t = t0; t < t1; ++t) {
 #pragma unroll
-            for (int i = 0; i < N; ++i) P.ftile_x[(size_t)t * N + i] = xv[i];
-            affine_apply_view<R, N>(AffineView<R, N>{P.ftile_agg + (size_t)t * Dims<N>::AFFINE, 1}, xv);
+            for (int i = 0; i < N; ++i) ends[(size_t)t * N + i] = xv[i];
+            affine_apply_view<R, N>(AffineView<R, N>{agg + (size_t)t * Dims<N>::AFFINE, 1}, xv);
         }
     }
 }
@@ -1211,21 +1170,7 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
         }
     }
     __syncthreads();
-#pragma unroll 1
-    for (int h = Weff / 2; h >= 1; h >>= 1) {
-        const int j = tid * 2 * h + 2 * h - 1;
-        if (j < Weff) {
-            R xv[N];
-#pragma unroll
-            for (int i = 0; i < N; ++i) xv[i] = xs[i * WS + tslot<R>(j)];
-#pragma unroll
-            for (int i = 0; i < N; ++i) xs[i * WS + tslot<R>(j - h)] = xv[i];
-            affine_apply_view<R, N>(AffineView<R, N>{ftree + tslot<R>(j - h), WS}, xv);
-#pragma unroll
-            for (int i = 0; i < N; ++i) xs[i * WS + tslot<R>(j)] = xv[i];
-        }
-        __syncthreads();
-    }
+    affine_descend<R, N, W>(ftree, xs, Weff);
     // The chunk stores its own start state (the tree value) and the states of
     // its steps; the state after its last step is the next chunk's start (or,
     // for the last chunk, its own x_T).  Stored states and the shifted data of
@@ -1419,6 +1364,314 @@ __global__ void __launch_bounds__(W, 1) k_fwd_down(const Params<R> P) {
 }
 
 // ===========================================================================
+// The second pass of a refined solve: its matrices, and so S, K and the chunk
+// maps Phi, are the first pass's, so only vectors are scanned.  With
+// w_k = v_{k+1} - S_{k+1} c_k and Ft_k = F_k - L_k K_k (Sec. II-B)
+//   v_k = Ft_k^T w_k + q_k,   d_k = G_k^{-1} L_k^T w_k,
+// so a chunk maps v at its end to v at its start by (Phi^T, beta).
+//   vec_up    per chunk beta, the in-tile sweep of the value maps (slots and
+//             tiles mirrored, so that the affine tree runs from the last chunk
+//             to the first),
+//   fwd_top<VALUE>  v at the end of every tile from v_T,
+//   vec_down  v at the end of every chunk, the chunk's steps again for d_k (into
+//             u) and the offset of its forward map, the in-tile forward sweep;
+// then fwd_top and fwd_down as in the first pass.  An element pass folds 44
+// numbers a step through 4 x 4 operators of 2300 cycles a tree level; the
+// vectors take a quarter of the arithmetic and levels of 500 cycles, for 96
+// bytes a step of S and K to read back.
+// ===========================================================================
+template <typename R, int N, int M>
+struct VecStep {
+    R F[N][N], L[N][M], K[M][N], S[Dims<N>::SYM], c[N], q[N];
+};
+
+template <typename R, int N, int M, bool INV>
+__device__ __forceinline__ void load_vec_step(const Params<R>& P, long long k, const R* sm,
+                                              VecStep<R, N, M>& st) {
+    using ML = ModelLayout<N, M>;
+    if (INV || P.dyn_invariant) {
+        load_row<R, N * N>(sm + ML::OF, &st.F[0][0]);
+        load_row<R, N * M>(sm + ML::OL, &st.L[0][0]);
+    } else {
+        ldg_vals<R, N * N>(P.F + k * P.sF, P.vec & VEC_F, &st.F[0][0]);
+        ldg_vals<R, N * M>(P.L + k * P.sL, P.vec & VEC_L, &st.L[0][0]);
+    }
+    R full[N * N];
+    ldg_vals<R, N * N>(P.S + (k + 1) * (N * N), P.vec & VEC_S, full);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = i; j < N; ++j) st.S[sym<N>(i, j)] = full[i * N + j];
+    ldg_vals<R, M * N>(P.K + k * (M * N), P.vec & VEC_K, &st.K[0][0]);
+    ldg_vals<R, N>(P.c + k * P.sc, P.vec & VEC_C, st.c);
+#pragma unroll
+    for (int i = 0; i < N; ++i) st.q[i] = R(0);
+    if (!P.r) return;
+    const int p = P.p;
+    const R* r = P.r + k * P.sr;
+    R r4[kRStage];  // r' is padded to kRStage values a step when p <= kRStage
+    if (p <= kRStage) ldg_vals<R, kRStage>(r, P.vec & VEC_R, r4);
+    if (INV || P.cost_invariant) {
+        const R* sHX = sm + ML::OHX;
+        if (p <= kRStage) {
+#pragma unroll
+            for (int a = 0; a < kRStage; ++a)
+                if (a < p) {
+                    R hx[N];
+                    load_row<R, N>(sHX + a * N, hx);
+#pragma unroll
+                    for (int i = 0; i < N; ++i) st.q[i] += hx[i] * r4[a];
+                }
+        } else {
+            for (int a = 0; a < p; ++a) {
+                const R ra = __ldg(r + a);
+#pragma unroll
+                for (int i = 0; i < N; ++i) st.q[i] += sHX[a * N + i] * ra;
+            }
+        }
+    } else {
+        const R* H = P.H + k * P.sH;
+        const R* X = P.X + k * P.sX;
+        for (int a = 0; a < p; ++a) {
+            R y = R(0), h[N];
+            if (p <= kRStage) {
+#pragma unroll
+                for (int b = 0; b < kRStage; ++b)
+                    if (b < p) y += __ldg(X + a * p + b) * r4[b];
+            } else {
+                for (int b = 0; b < p; ++b) y += __ldg(X + a * p + b) * __ldg(r + b);
+            }
+            ldg_vals<R, N>(H + a * N, P.vec & VEC_H, h);
+#pragma unroll
+            for (int i = 0; i < N; ++i) st.q[i] += h[i] * y;
+        }
+    }
+}
+
+// v <- Ft^T w + q with w = v - S c; y = L^T w for the caller
+template <typename R, int N, int M>
+__device__ __forceinline__ void vec_back(const VecStep<R, N, M>& st, R (&v)[N], R (&y)[M]) {
+    R w[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        R t = v[i];
+#pragma unroll
+        for (int j = 0; j < N; ++j) t -= st.S[sym<N>(i, j)] * st.c[j];
+        w[i] = t;
+    }
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+        R t = R(0);
+#pragma unroll
+        for (int i = 0; i < N; ++i) t += st.L[i][a] * w[i];
+        y[a] = t;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        R t = st.q[i];
+#pragma unroll
+        for (int l = 0; l < N; ++l) t += st.F[l][i] * w[l];
+#pragma unroll
+        for (int a = 0; a < M; ++a) t -= st.K[a][i] * y[a];
+        v[i] = t;
+    }
+}
+
+template <typename R, int N, int M, int W, bool SOLO, bool INV>
+__device__ __forceinline__ void vec_up_body(const Params<R>& P, unsigned tile, R* ftree,
+                                            const R* sm) {
+    const int tid = threadIdx.x;
+    const TileGeo geo{P.T, (long long)tile * W, P.B};
+    const int Weff = next_pow2(geo.live(W));
+    long long s, e;
+    geo.chunk(tid, s, e);
+    R Psi[N][N], v[N];
+    const R* keep = kept_maps<R, N, W>(P.tree, tile);
+#pragma unroll
+    for (int i = 0; i < N * N; ++i)
+        Psi[i % N][i / N] = keep[i * W + tid];
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = R(0);
+    for (long long k = e - 1; k >= s; --k) {
+        VecStep<R, N, M> st;
+        load_vec_step<R, N, M, INV>(P, k, sm, st);
+        R y[M];
+        vec_back(st, v, y);
+    }
+    affine_sweep<R, N, W, SOLO>(ftree, Psi, v, Weff - 1 - tid, Weff, P.tree,
+                                Dims<N>::ELEM * tstride(W, (int)sizeof(R)), P.tile_agg,
+                                P.tiles - 1 - tile);
+}
+
+// xs: the down-swept values, slot Weff - 1 - tid for this thread's chunk
+template <typename R, int N, int M, int W, bool SOLO, bool INV>
+__device__ __forceinline__ void vec_down_body(const Params<R>& P, unsigned tile, R* ftree, R* xs,
+                                              const R* sm) {
+    using ML = ModelLayout<N, M>;
+    constexpr int WS = tstride(W, (int)sizeof(R));
+    const int tid = threadIdx.x;
+    const TileGeo geo{P.T, (long long)tile * W, P.B};
+    const int Weff = next_pow2(geo.live(W));
+    affine_descend<R, N, W>(ftree, xs, Weff);
+    long long s, e;
+    geo.chunk(tid, s, e);
+    R v[N], Phi[N][N], gam[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[i] = tid < Weff ? xs[i * WS + tslot<R>(Weff - 1 - tid)] : R(0);
+        gam[i] = R(0);
+#pragma unroll
+        for (int j = 0; j < N; ++j) Phi[i][j] = i == j ? R(1) : R(0);
+    }
+    __syncthreads();  // the tree area becomes the forward tree
+    bool ok = true;
+    for (long long k = e - 1; k >= s; --k) {
+        VecStep<R, N, M> st;
+        load_vec_step<R, N, M, INV>(P, k, sm, st);
+        R U[M][M];
+        if (INV || P.dyn_invariant)
+            load_row<R, M * M>(sm + ML::OU, &U[0][0]);
+        else
+            ldg_vals<R, M * M>(P.U + k * P.sU, P.vec & VEC_U, &U[0][0]);
+        R d[M];
+        vec_back(st, v, d);
+        // G = L^T S L + U = Rc Rc^T, d <- G^{-1} d (as in riccati_step)
+        R SL[N][M], Rc[M][M], Rinv[M];
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int a = 0; a < M; ++a) {
+                R t = R(0);
+#pragma unroll
+                for (int j = 0; j < N; ++j) t += st.S[sym<N>(i, j)] * st.L[j][a];
+                SL[i][a] = t;
+            }
+#pragma unroll
+        for (int a = 0; a < M; ++a) {
+            R g = U[a][a];
+#pragma unroll
+            for (int i = 0; i < N; ++i) g += st.L[i][a] * SL[i][a];
+#pragma unroll
+            for (int l = 0; l < a; ++l) g -= Rc[a][l] * Rc[a][l];
+            ok = ok && (g > R(0));
+            const R rt = sqrt(g);
+            Rc[a][a] = rt;
+            Rinv[a] = rcp_(rt);
+#pragma unroll
+            for (int b = a + 1; b < M; ++b) {
+                R t = U[a][b];
+#pragma unroll
+                for (int i = 0; i < N; ++i) t += st.L[i][a] * SL[i][b];
+#pragma unroll
+                for (int l = 0; l < a; ++l) t -= Rc[b][l] * Rc[a][l];
+                Rc[b][a] = t * Rinv[a];
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < M; ++a) {
+            R t = d[a];
+#pragma unroll
+            for (int l = 0; l < a; ++l) t -= Rc[a][l] * d[l];
+            d[a] = t * Rinv[a];
+        }
+#pragma unroll
+        for (int a = M - 1; a >= 0; --a) {
+            R t = d[a];
+#pragma unroll
+            for (int l = a + 1; l < M; ++l) t -= Rc[l][a] * d[l];
+            d[a] = t * Rinv[a];
+        }
+        if (M * sizeof(R) == 8 && (P.vec & VEC_K))
+            store_row<R, M>(P.u + k * M, d);  // u is aligned with K, see fill_params
+        else
+#pragma unroll
+            for (int a = 0; a < M; ++a) P.u[k * M + a] = d[a];
+        // the chunk's forward map: gam <- gam + Phi ct, Phi <- Phi Ft
+        R Pn[N][N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            R ft[N];
+            R ct = st.c[j];
+#pragma unroll
+            for (int a = 0; a < M; ++a) ct += st.L[j][a] * d[a];
+#pragma unroll
+            for (int i = 0; i < N; ++i) gam[i] += Phi[i][j] * ct;
+            // column j of Ft
+#pragma unroll
+            for (int l = 0; l < N; ++l) {
+                R t = st.F[l][j];
+#pragma unroll
+                for (int a = 0; a < M; ++a) t -= st.L[l][a] * st.K[a][j];
+                ft[l] = t;
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                R t = R(0);
+#pragma unroll
+                for (int l = 0; l < N; ++l) t += Phi[i][l] * ft[l];
+                Pn[i][j] = t;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) Phi[i][j] = Pn[i][j];
+    }
+    affine_sweep<R, N, W, SOLO>(ftree, Phi, gam, tid, Weff, P.ftree, Dims<N>::AFFINE * WS,
+                                P.ftile_agg, tile);
+    if (!ok) set_status(P.status, ST_NOTSPD);
+}
+
+// Dynamic shared memory of vec_up and vec_down: head, tree and values, model.
+template <typename R, int N, int M, int W>
+struct VecSmem {
+    static constexpr int WS = tstride(W, (int)sizeof(R));
+    static constexpr int XS = Dims<N>::AFFINE * WS, MODEL = XS + N * WS;
+    static_assert(MODEL % 4 == 0, "16-byte model area");
+    static size_t bytes(int p) {
+        return kSmemHead + (size_t)(MODEL + ModelLayout<N, M>::size(p)) * sizeof(R);
+    }
+};
+
+template <typename R, int N, int M, int W, bool INV>
+__global__ void __launch_bounds__(W, 1) k_vec_up(const Params<R> P) {
+    griddep_launch_dependents();
+    griddep_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    R* tree = reinterpret_cast<R*>(smem_raw + kSmemHead);
+    R* sm = tree + VecSmem<R, N, M, W>::MODEL;
+    model_prologue<R, N, M>(P, sm);
+    vec_up_body<R, N, M, W, false, INV>(P, blockIdx.x, tree, sm);
+}
+
+template <typename R, int N, int M, int W, bool INV>
+__global__ void __launch_bounds__(W, 1) k_vec_down(const Params<R> P) {
+    griddep_launch_dependents();
+    griddep_wait();
+    using V = VecSmem<R, N, M, W>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
+    R* tree = reinterpret_cast<R*>(smem_raw + kSmemHead);
+    R* xs = tree + V::XS;
+    R* sm = tree + V::MODEL;
+    const unsigned tile = blockIdx.x, mirror = P.tiles - 1 - tile;
+    const int tid = threadIdx.x;
+    if (tid == 0) mbar_init(bar, 1);
+    model_prologue<R, N, M>(P, sm);
+    uint32_t phase = 0;
+    const bool ok_load = cta_bulk_load(tree, P.tree + (size_t)mirror * Dims<N>::ELEM * V::WS,
+                                       (uint32_t)(Dims<N>::AFFINE * V::WS * sizeof(R)), bar, phase,
+                                       P.wait_limit);
+    const TileGeo geo{P.T, (long long)tile * W, P.B};
+    if (tid < N)
+        xs[tid * V::WS + tslot<R>(next_pow2(geo.live(W)) - 1)] =
+            P.tile_carry[(size_t)mirror * N + tid];
+    __syncthreads();
+    vec_down_body<R, N, M, W, false, INV>(P, tile, tree, xs, sm);
+    if (!ok_load) set_status(P.status, ST_TIMEOUT);
+}
+
+// ===========================================================================
 // solo: a problem of one tile in one CTA -- the pass's up-sweep, value
 // down-sweep with the Riccati re-folds, forward up-sweep and rollout back to
 // back (the bodies above with SOLO), the trees kept in shared memory between
@@ -1446,6 +1699,33 @@ __global__ void __launch_bounds__(W, 1) k_solo(const Params<R> P) {
     bwd_up_body<R, N, M, W, true, INV>(P, 0, big, sm);
     __syncthreads();
     bwd_down_body<R, N, M, W, true, INV>(P, 0, smem_raw, big + BIG + threadIdx.x, sm);
+    __syncthreads();
+    fwd_down_body<R, N, M, W, true, INV>(P, 0, smem_raw, sm);
+}
+
+// The second pass of a one-tile problem: the vector recursions and the rollout.
+template <typename R, int N, int M, int W, bool INV>
+__global__ void __launch_bounds__(W, 1) k_solo_vec(const Params<R> P) {
+    griddep_launch_dependents();
+    griddep_wait();
+    using SM = Smem<R, N, M, W>;
+    using V = VecSmem<R, N, M, W>;
+    constexpr int BIG = SoloSmem<R, N, M, W>::BIG;
+    static_assert(V::MODEL <= BIG, "the value tree fits the common area");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    R* big = reinterpret_cast<R*>(smem_raw + kSmemHead);
+    R* sm = big + BIG + SM::RBUF;
+    R* xs = big + V::XS;
+    model_prologue<R, N, M>(P, sm);  // ends with __syncthreads
+    const TileGeo geo{P.T, 0, P.B};
+    if (threadIdx.x == W - 1) {
+        Value<R, N> z;
+        terminal_value<R, N>(P, z);
+#pragma unroll
+        for (int i = 0; i < N; ++i) xs[i * V::WS + tslot<R>(next_pow2(geo.live(W)) - 1)] = z.v[i];
+    }
+    vec_up_body<R, N, M, W, true, INV>(P, 0, big, sm);
+    vec_down_body<R, N, M, W, true, INV>(P, 0, big, xs, sm);
     __syncthreads();
     fwd_down_body<R, N, M, W, true, INV>(P, 0, smem_raw, sm);
 }

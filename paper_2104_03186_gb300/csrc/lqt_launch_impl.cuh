@@ -55,7 +55,7 @@ static lqt_status launch_solve_inv(const Params<R>& P, const Plan& plan, cudaStr
     constexpr int W = tile_threads<R, N, M>();
     constexpr int TP = top_threads();
     using SM = Smem<R, N, M, W>;
-    static std::atomic<bool> done_up[64], done_top[64], done_top1[64], done_top2[64], done_down[64],
+    static std::atomic<bool> done_up[64], done_top[64], done_down[64],
         done_ftop[64], done_fdown[64], done_solo[64];
     if (plan.solo) {
         // one tile: the whole pass in one CTA
@@ -63,58 +63,82 @@ static lqt_status launch_solve_inv(const Params<R>& P, const Plan& plan, cudaStr
         if (plan.tiles != 1 || allow_smem(k_solo<R, N, M, W, INV>, done_solo, smem) != cudaSuccess)
             return plan.tiles != 1 ? LQT_EINVAL : LQT_ECUDA;
         prof_mark(prof, stream, P.refine_add ? "solo.refine" : "solo");
-        if (launch_pdl<R>(k_solo<R, N, M, W, INV>, 1, W, smem, stream, P, true) != cudaSuccess)
+        static std::atomic<bool> done_svec[64];
+        if (P.vector_pass &&
+            allow_smem(k_solo_vec<R, N, M, W, INV>, done_svec, smem) != cudaSuccess)
+            return LQT_ECUDA;
+        if (launch_pdl<R>(P.vector_pass ? k_solo_vec<R, N, M, W, INV> : k_solo<R, N, M, W, INV>, 1,
+                          W, smem, stream, P, true) != cudaSuccess)
             return LQT_ECUDA;
         if (bwd_done && cudaEventRecord(bwd_done, stream) != cudaSuccess) return LQT_ECUDA;
         return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;
     }
+    if (P.vector_pass) {
+        // the second pass of a refined solve (tiles > 0)
+        static std::atomic<bool> dv_up[64], dv_top[64], dv_down[64], dv_ftop[64], dv_fdown[64];
+        const size_t sv = VecSmem<R, N, M, W>::bytes(P.p);
+        const size_t st = (size_t)(Dims<N>::AFFINE + N) * tstride(TP, (int)sizeof(R)) * sizeof(R);
+        const size_t sf = SM::bytes(SM::FDOWN_BIG, P.p);
+        if (allow_smem(k_vec_up<R, N, M, W, INV>, dv_up, sv) != cudaSuccess ||
+            allow_smem(k_fwd_top<R, N, TP, true>, dv_top, st) != cudaSuccess ||
+            allow_smem(k_vec_down<R, N, M, W, INV>, dv_down, sv) != cudaSuccess ||
+            allow_smem(k_fwd_top<R, N, TP, false>, dv_ftop, st) != cudaSuccess ||
+            allow_smem(k_fwd_down<R, N, M, W, INV>, dv_fdown, sf) != cudaSuccess)
+            return LQT_ECUDA;
+        const bool pdl = plan.B <= kPdlMaxChunk;
+        const int tiles = plan.tiles;
+        prof_mark(prof, stream, "bwd_up.refine");
+        if (launch_pdl<R>(k_vec_up<R, N, M, W, INV>, tiles, W, sv, stream, P, pdl) != cudaSuccess)
+            return LQT_ECUDA;
+        prof_mark(prof, stream, "bwd_top.refine");
+        if (launch_pdl<R>(k_fwd_top<R, N, TP, true>, 1, TP, st, stream, P, pdl) != cudaSuccess)
+            return LQT_ECUDA;
+        prof_mark(prof, stream, "bwd_down.refine");
+        if (launch_pdl<R>(k_vec_down<R, N, M, W, INV>, tiles, W, sv, stream, P, pdl) != cudaSuccess)
+            return LQT_ECUDA;
+        prof_mark(prof, stream, "fwd_top.refine");
+        if (launch_pdl<R>(k_fwd_top<R, N, TP, false>, 1, TP, st, stream, P, pdl) != cudaSuccess)
+            return LQT_ECUDA;
+        prof_mark(prof, stream, "fwd_down.refine");
+        if (launch_pdl<R>(k_fwd_down<R, N, M, W, INV>, tiles, W, sf, stream, P, pdl) != cudaSuccess)
+            return LQT_ECUDA;
+        return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;
+    }
     const size_t smem_up = SM::bytes(SM::UP_BIG, P.p);
-    constexpr long long kTopReplay =
-        top_smem_bytes(Dims<N>::ELEM, Dims<N>::VALUE, N, TP, (int)sizeof(R), true);
-    const size_t smem_top_full = (size_t)top_smem_bytes(Dims<N>::ELEM, Dims<N>::VALUE, N, TP,
-                                                        (int)sizeof(R), false);
-    const size_t smem_top_max = kTopReplay <= kTopSmemMax ? (size_t)kTopReplay : smem_top_full;
-    const size_t smem_top = P.top_mode == 2 ? (size_t)kTopReplay : smem_top_full;
-    // recording and replay need one tile per top-scan thread (layout() only
-    // reserves the factor store then); k_bwd_top re-checks
-    if (smem_top > smem_top_max || (P.top_mode != 0 && plan.tiles > TP)) return LQT_EINVAL;
+    const size_t smem_top = (size_t)top_smem_bytes(Dims<N>::ELEM, Dims<N>::VALUE, N, TP,
+                                                   (int)sizeof(R), false);
     const size_t smem_down = SM::bytes(SM::DOWN_BIG, P.p);
     const size_t smem_ftop = (size_t)(Dims<N>::AFFINE + N) * tstride(TP, (int)sizeof(R)) * sizeof(R);
     const size_t smem_fdown = SM::bytes(SM::FDOWN_BIG, P.p);
     cudaError_t err;
     if ((err = allow_smem(k_bwd_up<R, N, M, W, INV>, done_up, smem_up)) != cudaSuccess ||
-        (err = allow_smem(k_bwd_top<R, N, TP, 0>, done_top, smem_top_full)) != cudaSuccess ||
-        (err = allow_smem(k_bwd_top<R, N, TP, 1>, done_top1, smem_top_full)) != cudaSuccess ||
-        (err = allow_smem(k_bwd_top<R, N, TP, 2>, done_top2, smem_top_max)) != cudaSuccess ||
+        (err = allow_smem(k_bwd_top<R, N, TP>, done_top, smem_top)) != cudaSuccess ||
         (err = allow_smem(k_bwd_down<R, N, M, W, INV>, done_down, smem_down)) != cudaSuccess ||
-        (err = allow_smem(k_fwd_top<R, N, TP>, done_ftop, smem_ftop)) != cudaSuccess ||
+        (err = allow_smem(k_fwd_top<R, N, TP, false>, done_ftop, smem_ftop)) != cudaSuccess ||
         (err = allow_smem(k_fwd_down<R, N, M, W, INV>, done_fdown, smem_fdown)) != cudaSuccess)
         return LQT_ECUDA;
     const int tiles = plan.tiles;
     const bool pdl = plan.B <= kPdlMaxChunk;
     if (tiles > 0) {
-        prof_mark(prof, stream, P.refine_add ? "bwd_up.refine" : "bwd_up");
+        prof_mark(prof, stream, "bwd_up");
         err = launch_pdl<R>(k_bwd_up<R, N, M, W, INV>, tiles, W, smem_up, stream, P, pdl);
         if (err != cudaSuccess) return LQT_ECUDA;
     }
-    prof_mark(prof, stream, P.refine_add ? "bwd_top.refine" : "bwd_top");
-    err = launch_pdl<R>(P.top_mode == 2   ? k_bwd_top<R, N, TP, 2>
-                        : P.top_mode == 1 ? k_bwd_top<R, N, TP, 1>
-                                          : k_bwd_top<R, N, TP, 0>,
-                        1, TP, smem_top, stream, P, pdl);
+    prof_mark(prof, stream, "bwd_top");
+    err = launch_pdl<R>(k_bwd_top<R, N, TP>, 1, TP, smem_top, stream, P, pdl);
     if (err != cudaSuccess) return LQT_ECUDA;
     if (tiles > 0) {
-        prof_mark(prof, stream, P.refine_add ? "bwd_down.refine" : "bwd_down");
+        prof_mark(prof, stream, "bwd_down");
         err = launch_pdl<R>(k_bwd_down<R, N, M, W, INV>, tiles, W, smem_down, stream, P, pdl);
         if (err != cudaSuccess) return LQT_ECUDA;
     }
     // S, v and K are final here (a second refinement pass does not write them)
     if (bwd_done && cudaEventRecord(bwd_done, stream) != cudaSuccess) return LQT_ECUDA;
-    prof_mark(prof, stream, P.refine_add ? "fwd_top.refine" : "fwd_top");
-    err = launch_pdl<R>(k_fwd_top<R, N, TP>, 1, TP, smem_ftop, stream, P, pdl);
+    prof_mark(prof, stream, "fwd_top");
+    err = launch_pdl<R>(k_fwd_top<R, N, TP, false>, 1, TP, smem_ftop, stream, P, pdl);
     if (err != cudaSuccess) return LQT_ECUDA;
     if (tiles > 0) {
-        prof_mark(prof, stream, P.refine_add ? "fwd_down.refine" : "fwd_down");
+        prof_mark(prof, stream, "fwd_down");
         err = launch_pdl<R>(k_fwd_down<R, N, M, W, INV>, tiles, W, smem_fdown, stream, P, pdl);
         if (err != cudaSuccess) return LQT_ECUDA;
     }

@@ -1,12 +1,13 @@
 // lqt_solve_static: the parallel solve with its scratch space in one array
 // compiled into the library, for callers that cannot allocate device memory
-// (see include/lqt.h).  It reuses lqt_solve unchanged and only supplies the
-// array as the workspace.
+// (see include/lqt.h).  It reuses lqt_solve and only supplies the array as the
+// workspace.
 #include <cuda_runtime.h>
 
 #include <mutex>
 
 #include "lqt.h"
+#include "lqt_chain_api.h"
 
 namespace {
 
@@ -44,13 +45,18 @@ extern "C" lqt_status lqt_solve_static(const lqt_problem* prob, const lqt_soluti
         // same diagnosis as lqt_solve for invalid or unsupported problems
         return lqt_solve(prob, sol, opts, nullptr, 0, stream);
     }
-    if (need > LQT_STATIC_SCRATCH_BYTES) return LQT_ENOMEM;
+    // a problem whose usual workspace does not fit may fit the least one (a
+    // refined solve at n >= 8 then keeps nothing for its correction pass)
+    const bool lean = need > LQT_STATIC_SCRATCH_BYTES;
+    if (lean && lqt::workspace_bytes(prob, opts, true) > LQT_STATIC_SCRATCH_BYTES)
+        return LQT_ENOMEM;
     void* ws = nullptr;
     lqt_status st = scratch_address(&ws);
     if (st != LQT_OK) return st;
     // lqt_solve clears the status word at the start of the array; every other
     // region it uses is written before it is read within the same solve.
-    st = lqt_solve(prob, sol, opts, ws, LQT_STATIC_SCRATCH_BYTES, stream);
+    st = lean ? lqt::solve_lean(prob, sol, opts, ws, LQT_STATIC_SCRATCH_BYTES, stream)
+              : lqt_solve(prob, sol, opts, ws, LQT_STATIC_SCRATCH_BYTES, stream);
     if (st != LQT_OK) return st;
     return lqt_workspace_status(ws, stream);
 }
