@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <string.h>
 
@@ -106,6 +107,7 @@ struct Launcher {
     using VW = VWalk<N, M>;
     static constexpr int VFWD_B = VW::NT * VW::FWD_SIZE * (int)sizeof(R);
     static constexpr int VBACK_B = VW::NT * VW::BACK_SIZE * (int)sizeof(R);
+    static constexpr int VRESID_B = VResid<N, M>::NT * VResid<N, M>::SIZE * (int)sizeof(R);
     static constexpr int NG_FOLD = groups_for<N>(FOLD_B);
     static constexpr int NG_REFOLD = groups_for<N>(REFOLD_B);
     static constexpr int NG_UP = groups_for<N>(UP_B);
@@ -144,8 +146,9 @@ struct Launcher {
                 (e = chain_allow_smem(k_tfup<RT, N, TT>, d_fup, (size_t)TT * TFUP_B)) !=
                     cudaSuccess)
                 return e;
-            static std::atomic<bool> d_vf[64], d_vfm[64], d_vb[64], d_vbm[64];
-            if ((e = chain_allow_smem(k_vfwd<R, RT, N, M, false>, d_vf, VFWD_B)) != cudaSuccess ||
+            static std::atomic<bool> d_vf[64], d_vfm[64], d_vb[64], d_vbm[64], d_vr[64];
+            if ((e = chain_allow_smem(k_vresid<R, N, M>, d_vr, VRESID_B)) != cudaSuccess ||
+                (e = chain_allow_smem(k_vfwd<R, RT, N, M, false>, d_vf, VFWD_B)) != cudaSuccess ||
                 (e = chain_allow_smem(k_vfwd<R, RT, N, M, true>, d_vfm, VFWD_B)) != cudaSuccess ||
                 (e = chain_allow_smem(k_vback<R, RT, N, M, false>, d_vb, VBACK_B)) !=
                     cudaSuccess ||
@@ -172,9 +175,11 @@ struct Launcher {
             (e = chain_allow_smem(k_m2roll<R, RT, N, M, NG_M2>, d_m2roll, (size_t)NG_M2 * M2_B)) !=
                 cudaSuccess)
             return e;
-        if ((e = chain_allow_smem(k_cresid<R, N, M, NG_RESID>, d_resid,
-                                  (size_t)NG_RESID * RESID_B)) != cudaSuccess)
-            return e;
+        if constexpr (!kTeam) {
+            if ((e = chain_allow_smem(k_cresid<R, N, M, NG_RESID>, d_resid,
+                                      (size_t)NG_RESID * RESID_B)) != cudaSuccess)
+                return e;
+        }
         if constexpr (kCompNewton) {
             static std::atomic<bool> d_nres_c[64], d_ngain_c[64];
             if ((e = chain_allow_smem(k_nresid_c<N, M, NG_NEWTON_C>, d_nres_c,
@@ -814,8 +819,20 @@ struct Launcher {
             prof_mark(prof, s, "chain_resid");
             int grid = blocks(r0, NG_RESID);
             if (grid > 4096) grid = 4096;
-            k_cresid<R, N, M, NG_RESID><<<grid, NG_RESID * N, (size_t)NG_RESID * RESID_B, s>>>(
-                d1, d2, count, r0, a.status);
+            if constexpr (kTeam) {
+                using VR = VResid<N, M>;
+                long long most = 0;
+                for (int q = 0; q < count; ++q)
+                    most = std::max(most, (long long)call.probs[q].problem->T);
+                const int run = resid_run(most);
+                k_vresid<R, N, M><<<dim3((unsigned)blocks((most + run - 1) / run, VR::NT),
+                                         (unsigned)count),
+                                    32 * VR::NT, VRESID_B, s>>>(d1, d2, run, a.status);
+            } else {
+                k_cresid<R, N, M, NG_RESID>
+                    <<<grid, NG_RESID * N, (size_t)NG_RESID * RESID_B, s>>>(d1, d2, count, r0,
+                                                                            a.status);
+            }
             Args<R, RT> b = a;
             b.items = d2;
             // the correction pass writes no S, v, K; with Method 2 its walk needs

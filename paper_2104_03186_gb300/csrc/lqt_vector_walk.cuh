@@ -289,5 +289,301 @@ __global__ void __launch_bounds__(N) k_vseed(Args<R, RT> a) {
         static_cast<RT>(VALUE ? it.D.etaT[threadIdx.x] : it.D.x0[threadIdx.x]);
 }
 
+// ---- KKT residuals of the first pass's iterate -------------------------------
+// k_cresid's residuals (lqt_chain.cuh: e_k, g_k, h_k and U^{-1} h_k, g_T) at the
+// team sizes, one warp per run of consecutive steps, walked from the last: lambda_{k+1} and x_{k+1} of a step are the step before's, so S_k is read
+// once instead of twice, and a ring of stages keeps the next step's matrices on
+// the way, where k_cresid waited for every step's loads (n = 32, T = 65536:
+// 853 -> 307 us).  The sums are compensated as there; blocks of a sum in
+// different lanes are merged by compensated additions.  A time-invariant U is
+// inverted once per run.  resid_run: the steps of a run, 16 where that leaves
+// 4096 warps, fewer down to 2 for shorter horizons (n = 16, T = 10007: runs of 16
+// took 52 us, of 2 24, k_cresid 37).
+inline int resid_run(long long T) {
+    const long long r = T / 4096;
+    return r > 16 ? 16 : r < 2 ? 2 : (int)r;
+}
+
+template <int N, int M>
+struct VResid {
+    static constexpr int r4(int x) { return (x + 3) / 4 * 4; }
+    // one stage: F, L, U, S_k, X_k (p = N) | x, u, v, c, r
+    static constexpr int F = 0, L = N * N, U = L + N * M, S = U + M * M, X = S + N * N,
+                         XV = X + N * N, UV = XV + N, VV = UV + M, CV = VV + N, RV = CV + N,
+                         STAGE = r4(RV + N);
+    static constexpr int ST = 2;
+    static constexpr int NT = N == 32 ? 1 : 4;  // warps per CTA
+    // vectors: lambda_{k+1}, x_{k+1}, H x - r and X (H x - r) as (hi, lo), U^{-1} h
+    static constexpr int L1 = ST * STAGE, X1 = L1 + N, HH = X1 + N, HL = HH + 2 * N,
+                         YH = HL + 2 * N, YL = YH + 2 * N, Q = YL + 2 * N, SIZE = r4(Q + M);
+};
+
+// Dot2 (or plain FP64) sums of a block each in the lanes of a row, merged over
+// lanes D apart, 2D apart, ... 16 apart
+template <int D, typename R>
+__device__ __forceinline__ void merge(XAcc<R>& a) {
+#pragma unroll
+    for (int d = D; d < 32; d <<= 1) {
+        if constexpr (sizeof(R) == 4) {
+            const float s = __shfl_xor_sync(0xffffffffu, a.d.s, d);
+            const float c = __shfl_xor_sync(0xffffffffu, a.d.c, d);
+            // the same operand order in both lanes keeps them identical
+            const bool low = ((threadIdx.x & 31) & d) == 0;
+            float t, e;
+            two_sum(low ? a.d.s : s, low ? s : a.d.s, t, e);
+            a.d.s = t;
+            a.d.c = add_rn(add_rn(a.d.c, c), e);
+        } else {
+            a.s += __shfl_xor_sync(0xffffffffu, a.s, d);
+        }
+    }
+}
+
+template <typename R, int N, int M>
+__global__ void __launch_bounds__(32 * VResid<N, M>::NT)
+    k_vresid(const Item<R>* items1, const Item<R>* items2, int steps, int* status) {
+    using W = VResid<N, M>;
+    using VL = VLane<N, M>;
+    using A = XAcc<R>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    R* sh = reinterpret_cast<R*>(smem_raw) + (threadIdx.x / 32) * W::SIZE;
+    const VL l;
+    const DescT<R>& D = items1[blockIdx.y].D;
+    const DescT<R>& D2 = items2[blockIdx.y].D;
+    R* const qh = const_cast<R*>(items2[blockIdx.y].qh);
+    R* const eta = const_cast<R*>(D2.eta);
+    R* const ctil = const_cast<R*>(D2.c);
+    const long long T = D.T;
+    const long long run = (long long)blockIdx.x * W::NT + threadIdx.x / 32;
+    const long long s = run * steps, e = s + steps < T ? s + steps : T;
+    if (s >= T) return;
+    R *lam1 = sh + W::L1, *x1 = sh + W::X1, *hh = sh + W::HH, *hl = sh + W::HL, *yh = sh + W::YH,
+      *yl = sh + W::YL, *qv = sh + W::Q;
+    const int p = D.p;
+    const R *F = D.F, *L = D.L, *U = D.U, *H = D.H, *X = D.X, *rp = D.r, *cp = D.c, *S = D.S;
+    const long long sF = D.sF, sL = D.sL, sU = D.sU, sH = D.sH, sX = D.sX, sr = D.sr, sc = D.sc;
+    const bool vF = vec_ok(F, sF), vL = vec_ok(L, sL), vU = vec_ok(U, sU), vS = vec_ok(S, 0),
+               vX = vec_ok(X, sX);
+    bool hid = sH == 0 && p == N;
+    if (hid)
+        for (int t = l.lane; t < N * N; t += 32)
+            hid = hid && H[t] == (t / N == t % N ? R(1) : R(0));
+    hid = __all_sync(0xffffffffu, hid);
+    auto stage = [&](long long k) {
+        if (k >= s) {
+            R* b = sh + (int)((e - 1 - k) % W::ST) * W::STAGE;
+            warp_cp_mat<N, N>(b + W::F, F + k * sF, vF, l.lane);
+            warp_cp_mat<N, M>(b + W::L, L + k * sL, vL, l.lane);
+            if (sU != 0 || k == e - 1) warp_cp_mat<M, M>(b + W::U, U + k * sU, vU, l.lane);
+            warp_cp_mat<N, N>(b + W::S, S + k * (N * N), vS, l.lane);
+            if (p == N) warp_cp_mat<N, N>(b + W::X, X + k * sX, vX, l.lane);
+            if (l.h == 0) {
+                cp_async<sizeof(R)>(b + W::XV + l.j, D.x + k * N + l.j);
+                cp_async<sizeof(R)>(b + W::VV + l.j, D.v + k * N + l.j);
+                if (cp) cp_async<sizeof(R)>(b + W::CV + l.j, cp + k * sc + l.j);
+                if (p == N && rp) cp_async<sizeof(R)>(b + W::RV + l.j, rp + k * sr + l.j);
+            }
+            if (l.ha == 0) cp_async<sizeof(R)>(b + W::UV + l.a, D.u + k * M + l.a);
+        }
+        cp_async_commit();
+    };
+    stage(e - 1);
+    // lambda_e = S_e x_e - v_e and x_e; the last run also the terminal condition
+    {
+        const R xe = D.x[e * N + l.j];
+        if (l.h == 0) x1[l.j] = xe;
+        __syncwarp();
+        R t = R(0);
+        for (int i = l.h * VL::BN; i < (l.h + 1) * VL::BN; ++i)
+            t = team::fma_(S[e * (N * N) + i * N + l.j], x1[i], t);
+        const R lam = l.sum_n(t) - D.v[e * N + l.j];
+        if (l.h == 0) lam1[l.j] = lam;
+        __syncwarp();
+        if (e == T) {
+            for (int i = l.lane; i < D.pT; i += 32) {
+                A h(D.rT ? -D.rT[i] : R(0));
+                for (int j = 0; j < N; ++j) h.add_prod(D.HT[i * N + j], x1[j]);
+                h.split(hh[i], hl[i]);
+            }
+            __syncwarp();
+            for (int i = l.lane; i < D.pT; i += 32) {
+                A t2(R(0));
+                for (int b = 0; b < D.pT; ++b) t2.add_prod2(D.XT[i * D.pT + b], hh[b], hl[b]);
+                t2.split(yh[i], yl[i]);
+            }
+            __syncwarp();
+            if (l.h == 0) {
+                A g(-lam1[l.j]);
+                for (int i = 0; i < D.pT; ++i) g.add_prod2(D.HT[i * N + l.j], yh[i], yl[i]);
+                const_cast<R*>(D2.etaT)[l.j] = -g.value();
+                const_cast<R*>(D2.x0)[l.j] = R(0);
+            }
+            __syncwarp();
+        }
+    }
+    constexpr int EP = 16 / (int)sizeof(R), V = VL::BN < EP ? VL::BN : EP;
+    bool ok = true;
+    R ui[M];  // a time-invariant U: column a of U^{-1} in lane a < M
+    for (long long k = e - 1; k >= s; --k) {
+        cp_async_wait<0>();
+        __syncwarp();
+        stage(k - 1);
+        const R* b = sh + (int)((e - 1 - k) % W::ST) * W::STAGE;
+        // h's solve: U (lanes a < M, column a) eliminated once or with its right side
+        const bool invert = sU == 0 && k == e - 1;
+        const R *xv = b + W::XV, *uv = b + W::UV;
+        // H x^ - r as (hi, lo)
+        if (hid) {
+            if (l.h == 0) {
+                A h(xv[l.j]);
+                if (rp) h.add(-b[W::RV + l.j]);
+                h.split(hh[l.j], hl[l.j]);
+            }
+        } else {
+            const R* Hk = H + k * sH;
+            const R* rk = rp ? rp + k * sr : nullptr;
+            for (int i = l.lane; i < p; i += 32) {
+                A h(rk ? -rk[i] : R(0));
+                for (int j = 0; j < N; ++j) h.add_prod(Hk[i * N + j], xv[j]);
+                h.split(hh[i], hl[i]);
+            }
+        }
+        __syncwarp();
+        // y = X (H x^ - r) as (hi, lo)
+        if (p == N) {
+            A t;
+#pragma unroll
+            for (int q = 0; q < VL::BN; q += V) {
+                const int i = l.h * VL::BN + q;
+                R x[V];
+                ldrow<N, V>(b + W::X, l.j, i, x);
+#pragma unroll
+                for (int w = 0; w < V; ++w) t.add_prod2(x[w], hh[i + w], hl[i + w]);
+            }
+            merge<N>(t);
+            if (l.h == 0) t.split(yh[l.j], yl[l.j]);
+        } else {
+            const R* Xk = X + k * sX;
+            for (int i = l.lane; i < p; i += 32) {
+                A t;
+                for (int q = 0; q < p; ++q) t.add_prod2(Xk[i * p + q], hh[q], hl[q]);
+                t.split(yh[i], yl[i]);
+            }
+        }
+        __syncwarp();
+        // lambda_k in the working precision (any iterate's exact residuals do)
+        const R lam =
+            l.sum_n(col_dot<VL::BN, N>(b + W::S, xv, l.h * VL::BN, l.j)) - b[W::VV + l.j];
+        // g = H^T y - lambda_k + F^T lambda_{k+1}
+        A g(l.h == 0 ? -lam : R(0));
+        if (hid) {
+            if (l.h == 0) {
+                g.add(yh[l.j]);
+                g.add(yl[l.j]);
+            }
+        } else {
+            const R* Hk = H + k * sH;
+            for (int i = l.h; i < p; i += VL::G) g.add_prod2(Hk[i * N + l.j], yh[i], yl[i]);
+        }
+#pragma unroll
+        for (int q = 0; q < VL::BN; ++q) {
+            const int i = l.h * VL::BN + q;
+            g.add_prod(b[W::F + Sw<R, N>::at(i, l.j)], lam1[i]);
+        }
+        merge<N>(g);
+        // h = U u^ + L^T lambda_{k+1}
+        const R* Uk = sU == 0 ? sh + W::U : b + W::U;  // an invariant U stays in slot 0
+        A hr;
+#pragma unroll
+        for (int q = 0; q < VL::BMM; ++q) {
+            const int i = l.ha * VL::BMM + q;
+            if (i < M) hr.add_prod(Uk[Sw<R, M>::at(l.a, i)], uv[i]);
+        }
+#pragma unroll
+        for (int q = 0; q < VL::BNM; ++q) {
+            const int i = l.ha * VL::BNM + q;
+            hr.add_prod(b[W::L + Sw<R, M>::at(i, l.a)], lam1[i]);
+        }
+        merge<M>(hr);
+        const R h = hr.value();
+        // U^{-1} h in the working precision (h is the residual itself)
+        R qa;
+        if (sU != 0 || invert) {
+            // column a of [U | h] per lane (lane M: h), Gauss-Jordan without
+            // pivoting; an invariant U's columns become those of U^{-1}
+            R col[M];
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const R hi = __shfl_sync(0xffffffffu, h, i);
+                col[i] = l.lane < M ? Uk[Sw<R, M>::at(l.a, i)] : hi;
+            }
+#pragma unroll
+            for (int q = 0; q < M; ++q) {
+                const R piv = __shfl_sync(0xffffffffu, col[q], q);
+                ok = ok && piv > R(0) && isfinite(piv);
+                const R inv = rcp(piv);
+                const bool own = invert && l.lane == q;
+                const R pk = own ? inv : col[q] * inv;
+#pragma unroll
+                for (int i = 0; i < M; ++i) {
+                    if (i == q) continue;
+                    const R f = __shfl_sync(0xffffffffu, col[i], q);
+                    col[i] = team::fma_(-f, pk, own ? R(0) : col[i]);
+                }
+                col[q] = pk;
+            }
+            qa = R(0);
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const R t = __shfl_sync(0xffffffffu, col[i], M);  // lane M's solution
+                if (l.a == i) qa = t;
+                ui[i] = col[i];
+            }
+        } else {
+            qa = R(0);
+#pragma unroll
+            for (int i = 0; i < M; ++i)  // U^{-1} symmetric: row a is lane a's column
+                qa = team::fma_(__shfl_sync(0xffffffffu, ui[i], l.a), __shfl_sync(0xffffffffu, h, i),
+                                qa);
+        }
+        if (l.ha == 0) {
+            qv[l.a] = qa;
+            qh[k * M + l.a] = qa;
+        }
+        __syncwarp();
+        // e = F x^ + c + L (u^ - U^{-1} h) - x^_{k+1}
+        A er(l.h == 0 && cp ? b[W::CV + l.j] : R(0));
+        if (l.h == 0) er.add(-x1[l.j]);
+#pragma unroll
+        for (int q = 0; q < VL::BN; q += V) {
+            const int i = l.h * VL::BN + q;
+            R f[V];
+            ldrow<N, V>(b + W::F, l.j, i, f);
+#pragma unroll
+            for (int w = 0; w < V; ++w) er.add_prod(f[w], xv[i + w]);
+        }
+#pragma unroll
+        for (int q = 0; q < VL::BM; ++q) {
+            const int i = l.h * VL::BM + q;
+            if (i < M) {
+                const R lv = b[W::L + Sw<R, M>::at(l.j, i)];
+                er.add_prod(lv, uv[i]);
+                er.add_prod(-lv, qv[i]);
+            }
+        }
+        merge<N>(er);
+        __syncwarp();  // lam1 and x1 are read
+        if (l.h == 0) {
+            eta[k * N + l.j] = -g.value();
+            ctil[k * N + l.j] = er.value();
+            lam1[l.j] = lam;
+            x1[l.j] = xv[l.j];
+        }
+        __syncwarp();
+    }
+    cp_async_wait<0>();
+    flag(status, ok);
+}
+
 }  // namespace chain
 }  // namespace lqt
