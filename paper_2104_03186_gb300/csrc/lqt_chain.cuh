@@ -2,31 +2,33 @@
 // (lqt_solve) or a ragged batch of problems of one (n, m) (lqt_solve_batched).
 //
 // Problem i's T_i steps are cut into NC_i chunks (NC_i a power of two) of B_i
-// steps; one lane group of N lanes (lane r owns row r) works on one chunk at a
-// time, and the scans over the chunk results run level by level, one launch
-// per level, with the chunk results in global memory.  The problems are laid
-// out by decreasing NC_i, problem i's chunks at [c0_i, c0_i + NC_i), so every
-// c0_i is a multiple of NC_i: at tree level h the pairs of all problems with
-// NC_i >= 2h are the pairs (i, i + h), i a multiple of 2h, of one prefix of the
-// chunk array, and the level kernels need no per-problem lookup.  Per pass:
-//   k_cfold    chunk totals a_s (x) ... (x) a_{e-1} (eq. lqt_comb), folded one
+// steps; one team of lanes works on one chunk at a time, and the scans over the
+// chunk results run over tree levels with the chunk results in global memory.
+// The problems are laid out by decreasing NC_i, problem i's chunks at
+// [c0_i, c0_i + NC_i), so every c0_i is a multiple of NC_i: at tree level h the
+// pairs of all problems with NC_i >= 2h are the pairs (i, i + h), i a multiple of
+// 2h, of one prefix of the chunk array, and the level kernels need no per-problem
+// lookup.  Per pass (n >= 8, lqt_team_chain.cuh; k_c* of this file at n = 4, a
+// lane group of N lanes per chunk and a launch per level):
+//   k_tfold    chunk totals a_s (x) ... (x) a_{e-1} (eq. lqt_comb), folded one
 //              step at a time from the end in the low-rank form of fold_step,
-//   k_cup      up-sweep levels of the chunk totals (Alg. 1, left-anchored),
+//   k_tup      up-sweep levels of the chunk totals (Alg. 1, left-anchored),
 //   k_cterm    the terminal value (H_T^T X_T r_T, H_T^T X_T H_T),
-//   k_cdown    down-sweep levels of the value carries (Lemma LQT_assoc: a
+//   k_tdown    down-sweep levels of the value carries (Lemma LQT_assoc: a
 //              suffix applied to the value element (0, 0, 0, v, S)),
-//   k_crefold  per chunk the Riccati recursion from its carry (Sec. II-B),
+//   k_trefold  per chunk the Riccati recursion from its carry (Sec. II-B),
 //              writing S_k, v_k, K_k and the feedforward d_k, and the chunk's
 //              closed-loop affine map (Sec. IV-C),
-//   k_cfup / k_cfdown  up- and down-sweeps of the affine maps from x_0
+//   k_tfup / k_tfdown  up- and down-sweeps of the affine maps from x_0
 //              (right-anchored), giving every chunk's start state,
-//   k_croll    per chunk the rollout of x*_k and u*_k (eq. Control_LQT).
+//   k_vfwd     per chunk the rollout of x*_k and u*_k (eq. Control_LQT,
+//              lqt_vector_walk.cuh).
 // The chunk phases compute in R; the tree levels store and compute in RT
 // (RT = double with R = float is the mixed-precision form: FP32 chunk work,
 // FP64 tree levels and their (I + C J) solves).
 //
 // Refinement (one step of iterative refinement of the KKT system of the QP):
-// k_cresid evaluates, in twice the working precision (FP64 arithmetic, or
+// k_vresid (n = 4: k_cresid) evaluates, in twice the working precision (FP64 arithmetic, or
 // compensated FP32 dot products for FP32 problems), the residuals of the
 // optimality conditions at
 // the first pass's iterate (x^, u^, lambda^ with lambda^_k = S_k x^_k - v_k,
@@ -39,9 +41,10 @@
 // 1/2 du^T U du + h^T du subject to dx_{k+1} = F dx_k + L du_k + e_k, dx_0 = 0.
 // With du = w - U^{-1} h this is the LQT problem of Sec. II-B with linear
 // state terms eta_k = -g_k, eta_T = -g_T (no reference), offsets
-// c~_k = e_k - L U^{-1} h_k and control w; the second pass solves it with the
-// same kernels (its S and K equal the first pass's) and adds
-// x = x^ + dx, u = u^ + w - U^{-1} h.
+// c~_k = e_k - L U^{-1} h_k and control w.  Its S and K equal the first pass's:
+// at n >= 8 the second pass is vector walks and affine scans (k_vback, k_vfwd),
+// otherwise (n = 4, Method 2, the sequential recursion, the least workspace) the
+// same kernels again; it adds x = x^ + dx, u = u^ + w - U^{-1} h.
 #pragma once
 
 #include <cuda_runtime.h>

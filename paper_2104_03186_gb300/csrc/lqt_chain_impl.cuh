@@ -216,10 +216,10 @@ struct Launcher {
     // block, as many CTAs as are co-resident (at most one team per chunk).
     static constexpr int PERSIST_B = kTeam ? persist_team_bytes<R, RT, N, M>() : 16;
     static constexpr int NT_PERSIST = 256 / LG;
-    // variants whose teams do not fit one SM (FP64 at n = 32 and FP64 trees)
-    // always take the per-level launches
+    // (batches are FP32)
     static constexpr bool kPersistFits =
-        kTeam && (long long)NT_PERSIST * PERSIST_B <= 227 * 1024 - 1024;
+        kTeam && sizeof(R) == 4 && sizeof(RT) == 4 &&
+        (long long)NT_PERSIST * PERSIST_B <= 227 * 1024 - 1024;
 
     static lqt_status run_persistent(const Args<R, RT>& a, const long long* active, int levels,
                                      GridBarrier* bar, cudaStream_t s) {
