@@ -243,10 +243,10 @@ lqt_status lqt_solve_host(const lqt_problem *host_prob, const lqt_solution *host
  * `items` reach the workspace as kernel parameters, so the call never waits
  * for the stream, and it may be captured in a CUDA graph (the graph keeps the
  * descriptors; replays solve the same problems, reading whatever their input
- * buffers hold then).  A batch of at least 2^20 steps in all runs its lane
- * sizes side by side on streams of the calling host thread (created on its
- * first such call on a device and kept until the process exits: make that
- * first call before any stream capture), forked from and joined back to
+ * buffers hold then).  A batch of two or more sizes and at least 1024 steps in
+ * all runs its lane sizes side by side on streams of the calling host thread
+ * (created on its first such call on a device, which may be a captured one, and
+ * handed to a later thread when it ends), forked from and joined back to
  * `stream` with events; the outputs are those of one stream, bit for bit.
  * Returns LQT_EINVAL, LQT_EUNSUPPORTED, LQT_ENOMEM or LQT_ECUDA on argument or
  * launch errors.  Work queued before a launch error stays queued, ordered
@@ -320,7 +320,9 @@ lqt_status lqt_batch_set_tuning(const lqt_batch_tune_entry *entries, int32_t cou
  *          aligned; its first word is the status word of
  *          lqt_workspace_status() (LQT_ENOTSPD when some
  *          L_k^T S_{k+1} L_k + U_k is not positive definite).
- * Asynchronous on `stream`; returns LQT_EINVAL, LQT_EUNSUPPORTED, LQT_ENOMEM
+ * Asynchronous on `stream`, the state sizes and types of a call side by side on
+ * auxiliary streams joined back to it, as in lqt_solve_batched; it may be
+ * captured in a CUDA graph.  Returns LQT_EINVAL, LQT_EUNSUPPORTED, LQT_ENOMEM
  * or LQT_ECUDA on argument or launch errors.  The result equals that of a
  * full solve of the same problem up to rounding when the given S and K are
  * that problem's. */

@@ -199,7 +199,7 @@ extern "C" lqt_status lqt_solve_batched(const lqt_batch_item* items, int32_t cou
     ForkSet* aux = nullptr;
     if (lanes_running >= 1 && lanes_running <= kForkStreams &&
         lanes_running + (descs.empty() ? 0 : 1) >= 2 && total_steps >= kForkSteps)
-        aux = next_fork_set();
+        aux = next_fork_set(s);
     if (aux && cudaEventRecord(aux->fork, s) != cudaSuccess) return LQT_ECUDA;
     if (!descs.empty()) {
         // through kernel parameters (lqt_upload.cuh): a pageable copy would

@@ -291,9 +291,10 @@ __global__ void __launch_bounds__(N) k_vseed(Args<R, RT> a) {
 
 // ---- KKT residuals of the first pass's iterate -------------------------------
 // k_cresid's residuals (lqt_chain.cuh: e_k, g_k, h_k and U^{-1} h_k, g_T) at the
-// team sizes, one warp per run of consecutive steps, walked from the last: lambda_{k+1} and x_{k+1} of a step are the step before's, so S_k is read
-// once instead of twice, and a ring of stages keeps the next step's matrices on
-// the way, where k_cresid waited for every step's loads (n = 32, T = 65536:
+// team sizes, one warp per run of consecutive steps, walked from the last:
+// lambda_{k+1} and x_{k+1} of a step are the step before's, so S_k is read once
+// instead of twice, and a ring of stages keeps the next step's matrices on the
+// way, where k_cresid waited for every step's loads (n = 32, T = 65536:
 // 853 -> 307 us).  The sums are compensated as there; blocks of a sum in
 // different lanes are merged by compensated additions.  A time-invariant U is
 // inverted once per run.  resid_run: the steps of a run, 16 where that leaves

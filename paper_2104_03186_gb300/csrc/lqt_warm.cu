@@ -105,7 +105,7 @@ extern "C" lqt_status lqt_solve_warm(const lqt_batch_item* items, int32_t count,
     if (cudaMemsetAsync(base, 0, sizeof(int), s) != cudaSuccess) return LQT_ECUDA;
     char* ws = base + up(256);
     const std::vector<std::vector<int>> groups = warm_groups(items, count);
-    ForkSet* aux = groups.size() > 1 ? next_fork_set() : nullptr;
+    ForkSet* aux = groups.size() > 1 ? next_fork_set(s) : nullptr;
     if (aux && cudaEventRecord(aux->fork, s) != cudaSuccess) return LQT_ECUDA;
     // the auxiliary streams in use rejoin the caller's stream on every return
     // (their work uses the workspace, and a capture must end joined)

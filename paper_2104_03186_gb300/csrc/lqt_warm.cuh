@@ -15,12 +15,13 @@
 //   k_wfold    per chunk [s, e), walking back from v_e: the map
 //              v_s = Psi v_e + beta with Psi = Ft_s^T ... Ft_{e-1}^T, stored at
 //              the chunk's mirrored slot so that the forward scan kernels
-//              (k_cfup, k_cfdown) compose the maps from the last chunk to the
+//              (k_tfup, k_tfdown) compose the maps from the last chunk to the
 //              first, seeded with v_T (k_wterm);
 //   k_wrefold  per chunk, from its v_e: v_k and d_k step by step, then the
 //              chunk's forward map x_e = Psi^T x_s + gamma (Psi^T = Ft_{e-1}
 //              ... Ft_s is the closed-loop chunk map) by a rollout from 0;
-//   k_wseed    x_0 into the top slot; the forward scan and k_croll follow.
+//   k_wseed    x_0 into the top slot; the forward scan and the rollout follow
+//              (n >= 8: k_tfup, k_tfdown, k_vfwd; n = 4: k_cfup, k_cfdown, k_croll).
 // Per step this costs one n x n product (Psi) and the m x m solve for d_k,
 // against the two folds and the Riccati step of a full solve.
 #pragma once

@@ -9,8 +9,8 @@ is.  The tuner times lqt_solve_batched on this GPU on a synthetic batch shaped
 like the benchmark's ragged batch (diagonal tracking, m = n / 2), choosing the
 chunk length of each (n, T-bucket) in turn with the others fixed, then times
 the three launch modes (one launch per tree level, one persistent launch per
-size, or the library's automatic choice between them by the number of chunk
-waves) with that table on the whole batch and on a small batch of the size a
+size, or the automatic mode, which is the per-level launches) with that table
+on the whole batch and on a small batch of the size a
 server forms, and keeps the mode that is fastest on the small batch among
 those within 1% of the best on the whole batch.  The library applies a tuned
 length only up to the batch's total steps over the resident lane groups, so

@@ -132,3 +132,57 @@ def test_batch_and_warm_sizes_side_by_side():
                 assert torch.equal(a[k], b[k]), (p.n, p.T, k)
             compare({k: v.double().cpu().numpy() for k, v in w.items()}, oracle_solve(p),
                     FP32_TOL, names=("v", "x", "u"))
+
+
+def test_first_forked_call_of_a_thread_may_be_captured():
+    """A new thread's first batch and warm calls inside a capture; then the same
+    from a second thread, which takes over the first one's streams, with an
+    eager call made while a capture holds some of them."""
+    import threading
+
+    import torch
+
+    from paper_2104_03186_gb300 import lqt
+
+    probs = [inputs.diag_tracking(n, T=600, seed=n).rounded_to(np.float32) for n in (4, 8, 16)]
+    Ps = [lqt.Problem.from_inputs(p) for p in probs]
+    want = lqt.solve_batched(Ps)
+    warm = lqt.solve_warm(Ps, want)
+    torch.cuda.synchronize()
+    errors = []
+
+    def run(eager_inside):
+        try:
+            outs = [P.allocate_outputs() for P in Ps]
+            other = [P.allocate_outputs() for P in Ps]
+            wout = [dict(P.allocate_outputs(), S=w["S"], K=w["K"]) for P, w in zip(Ps, want)]
+            nb = lqt.lqt_batch_workspace_bytes(Ps, outs)
+            ws, ws2 = (torch.zeros(nb, dtype=torch.uint8, device="cuda") for _ in range(2))
+            wws = torch.zeros(lqt.lqt_warm_workspace_bytes(Ps, wout), dtype=torch.uint8,
+                              device="cuda")
+            side, side2 = torch.cuda.Stream(), torch.cuda.Stream()
+            torch.cuda.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            mode = "thread_local" if not eager_inside else "relaxed"
+            with torch.cuda.graph(graph, stream=side, capture_error_mode=mode):
+                lqt.lqt_solve_batched(Ps, outs, ws, side)
+                for _ in range(5 if eager_inside else 0):
+                    lqt.lqt_solve_batched(Ps, other, ws2, side2)
+                lqt.lqt_solve_warm(Ps, wout, wws, side)
+            graph.replay()
+            torch.cuda.synchronize()
+            for o, e, a in zip(outs, want, other):
+                for k in e:
+                    assert torch.equal(o[k], e[k]), k
+                    assert not eager_inside or torch.equal(a[k], e[k]), k
+            for o, e in zip(wout, warm):
+                for k in ("v", "x", "u"):
+                    assert torch.equal(o[k], e[k]), k
+        except BaseException as e:  # noqa: BLE001 - reported by the test's own thread
+            errors.append(e)
+
+    for eager_inside in (False, True):
+        th = threading.Thread(target=run, args=(eager_inside,))
+        th.start()
+        th.join()
+        assert not errors, errors
