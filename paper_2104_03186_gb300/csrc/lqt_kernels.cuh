@@ -130,6 +130,7 @@ __device__ __forceinline__ void model_prologue(const Params<R>& P, R* sm) {
         for (int e = threadIdx.x; e < p * N; e += blockDim.x) {
             const int a = e / N, i = e % N;
             R t = R(0);
+#pragma unroll 1
             for (int b = 0; b < p; ++b) t += P.H[b * N + i] * P.X[b * p + a];
             sHX[e] = t;
             sH[e] = P.H[e];
@@ -139,6 +140,7 @@ __device__ __forceinline__ void model_prologue(const Params<R>& P, R* sm) {
             const int i = e / N, j = e % N;
             if (i > j) continue;
             R t = R(0);
+#pragma unroll 1
             for (int a = 0; a < p; ++a) t += sHX[a * N + i] * P.H[a * N + j];
             sm[ML::OQ + sym<N>(i, j)] = t;
         }
@@ -282,11 +284,13 @@ __device__ __forceinline__ void load_cost(const Params<R>& P, long long k, const
                 }
             return;
         }
+#pragma unroll 1
         for (int a = 0; a < p; ++a) {
             R y[N];
 #pragma unroll
             for (int j = 0; j < N; ++j) y[j] = R(0);
             R xr = R(0);
+#pragma unroll 1
             for (int b = 0; b < p; ++b) {
                 const R xab = __ldg(X + a * p + b);
 #pragma unroll
@@ -492,7 +496,7 @@ constexpr int tile_threads() {
 // operator's latency: a team level of up to four warps (one per scheduler)
 // takes about 1350 cycles against 2300 for a thread per pair, one of 16 warps
 // 4100.  ONE_CTA: the kernels whose trees are the whole grid's critical path
-// (k_bwd_top, k_solo).  The per-tile kernels of a larger FP32 problem, where
+// (k_bwd_top, k_solo of one pass).  The per-tile kernels of a larger FP32 problem, where
 // 152 CTAs fetch the code of both forms, lost (T = 100003, time-varying model:
 // 249 -> 254 us) and keep the thread form.
 template <typename R, int N, bool ONE_CTA>
@@ -563,7 +567,7 @@ __device__ __forceinline__ bool team_apply_level(R* tree, R* carry, int ts, int 
 // that the single-tile solve (k_solo) runs the same code back to back with
 // its trees left in shared memory.  SOLO: the only tile of the problem; the
 // tree is not stored for another kernel.  The model area `sm` is filled.
-template <typename R, int N, int M, int W, bool SOLO, bool INV>
+template <typename R, int N, int M, int W, bool SOLO, bool INV, bool TEAMS = SOLO>
 __device__ __forceinline__ void bwd_up_body(const Params<R>& P, unsigned tile, R* tree,
                                             const R* sm) {
     using SM = Smem<R, N, M, W>;
@@ -587,7 +591,7 @@ __device__ __forceinline__ void bwd_up_body(const Params<R>& P, unsigned tile, R
 #pragma unroll 1
     for (int h = 1; h < Weff; h <<= 1) {
         const int i = tid * 2 * h;
-        if (team_level<R, N, SOLO>(Weff / (2 * h)))
+        if (team_level<R, N, TEAMS>(Weff / (2 * h)))
             ok2 &= team_combine_level<R, N>(tree, WS, h, Weff / (2 * h), tid);
         else if (i < Weff)
             ok2 &= combine_view<R, N>(ElemView<R, N>{tree + tslot<R>(i), WS},
@@ -624,11 +628,13 @@ __device__ __forceinline__ void terminal_value(const Params<R>& P, Value<R, N>& 
     for (int k = 0; k < Dims<N>::SYM; ++k) z.S[k] = R(0);
 #pragma unroll
     for (int i = 0; i < N; ++i) z.v[i] = R(0);
+#pragma unroll 1
     for (int a = 0; a < pT; ++a) {
         R y[N];
         R xr = R(0);
 #pragma unroll
         for (int j = 0; j < N; ++j) y[j] = R(0);
+#pragma unroll 1
         for (int b = 0; b < pT; ++b) {
             const R xab = P.XT[a * pT + b];
 #pragma unroll
@@ -862,7 +868,7 @@ __device__ __forceinline__ void affine_descend(const R* ftree, R* xs, int Weff) 
 // W); sm: the model area, filled here unless SOLO (the caller filled it).
 // SOLO: the up-sweep's tree is already in `big`, and the value carried into
 // the tile is the terminal value (Lemma LQT_assoc), formed here.
-template <typename R, int N, int M, int W, bool SOLO, bool INV>
+template <typename R, int N, int M, int W, bool SOLO, bool INV, bool TEAMS = SOLO>
 __device__ __forceinline__ void bwd_down_body(const Params<R>& P, unsigned tile,
                                               unsigned char* smem_raw, R* rbuf, R* sm) {
     using SM = Smem<R, N, M, W>;
@@ -918,7 +924,7 @@ __device__ __forceinline__ void bwd_down_body(const Params<R>& P, unsigned tile,
 #pragma unroll 1
     for (int h = Weff / 2; h >= 1; h >>= 1) {
         const int i = tid * 2 * h;
-        if (team_level<R, N, SOLO>(Weff / (2 * h))) {
+        if (team_level<R, N, TEAMS>(Weff / (2 * h))) {
             ok_sing &= team_apply_level<R, N>(tree, carry, WS, h, Weff / (2 * h), tid);
         } else if (i < Weff) {
             Value<R, N> c;
@@ -1280,6 +1286,7 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
                 const R* rk = P.r ? P.r + k * P.sr : nullptr;
                 const R* Hk = cost ? sHm : P.H + k * P.sH;
                 R* rrow = myrow + SM::FR + jj * kRStage;
+#pragma unroll 1
                 for (int a = 0; a < p; ++a) {
                     R h[N];
                     if (cost)
@@ -1329,6 +1336,7 @@ __device__ __forceinline__ void fwd_down_body(const Params<R>& P, unsigned tile,
                     for (int i = 0; i < N; ++i) xT[i] = xn[i];
                 }
                 if (P.refine_emit)
+#pragma unroll 1
                     for (int a = 0; a < P.pT; ++a) {
                         Dot2<R> acc(P.rT ? P.rT[a] : R(0));
 #pragma unroll
@@ -1423,6 +1431,7 @@ __device__ __forceinline__ void load_vec_step(const Params<R>& P, long long k, c
                     for (int i = 0; i < N; ++i) st.q[i] += hx[i] * r4[a];
                 }
         } else {
+#pragma unroll 1
             for (int a = 0; a < p; ++a) {
                 const R ra = __ldg(r + a);
 #pragma unroll
@@ -1439,6 +1448,7 @@ __device__ __forceinline__ void load_vec_step(const Params<R>& P, long long k, c
                 for (int b = 0; b < kRStage; ++b)
                     if (b < p) y += __ldg(X + a * p + b) * r4[b];
             } else {
+#pragma unroll 1
                 for (int b = 0; b < p; ++b) y += __ldg(X + a * p + b) * __ldg(r + b);
             }
             ldg_vals<R, N>(H + a * N, P.vec & VEC_H, h);
@@ -1686,7 +1696,20 @@ struct SoloSmem {
     static size_t bytes(int p) { return SM::bytes(BIG, p); }
 };
 
-template <typename R, int N, int M, int W, bool INV>
+// BOTH: the kernel of both passes of a refined solve.  What a second pass in a
+// kernel of its own costs is its code: a launch's instructions come from the L2
+// once they have left the SM's instruction cache (about 128 KB), and from HBM
+// when other work has run between two solves.  Refined vehicle (n = 4, m = 2,
+// time-invariant), T = 100 and 1000, us, and with the L2 flushed before each
+// solve:
+//   a full second pass (one kernel, 114 KB)         51.1   75.3   52.4   79.0
+//   a kernel for the vector pass (116 + 60 KB)      46.0   67.7   69.4   93.3
+//   both in one, team levels (142 KB)               46.3   69.9   68.7   91.3
+//   both in one, a thread per pair (129 KB)         43.2   66.9   48.3   72.8
+//   and the loops over outputs not unrolled (113)   41.0   65.1   46.2   68.7
+// An unrefined solve has one pass and keeps the team levels (T = 100: 26.4
+// against 28.5 us without them, flushed 29.8 against 34.0).
+template <typename R, int N, int M, int W, bool INV, bool BOTH>
 __global__ void __launch_bounds__(W, 1) k_solo(const Params<R> P) {
     griddep_launch_dependents();
     griddep_wait();
@@ -1696,36 +1719,25 @@ __global__ void __launch_bounds__(W, 1) k_solo(const Params<R> P) {
     R* big = reinterpret_cast<R*>(smem_raw + kSmemHead);
     R* sm = big + BIG + SM::RBUF;
     model_prologue<R, N, M>(P, sm);  // ends with __syncthreads
-    bwd_up_body<R, N, M, W, true, INV>(P, 0, big, sm);
-    __syncthreads();
-    bwd_down_body<R, N, M, W, true, INV>(P, 0, smem_raw, big + BIG + threadIdx.x, sm);
-    __syncthreads();
-    fwd_down_body<R, N, M, W, true, INV>(P, 0, smem_raw, sm);
-}
-
-// The second pass of a one-tile problem: the vector recursions and the rollout.
-template <typename R, int N, int M, int W, bool INV>
-__global__ void __launch_bounds__(W, 1) k_solo_vec(const Params<R> P) {
-    griddep_launch_dependents();
-    griddep_wait();
-    using SM = Smem<R, N, M, W>;
-    using V = VecSmem<R, N, M, W>;
-    constexpr int BIG = SoloSmem<R, N, M, W>::BIG;
-    static_assert(V::MODEL <= BIG, "the value tree fits the common area");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    R* big = reinterpret_cast<R*>(smem_raw + kSmemHead);
-    R* sm = big + BIG + SM::RBUF;
-    R* xs = big + V::XS;
-    model_prologue<R, N, M>(P, sm);  // ends with __syncthreads
-    const TileGeo geo{P.T, 0, P.B};
-    if (threadIdx.x == W - 1) {
-        Value<R, N> z;
-        terminal_value<R, N>(P, z);
+    if (BOTH && P.vector_pass) {
+        using V = VecSmem<R, N, M, W>;
+        static_assert(V::MODEL <= BIG, "the value tree fits the common area");
+        R* xs = big + V::XS;
+        const TileGeo geo{P.T, 0, P.B};
+        if (threadIdx.x == W - 1) {
+            Value<R, N> z;
+            terminal_value<R, N>(P, z);
 #pragma unroll
-        for (int i = 0; i < N; ++i) xs[i * V::WS + tslot<R>(next_pow2(geo.live(W)) - 1)] = z.v[i];
+            for (int i = 0; i < N; ++i)
+                xs[i * V::WS + tslot<R>(next_pow2(geo.live(W)) - 1)] = z.v[i];
+        }
+        vec_up_body<R, N, M, W, true, INV>(P, 0, big, sm);
+        vec_down_body<R, N, M, W, true, INV>(P, 0, big, xs, sm);
+    } else {
+        bwd_up_body<R, N, M, W, true, INV, !BOTH>(P, 0, big, sm);
+        __syncthreads();
+        bwd_down_body<R, N, M, W, true, INV, !BOTH>(P, 0, smem_raw, big + BIG + threadIdx.x, sm);
     }
-    vec_up_body<R, N, M, W, true, INV>(P, 0, big, sm);
-    vec_down_body<R, N, M, W, true, INV>(P, 0, big, xs, sm);
     __syncthreads();
     fwd_down_body<R, N, M, W, true, INV>(P, 0, smem_raw, sm);
 }

@@ -60,14 +60,15 @@ static lqt_status launch_solve_inv(const Params<R>& P, const Plan& plan, cudaStr
     if (plan.solo) {
         // one tile: the whole pass in one CTA
         const size_t smem = SoloSmem<R, N, M, W>::bytes(P.p);
-        if (plan.tiles != 1 || allow_smem(k_solo<R, N, M, W, INV>, done_solo, smem) != cudaSuccess)
-            return plan.tiles != 1 ? LQT_EINVAL : LQT_ECUDA;
-        prof_mark(prof, stream, P.refine_add ? "solo.refine" : "solo");
-        static std::atomic<bool> done_svec[64];
-        if (P.vector_pass &&
-            allow_smem(k_solo_vec<R, N, M, W, INV>, done_svec, smem) != cudaSuccess)
+        // a refined solve runs both its passes through one kernel (see k_solo)
+        static std::atomic<bool> done_both[64];
+        const bool both = P.refine_emit || P.vector_pass;
+        if (plan.tiles != 1) return LQT_EINVAL;
+        if ((both ? allow_smem(k_solo<R, N, M, W, INV, true>, done_both, smem)
+                  : allow_smem(k_solo<R, N, M, W, INV, false>, done_solo, smem)) != cudaSuccess)
             return LQT_ECUDA;
-        if (launch_pdl<R>(P.vector_pass ? k_solo_vec<R, N, M, W, INV> : k_solo<R, N, M, W, INV>, 1,
+        prof_mark(prof, stream, P.refine_add ? "solo.refine" : "solo");
+        if (launch_pdl<R>(both ? k_solo<R, N, M, W, INV, true> : k_solo<R, N, M, W, INV, false>, 1,
                           W, smem, stream, P, true) != cudaSuccess)
             return LQT_ECUDA;
         if (bwd_done && cudaEventRecord(bwd_done, stream) != cudaSuccess) return LQT_ECUDA;
