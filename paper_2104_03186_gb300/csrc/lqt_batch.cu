@@ -133,8 +133,9 @@ static size_t head_bytes(int32_t count) {
 // (lqt_fork.h) forked from the caller's stream after the workspace head is
 // cleared and joined back to it, beside the n = 4 launch on the caller's
 // stream: the sizes are independent, and one size's tree levels and last wave
-// leave most SMs idle.  Batches of fewer steps than this stay on one stream:
-// the fork and joins cost about what they save.
+// leave most SMs idle (48 mixed requests, four sizes: the kernels' times add up
+// to 1.34 ms, the call takes 0.64).  Batches of fewer steps than this stay on
+// one stream: the fork and joins cost about what they save.
 constexpr long long kForkSteps = 1024;
 
 // Workspace bytes of each lane group (its own region, so that the groups may
