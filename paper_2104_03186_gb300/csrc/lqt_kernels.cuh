@@ -22,6 +22,10 @@
 //             and, when refining, the shifted data of the second pass (first
 //             pass) or x* = x^ + xi (second pass).
 //
+// The second pass of a refined solve has the first one's matrices, so it scans
+// vectors: vec_up, fwd_top over the values, vec_down, fwd_top, fwd_down.  A
+// problem of one tile runs each pass as one launch of solo.
+//
 // Per-step records move between HBM and registers through per-warp shared
 // memory rows (WarpRows), so that global accesses are coalesced although each
 // thread walks its own chunk.
