@@ -138,28 +138,29 @@ static size_t head_bytes(int32_t count) {
 // one stream: the fork and joins cost about what they save.
 constexpr long long kForkSteps = 1024;
 
-// Workspace bytes of each lane group (its own region, so that the groups may
-// run at once); false if a group is invalid.
-static bool lane_bytes_of(const lqt_batch_item* items, const std::vector<std::vector<int>>& groups,
-                          std::vector<size_t>* bytes) {
-    bytes->clear();
-    for (const std::vector<int>& g : groups) {
-        size_t b = 0;
-        if (chain_batch_workspace(items, g.data(), (int)g.size(), &b) != LQT_OK) return false;
-        bytes->push_back(up(b));
+// The lane groups' plans and the workspace bytes of the whole batch (a region of
+// its own for each group, so that the groups may run at once); 0 if an item is
+// invalid.
+static size_t plan_batch(const lqt_batch_item* items, int32_t count,
+                         std::vector<ChainPlan>* plans) {
+    const std::vector<std::vector<int>> groups = lane_groups(items, count);
+    plans->resize(groups.size());
+    size_t bytes = head_bytes(count);
+    for (size_t i = 0; i < groups.size(); ++i) {
+        if (chain_batch_plan(items, groups[i].data(), (int)groups[i].size(), &(*plans)[i]) !=
+            LQT_OK)
+            return 0;
+        bytes += up((*plans)[i].bytes);
     }
-    return true;
+    return bytes;
 }
 
 extern "C" size_t lqt_batch_workspace_bytes(const lqt_batch_item* items, int32_t count) {
     if (count < 0 || (count > 0 && !items)) return 0;
     for (int i = 0; i < count; ++i)
         if (check_item(items[i]) != LQT_OK) return 0;
-    std::vector<size_t> bytes;
-    if (!lane_bytes_of(items, lane_groups(items, count), &bytes)) return 0;
-    size_t lane = 0;
-    for (size_t b : bytes) lane += b;
-    return head_bytes(count) + lane;
+    std::vector<ChainPlan> plans;
+    return plan_batch(items, count, &plans);
 }
 
 extern "C" lqt_status lqt_solve_batched(const lqt_batch_item* items, int32_t count,
@@ -170,7 +171,9 @@ extern "C" lqt_status lqt_solve_batched(const lqt_batch_item* items, int32_t cou
         const lqt_status st = check_item(items[i]);
         if (st != LQT_OK) return st;
     }
-    const size_t need = lqt_batch_workspace_bytes(items, count);
+    // cut once: the sizes checked here are those the groups run with
+    std::vector<ChainPlan> plans;
+    const size_t need = plan_batch(items, count, &plans);
     if (need == 0 || workspace_bytes < need) return LQT_ENOMEM;
     // descriptors of the one-CTA-per-problem kernel, grouped by (n, m)
     std::vector<BatchDesc> descs;
@@ -191,12 +194,9 @@ extern "C" lqt_status lqt_solve_batched(const lqt_batch_item* items, int32_t cou
     if (cudaMemsetAsync(base, 0, up(256) + up(64 * sizeof(int)), s) != cudaSuccess)
         return LQT_ECUDA;
     if (count == 0) return LQT_OK;
-    const std::vector<std::vector<int>> groups = lane_groups(items, count);
-    std::vector<size_t> group_bytes;
-    if (!lane_bytes_of(items, groups, &group_bytes)) return LQT_EINVAL;
     long long total_steps = 0;
     for (int i = 0; i < count; ++i) total_steps += items[i].problem.T;
-    const int lanes_running = (int)groups.size();
+    const int lanes_running = (int)plans.size();
     ForkSet* aux = nullptr;
     if (lanes_running >= 1 && lanes_running <= kForkStreams &&
         lanes_running + (descs.empty() ? 0 : 1) >= 2 && total_steps >= kForkSteps)
@@ -228,18 +228,16 @@ extern "C" lqt_status lqt_solve_batched(const lqt_batch_item* items, int32_t cou
                 st = st == LQT_OK ? LQT_ECUDA : st;
         return st;
     };
-    for (size_t i = 0; i < groups.size(); ++i) {
-        const std::vector<int>& g = groups[i];
+    for (size_t i = 0; i < plans.size(); ++i) {
         cudaStream_t gs = s;
         if (aux) {
             gs = aux->s[i];
             if (cudaStreamWaitEvent(gs, aux->fork, 0) != cudaSuccess) return rejoin(LQT_ECUDA);
             forked = (int)i + 1;
         }
-        const lqt_status st = chain_batch_solve(items, g.data(), (int)g.size(), lane_ws,
-                                                group_bytes[i], status, gs);
+        const lqt_status st = chain_batch_solve(plans[i], lane_ws, status, gs);
         if (st != LQT_OK) return rejoin(st);
-        lane_ws += group_bytes[i];
+        lane_ws += up(plans[i].bytes);
     }
     return rejoin(LQT_OK);
 }

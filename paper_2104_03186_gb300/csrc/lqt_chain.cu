@@ -34,11 +34,16 @@ std::mutex g_tune_mu;
 lqt_batch_tune_entry g_tune[kMaxTune];
 int g_tune_count = 0;
 
-// The tuned chunk length for a problem, or 0 (none).
-long long tuned_chunk(int n, long long T) {
+// A copy of the table, for the problems of one batch.
+std::vector<lqt_batch_tune_entry> tune_table() {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    for (int i = 0; i < g_tune_count; ++i)
-        if (g_tune[i].n == n && T <= g_tune[i].t_max) return g_tune[i].chunk_steps;
+    return std::vector<lqt_batch_tune_entry>(g_tune, g_tune + g_tune_count);
+}
+
+// The tuned chunk length for a problem, or 0 (none).
+long long tuned_chunk(const std::vector<lqt_batch_tune_entry>& table, int n, long long T) {
+    for (const lqt_batch_tune_entry& e : table)
+        if (e.n == n && T <= e.t_max) return e.chunk_steps;
     return 0;
 }
 
@@ -114,13 +119,14 @@ lqt_status batch_geometry(const ChainVariant& v, const lqt_batch_item* items, co
     long long fill = (total + slots - 1) / (slots > 0 ? slots : 1);
     if (fill < kMinChunk) fill = kMinChunk;
     const long long Bt = fill < kMaxBatchChunk ? fill : kMaxBatchChunk;
+    const std::vector<lqt_batch_tune_entry> table = tune_table();
     out->resize((size_t)count);
     for (int i = 0; i < count; ++i) {
         const lqt_batch_item& it = items[idx[i]];
         const long long T = it.problem.T;
         // a tuned length applies up to the one that fills the device: a batch
         // with less work than that keeps every resident group busy instead
-        const long long tuned = tuned_chunk(it.problem.n, T);
+        const long long tuned = tuned_chunk(table, it.problem.n, T);
         const long long Bi = tuned > 0 ? (tuned < fill ? tuned : fill) : Bt;
         long long nc = 1;
         while (nc * 2 * Bi <= T && nc < (1LL << 20)) nc *= 2;
@@ -187,32 +193,22 @@ lqt_status chain_solve(const lqt_problem* P, const lqt_solution* sol, bool refin
     return v->run(call, s, prof);
 }
 
-lqt_status chain_batch_workspace(const lqt_batch_item* items, const int* idx, int count,
-                                 size_t* bytes) {
-    *bytes = 0;
-    if (count <= 0) return LQT_OK;
+lqt_status chain_batch_plan(const lqt_batch_item* items, const int* idx, int count,
+                            ChainPlan* plan) {
     const lqt_problem& P0 = items[idx[0]].problem;
-    const ChainVariant* v = find_chain(LQT_F32, P0.n, P0.m, false);
-    if (!v) return LQT_EUNSUPPORTED;
-    std::vector<ChainProblem> probs;
-    const lqt_status st = batch_geometry(*v, items, idx, count, &probs);
+    plan->variant = find_chain(LQT_F32, P0.n, P0.m, false);
+    if (!plan->variant) return LQT_EUNSUPPORTED;
+    const lqt_status st = batch_geometry(*plan->variant, items, idx, count, &plan->probs);
     if (st != LQT_OK) return st;
-    *bytes = v->workspace(probs.data(), count, false, false, false, false);
+    plan->bytes = plan->variant->workspace(plan->probs.data(), count, false, false, false, false);
     return LQT_OK;
 }
 
-lqt_status chain_batch_solve(const lqt_batch_item* items, const int* idx, int count, void* ws,
-                             size_t ws_bytes, int* status, cudaStream_t s) {
-    if (count <= 0) return LQT_OK;
-    const lqt_problem& P0 = items[idx[0]].problem;
-    const ChainVariant* v = find_chain(LQT_F32, P0.n, P0.m, false);
-    if (!v) return LQT_EUNSUPPORTED;
-    std::vector<ChainProblem> probs;
-    const lqt_status st = batch_geometry(*v, items, idx, count, &probs);
-    if (st != LQT_OK) return st;
-    ChainCall call{probs.data(), count, false, false, false, false, ws, ws_bytes, status};
+lqt_status chain_batch_solve(const ChainPlan& plan, void* ws, int* status, cudaStream_t s) {
+    ChainCall call{plan.probs.data(), (int)plan.probs.size(), false, false, false, false, ws,
+                   plan.bytes, status};
     call.persistent = g_batch_mode.load() == LQT_BATCH_PERSISTENT;
-    return v->run(call, s, nullptr);
+    return plan.variant->run(call, s, nullptr);
 }
 
 bool chain_warm_supported(int dtype, int n, int m) {
@@ -239,32 +235,22 @@ lqt_status warm_geometry(const ChainVariant& v, const lqt_batch_item* items, con
 
 }  // namespace
 
-lqt_status chain_warm_workspace(const lqt_batch_item* items, const int* idx, int count,
-                                size_t* bytes) {
-    *bytes = 0;
-    if (count <= 0) return LQT_OK;
+lqt_status chain_warm_plan(const lqt_batch_item* items, const int* idx, int count,
+                           ChainPlan* plan) {
     const lqt_problem& P0 = items[idx[0]].problem;
-    const ChainVariant* v = find_chain(P0.dtype, P0.n, P0.m, false);
-    if (!v) return LQT_EUNSUPPORTED;
-    std::vector<ChainProblem> probs;
-    const lqt_status st = warm_geometry(*v, items, idx, count, &probs);
+    plan->variant = find_chain(P0.dtype, P0.n, P0.m, false);
+    if (!plan->variant) return LQT_EUNSUPPORTED;
+    const lqt_status st = warm_geometry(*plan->variant, items, idx, count, &plan->probs);
     if (st != LQT_OK) return st;
-    *bytes = v->workspace(probs.data(), count, false, false, false, false);
+    plan->bytes = plan->variant->workspace(plan->probs.data(), count, false, false, false, false);
     return LQT_OK;
 }
 
-lqt_status chain_warm_solve(const lqt_batch_item* items, const int* idx, int count, void* ws,
-                            size_t ws_bytes, int* status, cudaStream_t s) {
-    if (count <= 0) return LQT_OK;
-    const lqt_problem& P0 = items[idx[0]].problem;
-    const ChainVariant* v = find_chain(P0.dtype, P0.n, P0.m, false);
-    if (!v) return LQT_EUNSUPPORTED;
-    std::vector<ChainProblem> probs;
-    const lqt_status st = warm_geometry(*v, items, idx, count, &probs);
-    if (st != LQT_OK) return st;
-    ChainCall call{probs.data(), count, false, false, false, false, ws, ws_bytes, status};
+lqt_status chain_warm_solve(const ChainPlan& plan, void* ws, int* status, cudaStream_t s) {
+    ChainCall call{plan.probs.data(), (int)plan.probs.size(), false, false, false, false, ws,
+                   plan.bytes, status};
     call.warm = true;
-    return v->run(call, s, nullptr);
+    return plan.variant->run(call, s, nullptr);
 }
 
 }  // namespace lqt

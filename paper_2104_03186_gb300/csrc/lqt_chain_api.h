@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "lqt.h"
 #include "lqt_lane_step.cuh"
 #include "lqt_launch.cuh"
@@ -112,17 +114,24 @@ lqt_status chain_workspace(const lqt_problem* P, bool refine, bool newton, bool 
 lqt_status chain_solve(const lqt_problem* P, const lqt_solution* sol, bool refine, bool newton,
                        bool sequential, bool method2, bool lean, void* ws, size_t ws_bytes,
                        cudaStream_t s, Prof* prof);
-// Batch of problems of one FP32 (n, m), no refinement: items[idx[0..count)].
-lqt_status chain_batch_workspace(const lqt_batch_item* items, const int* idx, int count,
-                                 size_t* bytes);
-lqt_status chain_batch_solve(const lqt_batch_item* items, const int* idx, int count, void* ws,
-                             size_t ws_bytes, int* status, cudaStream_t s);
+// A batch of problems of one (n, m) cut into chunks, once per call: the bytes of
+// its workspace and its run use the same cut.  (A second cut could be another
+// one: lqt_batch_set_tuning may change the table at any time.)  Its problems
+// point into the caller's items.
+struct ChainPlan {
+    const ChainVariant* variant = nullptr;
+    std::vector<ChainProblem> probs;
+    size_t bytes = 0;
+};
+// Batch of problems of one FP32 (n, m), no refinement: items[idx[0..count)], count > 0.
+lqt_status chain_batch_plan(const lqt_batch_item* items, const int* idx, int count,
+                            ChainPlan* plan);
+lqt_status chain_batch_solve(const ChainPlan& plan, void* ws, int* status, cudaStream_t s);
 // Warm solves (S and K known): the sizes with a chain variant, FP32 or FP64.
 bool chain_warm_supported(int dtype, int n, int m);
-lqt_status chain_warm_workspace(const lqt_batch_item* items, const int* idx, int count,
-                                size_t* bytes);
-lqt_status chain_warm_solve(const lqt_batch_item* items, const int* idx, int count, void* ws,
-                            size_t ws_bytes, int* status, cudaStream_t s);
+lqt_status chain_warm_plan(const lqt_batch_item* items, const int* idx, int count,
+                           ChainPlan* plan);
+lqt_status chain_warm_solve(const ChainPlan& plan, void* ws, int* status, cudaStream_t s);
 
 // lqt_workspace_bytes, and with lean the least that solve_lean takes (lqt_api.cu).
 size_t workspace_bytes(const lqt_problem* prob, const lqt_options* opts, bool lean);

@@ -71,6 +71,21 @@ std::vector<std::vector<int>> warm_groups(const lqt_batch_item* items, int32_t c
     return groups;
 }
 
+// The groups' plans and the workspace bytes of the whole call (a region of its
+// own for each group); 0 if a group is invalid.
+size_t plan_warm(const lqt_batch_item* items, int32_t count, std::vector<ChainPlan>* plans) {
+    const std::vector<std::vector<int>> groups = warm_groups(items, count);
+    plans->resize(groups.size());
+    size_t bytes = up(256);
+    for (size_t i = 0; i < groups.size(); ++i) {
+        if (chain_warm_plan(items, groups[i].data(), (int)groups[i].size(), &(*plans)[i]) !=
+            LQT_OK)
+            return 0;
+        bytes += up((*plans)[i].bytes);
+    }
+    return bytes;
+}
+
 }  // namespace
 }  // namespace lqt
 
@@ -80,13 +95,8 @@ extern "C" size_t lqt_warm_workspace_bytes(const lqt_batch_item* items, int32_t 
     if (count < 0 || (count > 0 && !items)) return 0;
     for (int i = 0; i < count; ++i)
         if (check_warm_item(items[i]) != LQT_OK) return 0;
-    size_t sum = 0;
-    for (const std::vector<int>& g : warm_groups(items, count)) {
-        size_t b = 0;
-        if (chain_warm_workspace(items, g.data(), (int)g.size(), &b) != LQT_OK) return 0;
-        sum += up(b);
-    }
-    return up(256) + sum;
+    std::vector<ChainPlan> plans;
+    return plan_warm(items, count, &plans);
 }
 
 extern "C" lqt_status lqt_solve_warm(const lqt_batch_item* items, int32_t count, void* workspace,
@@ -97,15 +107,16 @@ extern "C" lqt_status lqt_solve_warm(const lqt_batch_item* items, int32_t count,
         const lqt_status st = check_warm_item(items[i]);
         if (st != LQT_OK) return st;
     }
-    const size_t need = lqt_warm_workspace_bytes(items, count);
+    // cut once: the sizes checked here are those the groups run with
+    std::vector<ChainPlan> plans;
+    const size_t need = plan_warm(items, count, &plans);
     if (need == 0 || workspace_bytes < need) return LQT_ENOMEM;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char* base = static_cast<char*>(workspace);
     int* status = reinterpret_cast<int*>(base);
     if (cudaMemsetAsync(base, 0, sizeof(int), s) != cudaSuccess) return LQT_ECUDA;
     char* ws = base + up(256);
-    const std::vector<std::vector<int>> groups = warm_groups(items, count);
-    ForkSet* aux = groups.size() > 1 ? next_fork_set(s) : nullptr;
+    ForkSet* aux = plans.size() > 1 ? next_fork_set(s) : nullptr;
     if (aux && cudaEventRecord(aux->fork, s) != cudaSuccess) return LQT_ECUDA;
     // the auxiliary streams in use rejoin the caller's stream on every return
     // (their work uses the workspace, and a capture must end joined)
@@ -117,11 +128,7 @@ extern "C" lqt_status lqt_solve_warm(const lqt_batch_item* items, int32_t count,
                 st = st == LQT_OK ? LQT_ECUDA : st;
         return st;
     };
-    for (size_t i = 0; i < groups.size(); ++i) {
-        const std::vector<int>& g = groups[i];
-        size_t bytes = 0;
-        lqt_status st = chain_warm_workspace(items, g.data(), (int)g.size(), &bytes);
-        if (st != LQT_OK) return rejoin(st);
+    for (size_t i = 0; i < plans.size(); ++i) {
         cudaStream_t gs = s;
         if (aux && i > 0) {  // group i on set stream (i - 1) mod kForkStreams
             const int q = (int)((i - 1) % kForkStreams);
@@ -131,9 +138,9 @@ extern "C" lqt_status lqt_solve_warm(const lqt_batch_item* items, int32_t count,
                 forked = q + 1;
             }
         }
-        st = chain_warm_solve(items, g.data(), (int)g.size(), ws, up(bytes), status, gs);
+        const lqt_status st = chain_warm_solve(plans[i], ws, status, gs);
         if (st != LQT_OK) return rejoin(st);
-        ws += up(bytes);
+        ws += up(plans[i].bytes);
     }
     return rejoin(LQT_OK);
 }
