@@ -1631,9 +1631,15 @@ __device__ __forceinline__ void vec_down_body(const Params<R>& P, unsigned tile,
 #pragma unroll
             for (int j = 0; j < N; ++j) Phi[i][j] = Pn[i][j];
     }
+    // a value that is not finite stays so down to the chunk's first step (every
+    // entry of w is in every entry of v and y), and a feedforward term in gam
+    bool finite = true;
+#pragma unroll
+    for (int i = 0; i < N; ++i) finite = finite && isfinite(v[i]) && isfinite(gam[i]);
     affine_sweep<R, N, W, SOLO>(ftree, Phi, gam, tid, Weff, P.ftree, Dims<N>::AFFINE * WS,
                                 P.ftile_agg, tile);
     if (!ok) set_status(P.status, ST_NOTSPD);
+    if (!finite) set_status(P.status, ST_NONFINITE);
 }
 
 // Dynamic shared memory of vec_up and vec_down: head, tree and values, model.
