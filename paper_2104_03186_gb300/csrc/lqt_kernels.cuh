@@ -84,7 +84,7 @@ struct Params {
     int out_mask;        // OUT_S | OUT_V | OUT_K: which of S, v, K this pass writes
     int refine_emit;     // first pass of a refined solve: write r', c', r'_T, x'_0
     int refine_add;      // second pass: x <- x + xi instead of x <- xi
-    int keep_maps;       // first pass: keep the chunk maps for the second (kept_map)
+    int keep_maps;       // first pass of several tiles: keep the chunk maps (kept_maps)
     int vector_pass;     // second pass: vector recursions from S, K and those maps
     long long wait_limit;  // polls of each bounded mbarrier wait
     int wait_probe;        // > 0: k_bwd_down also waits this many polls on a barrier
@@ -1028,7 +1028,7 @@ __device__ __forceinline__ void bwd_down_body(const Params<R>& P, unsigned tile,
         WarpRows<R, M, kStageG>::store(P.u, tbase, rows + SM::DD, SM::DROW, lrel, cnt);
         __syncwarp();
     }
-    if (P.keep_maps) {
+    if (!SOLO && P.keep_maps) {
         R* keep = kept_maps<R, N, W>(P.tree, tile);
 #pragma unroll
         for (int i = 0; i < N * N; ++i) keep[i * W + tid] = Phi[i / N][i % N];
@@ -1571,7 +1571,41 @@ __device__ __forceinline__ bool vec_back(const VecStep<R, N, M>& st, R (&v)[N], 
     return ok;
 }
 
-template <typename R, int N, int M, int W, bool SOLO, bool INV>
+// Step k of a downward walk (store: d_k goes to u), with the chunk's forward map:
+// gam <- gam + Phi ct, Phi <- Phi Ft.
+template <typename R, int N, int M, bool INV>
+__device__ __forceinline__ bool vec_walk(const Params<R>& P, long long k, const R* sm, bool store,
+                                         R (&v)[N], R (&Phi)[N][N], R (&gam)[N]) {
+    VecStep<R, N, M> st;
+    load_vec_step<R, N, M, INV>(P, k, sm, st);
+    R d[M], ct[N], Ft[N][N];
+    const bool ok = vec_back(st, v, d, ct, Ft);
+    if (store) {
+        if (M * sizeof(R) == 8 && (P.vec & VEC_K))
+            store_row<R, M>(P.u + k * M, d);  // u is aligned with K, see fill_params
+        else
+#pragma unroll
+            for (int a = 0; a < M; ++a) P.u[k * M + a] = d[a];
+    }
+    R Pn[N][N];
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            gam[i] += Phi[i][j] * ct[j];
+            R t = R(0);
+#pragma unroll
+            for (int l = 0; l < N; ++l) t += Phi[i][l] * Ft[l][j];
+            Pn[i][j] = t;
+        }
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) Phi[i][j] = Pn[i][j];
+    return ok;
+}
+
+template <typename R, int N, int M, int W, bool INV>
 __device__ __forceinline__ void vec_up_body(const Params<R>& P, unsigned tile, R* ftree,
                                             const R* sm) {
     const int tid = threadIdx.x;
@@ -1592,13 +1626,13 @@ __device__ __forceinline__ void vec_up_body(const Params<R>& P, unsigned tile, R
         R d[M], ct[N], Ft[N][N];
         vec_back(st, v, d, ct, Ft);
     }
-    affine_sweep<R, N, W, SOLO>(ftree, Psi, v, Weff - 1 - tid, Weff, P.tree,
+    affine_sweep<R, N, W, false>(ftree, Psi, v, Weff - 1 - tid, Weff, P.tree,
                                 Dims<N>::ELEM * tstride(W, (int)sizeof(R)), P.tile_agg,
                                 P.tiles - 1 - tile);
 }
 
 // xs: the down-swept values, slot Weff - 1 - tid for this thread's chunk
-template <typename R, int N, int M, int W, bool SOLO, bool INV>
+template <typename R, int N, int M, int W, bool INV>
 __device__ __forceinline__ void vec_down_body(const Params<R>& P, unsigned tile, R* ftree, R* xs,
                                               const R* sm) {
     constexpr int WS = tstride(W, (int)sizeof(R));
@@ -1618,40 +1652,72 @@ __device__ __forceinline__ void vec_down_body(const Params<R>& P, unsigned tile,
     }
     __syncthreads();  // the tree area becomes the forward tree
     bool ok = true;
-    for (long long k = e - 1; k >= s; --k) {
-        VecStep<R, N, M> st;
-        load_vec_step<R, N, M, INV>(P, k, sm, st);
-        R d[M], ct[N], Ft[N][N];
-        ok &= vec_back(st, v, d, ct, Ft);
-        if (M * sizeof(R) == 8 && (P.vec & VEC_K))
-            store_row<R, M>(P.u + k * M, d);  // u is aligned with K, see fill_params
-        else
-#pragma unroll
-            for (int a = 0; a < M; ++a) P.u[k * M + a] = d[a];
-        // the chunk's forward map: gam <- gam + Phi ct, Phi <- Phi Ft
-        R Pn[N][N];
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                gam[i] += Phi[i][j] * ct[j];
-                R t = R(0);
-#pragma unroll
-                for (int l = 0; l < N; ++l) t += Phi[i][l] * Ft[l][j];
-                Pn[i][j] = t;
-            }
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-#pragma unroll
-            for (int j = 0; j < N; ++j) Phi[i][j] = Pn[i][j];
-    }
+    for (long long k = e - 1; k >= s; --k)
+        ok &= vec_walk<R, N, M, INV>(P, k, sm, true, v, Phi, gam);
     // a value that is not finite stays so down to the chunk's first step (every
-    // entry of w is in every entry of v and y), and a feedforward term in gam
+    // entry of v is in every entry of the step before's), a feedforward term in gam
     bool finite = true;
 #pragma unroll
     for (int i = 0; i < N; ++i) finite = finite && isfinite(v[i]) && isfinite(gam[i]);
-    affine_sweep<R, N, W, SOLO>(ftree, Phi, gam, tid, Weff, P.ftree, Dims<N>::AFFINE * WS,
+    affine_sweep<R, N, W, false>(ftree, Phi, gam, tid, Weff, P.ftree, Dims<N>::AFFINE * WS,
                                 P.ftile_agg, tile);
+    if (!ok) set_status(P.status, ST_NOTSPD);
+    if (!finite) set_status(P.status, ST_NONFINITE);
+}
+
+// Both over the only tile of a problem: one loop body walks twice, up from v = 0
+// and down from the values, so that the kernel holds the walk's and the sweep's
+// code once (see k_solo).  The map of the upward walk is formed again, from the
+// first pass's K: one tile keeps no maps.
+template <typename R, int N, int M, int W, bool INV>
+__device__ __forceinline__ void vec_solo_body(const Params<R>& P, R* ftree, R* xs, const R* sm) {
+    constexpr int WS = tstride(W, (int)sizeof(R));
+    const int tid = threadIdx.x;
+    const TileGeo geo{P.T, 0, P.B};
+    const int Weff = next_pow2(geo.live(W));
+    long long s, e;
+    geo.chunk(tid, s, e);
+    bool ok = true, finite = true;
+    R v[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = R(0);
+#pragma unroll 1
+    for (int down = 0; down < 2; ++down) {
+        R Phi[N][N], gam[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            gam[i] = R(0);
+#pragma unroll
+            for (int j = 0; j < N; ++j) Phi[i][j] = i == j ? R(1) : R(0);
+        }
+#pragma unroll 1
+        for (long long k = e - 1; k >= s; --k)
+            ok &= vec_walk<R, N, M, INV>(P, k, sm, down != 0, v, Phi, gam);
+        if (down) {  // as in vec_down_body
+#pragma unroll
+            for (int i = 0; i < N; ++i) finite = finite && isfinite(v[i]) && isfinite(gam[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                gam[i] = v[i];
+#pragma unroll
+                for (int j = 0; j < i; ++j) {
+                    const R t = Phi[i][j];
+                    Phi[i][j] = Phi[j][i];
+                    Phi[j][i] = t;
+                }
+            }
+        }
+        affine_sweep<R, N, W, true>(ftree, Phi, gam, down ? tid : Weff - 1 - tid, Weff, nullptr, 0,
+                                    nullptr, 0);
+        if (!down) {
+            affine_descend<R, N, W>(ftree, xs, Weff);
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                v[i] = tid < Weff ? xs[i * WS + tslot<R>(Weff - 1 - tid)] : R(0);
+            __syncthreads();  // the tree area becomes the forward tree
+        }
+    }
     if (!ok) set_status(P.status, ST_NOTSPD);
     if (!finite) set_status(P.status, ST_NONFINITE);
 }
@@ -1675,7 +1741,7 @@ __global__ void __launch_bounds__(W, 1) k_vec_up(const Params<R> P) {
     R* tree = reinterpret_cast<R*>(smem_raw + kSmemHead);
     R* sm = tree + VecSmem<R, N, M, W>::MODEL;
     model_prologue<R, N, M>(P, sm);
-    vec_up_body<R, N, M, W, false, INV>(P, blockIdx.x, tree, sm);
+    vec_up_body<R, N, M, W, INV>(P, blockIdx.x, tree, sm);
 }
 
 template <typename R, int N, int M, int W, bool INV>
@@ -1701,7 +1767,7 @@ __global__ void __launch_bounds__(W, 1) k_vec_down(const Params<R> P) {
         xs[tid * V::WS + tslot<R>(next_pow2(geo.live(W)) - 1)] =
             P.tile_carry[(size_t)mirror * N + tid];
     __syncthreads();
-    vec_down_body<R, N, M, W, false, INV>(P, tile, tree, xs, sm);
+    vec_down_body<R, N, M, W, INV>(P, tile, tree, xs, sm);
     if (!ok_load) set_status(P.status, ST_TIMEOUT);
 }
 
@@ -1731,6 +1797,9 @@ struct SoloSmem {
 //   both in one, team levels (142 KB)               46.3   69.9   68.7   91.3
 //   both in one, a thread per pair (129 KB)         43.2   66.9   48.3   72.8
 //   and the loops over outputs not unrolled (113)   41.0   65.1   46.2   68.7
+// and with the value recursion of vec_back, beside a time-varying model, p = 1:
+//   two walks (117 and 140 KB)     39.1   63.8   46.2   70.8 | 46.7   89.7   64.6  109.7
+//   one walk, run twice (107, 127) 39.1   63.7   44.2   69.8 | 43.1   84.5   48.3   91.3
 // An unrefined solve has one pass and keeps the team levels (T = 100: 26.4
 // against 28.5 us without them, flushed 29.8 against 34.0).
 template <typename R, int N, int M, int W, bool INV, bool BOTH>
@@ -1755,8 +1824,7 @@ __global__ void __launch_bounds__(W, 1) k_solo(const Params<R> P) {
             for (int i = 0; i < N; ++i)
                 xs[i * V::WS + tslot<R>(next_pow2(geo.live(W)) - 1)] = z.v[i];
         }
-        vec_up_body<R, N, M, W, true, INV>(P, 0, big, sm);
-        vec_down_body<R, N, M, W, true, INV>(P, 0, big, xs, sm);
+        vec_solo_body<R, N, M, W, INV>(P, big, xs, sm);
     } else {
         bwd_up_body<R, N, M, W, true, INV, !BOTH>(P, 0, big, sm);
         __syncthreads();
