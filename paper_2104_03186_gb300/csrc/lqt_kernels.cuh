@@ -115,6 +115,31 @@ struct ModelLayout {
     __host__ __device__ static constexpr int size(int p) { return round4(OH(p) + p * N); }
 };
 
+// The cost parts of the model area for many outputs, loops unrolled so that
+// several loads are in flight; out of line, away from the code of the common
+// sizes (condensed blocks of 16 steps, p = 32: a load at a time took 1.20 ms, not
+// 1.17, at T = 10^6; unrolled in every kernel, small problems lost 2 us).
+template <typename R, int N>
+__device__ __noinline__ void cost_model_wide(const R* H, const R* X, int p, R* sHX, R* sH, R* sQ) {
+    for (int e = threadIdx.x; e < p * N; e += blockDim.x) {
+        const int a = e / N, i = e % N;
+        R t = R(0);
+#pragma unroll 8
+        for (int b = 0; b < p; ++b) t += H[b * N + i] * X[b * p + a];
+        sHX[e] = t;
+        sH[e] = H[e];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
+        const int i = e / N, j = e % N;
+        if (i > j) continue;
+        R t = R(0);
+#pragma unroll 8
+        for (int a = 0; a < p; ++a) t += sHX[a * N + i] * H[a * N + j];
+        sQ[sym<N>(i, j)] = t;
+    }
+}
+
 // Fill the model area from the time-invariant inputs (each part only when its
 // stride is 0).  Ends with __syncthreads.
 template <typename R, int N, int M>
@@ -128,7 +153,9 @@ __device__ __forceinline__ void model_prologue(const Params<R>& P, R* sm) {
     }
     if (P.c_invariant)
         for (int e = threadIdx.x; e < N; e += blockDim.x) sm[ML::OC + e] = P.has_c ? P.c[e] : R(0);
-    if (P.cost_invariant) {
+    if (P.cost_invariant && p > 8) {
+        cost_model_wide<R, N>(P.H, P.X, p, sm + ML::OHX, sm + ML::OH(p), sm + ML::OQ);
+    } else if (P.cost_invariant) {
         R* sHX = sm + ML::OHX;
         R* sH = sm + ML::OH(p);
         for (int e = threadIdx.x; e < p * N; e += blockDim.x) {
