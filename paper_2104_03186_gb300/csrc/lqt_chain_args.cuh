@@ -38,7 +38,7 @@ struct Args {
     int* status;
     int out_mask;    // bit 1: write S; bit 2: write K; bit 4: write v
     RT* maps;        // refinement: a copy of every chunk map, or nullptr
-    int first_total; // 1: the totals of the problems' first chunks are wanted (Method 2)
+    int first_total; // 1: the problems' first chunks need whole totals (Method 2)
     int refine_add;  // 1: correction pass: x <- x^ + dx, u_out <- u^ + w - qh
 };
 

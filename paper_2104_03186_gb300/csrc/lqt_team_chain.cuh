@@ -255,10 +255,13 @@ __device__ __forceinline__ void b_tfold(const Args<R, RT>& a, long long c, R* sh
     constexpr int LD = S::Sy::LD, CZ = M, CW = M + N, CO = M + 2 * N;  // columns of the system
     const long long T = D.T;
     const long long lc = c - it.c0, B = it.B;
-    // no suffix holds a problem's first chunk: unless Method 2 wants its total,
-    // it is left neutral
-    const long long e1 = lc * B + B < T ? lc * B + B : T;
-    const long long s0 = lc * B < T ? lc * B : T, e0 = lc == 0 && !a.first_total ? s0 : e1;
+    // no suffix holds a problem's first chunk.  Unless Method 2 wants its total, it
+    // is walked for its status alone: U_k has to be positive definite, which the
+    // re-fold, whose G_k has the terminal cost in S, does not see.  Every U of a
+    // time-invariant one is the G of the chunk's last step (J = 0 there).
+    const long long e0 = lc * B + B < T ? lc * B + B : T;
+    long long s0 = lc * B < T ? lc * B : T;
+    if (lc == 0 && !a.first_total && D.sU == 0 && s0 < e0) s0 = e0 - 1;
     const TeamWalk<R, N, M, TR> wk(D, g);
     if (s0 < e0) wk.stage(D, e0 - 1, sh + S::IN, 0, true, g);
     {
