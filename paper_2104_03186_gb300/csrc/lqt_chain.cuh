@@ -45,6 +45,12 @@
 // at n >= 8 the second pass is vector walks and affine scans (k_vback, k_vfwd),
 // otherwise (n = 4, Method 2, the sequential recursion, the least workspace) the
 // same kernels again; it adds x = x^ + dx, u = u^ + w - U^{-1} h.
+// After a Newton step (FULL) the walks read the corrected S and K, while the maps
+// and G^{-1} kept by the re-fold are those before it.  They carry dx and dv, 1e-5
+// of x and v at most, so their own error (that of the first pass's K, 1e-5 to 1e-2
+// relative) stays below a rounding of x* and u*: the precision study (cond(X_k) =
+// 1e6, T = 8192) has 2.56e-8 and 2.55e-8 with the mixed operators, 2.63e-8 and
+// 2.64e-8 with a full second pass.
 #pragma once
 
 #include <cuda_runtime.h>
