@@ -630,16 +630,11 @@ HostAux* host_aux() {
     return &a;
 }
 
-}  // namespace
-}  // namespace lqt
-
-extern "C" {
-
-size_t lqt_host_solve_bytes(const lqt_problem* prob, const lqt_options* opts) {
-    if (validate(prob, nullptr) != LQT_OK) return 0;
+// Device bytes of a host solve whose workspace takes ws_bytes; 0 if that is 0.
+size_t host_bytes(const lqt_problem* prob, size_t ws_bytes) {
     const size_t es = elem_bytes(prob->dtype);
     const int64_t n = prob->n, m = prob->m, p = prob->p, pT = prob->pT, T = prob->T;
-    size_t total = lqt_workspace_bytes(prob, opts);
+    size_t total = ws_bytes;
     if (total == 0) return 0;
     const size_t in_elems[] = {input_elems(prob->F, n * n, T), input_elems(prob->c, n, T),
                                input_elems(prob->L, n * m, T), input_elems(prob->U, m * m, T),
@@ -654,12 +649,25 @@ size_t lqt_host_solve_bytes(const lqt_problem* prob, const lqt_options* opts) {
     return total;
 }
 
+}  // namespace
+}  // namespace lqt
+
+extern "C" {
+
+size_t lqt_host_solve_bytes(const lqt_problem* prob, const lqt_options* opts) {
+    if (validate(prob, nullptr) != LQT_OK) return 0;
+    return host_bytes(prob, lqt_workspace_bytes(prob, opts));
+}
+
 lqt_status lqt_solve_host(const lqt_problem* hp, const lqt_solution* hs, const lqt_options* opts,
                           void* device_buffer, size_t device_bytes, void* stream) {
     lqt_status st = validate(hp, hs);
     if (st != LQT_OK) return st;
     if (!device_buffer || !aligned(device_buffer, kAlign)) return LQT_EINVAL;
-    const size_t need = lqt_host_solve_bytes(hp, opts);
+    // asked for once: lqt_set_single_tile_chunk may change it at any time, and the
+    // buffer is checked against, and laid out with, the same size
+    const size_t ws_bytes = lqt_workspace_bytes(hp, opts);
+    const size_t need = host_bytes(hp, ws_bytes);
     if (need == 0)
         return find_variant(hp->dtype, hp->n, hp->m) || chain_supported(hp->dtype, hp->n, hp->m)
                    ? LQT_EINVAL
@@ -669,7 +677,6 @@ lqt_status lqt_solve_host(const lqt_problem* hp, const lqt_solution* hs, const l
     const size_t es = elem_bytes(hp->dtype);
     const int64_t n = hp->n, m = hp->m, p = hp->p, pT = hp->pT, T = hp->T;
     char* base = static_cast<char*>(device_buffer);
-    const size_t ws_bytes = lqt_workspace_bytes(hp, opts);
     void* ws = base;
     size_t off = ws_bytes;
     auto put = [&](const void* src, size_t elems) -> const void* {
