@@ -1506,6 +1506,7 @@ lqt_status solve_reduced(const lqt_problem* prob, int32_t B, const lqt_solution*
     RedPlan rp;
     lqt_status st = plan_red(prob, B, opts, base, &rp, cross);
     if (st != LQT_OK) return st;
+    if (rp.cross_ws != cross) return LQT_ENOMEM;  // as in solve_once
     st = lqt_solve_cross(&rp.Pc, &rp.cross, &rp.sc, opts, base, 0, s);
     if (st != LQT_ENOMEM) return st == LQT_OK ? LQT_EINVAL : st;
     const RedVariant* var = find_red(prob->dtype, prob->n, prob->m);
@@ -1539,6 +1540,10 @@ lqt_status solve_once(const lqt_problem* prob, int32_t B, const lqt_solution* so
     if (st == LQT_EUNSUPPORTED)
         return solve_reduced(prob, B, sol, opts, base, pre, shift_add, cross, s);
     if (st != LQT_OK) return st;
+    // the plan starts with the condensed solve's workspace, whose size another
+    // thread may change (lqt_set_single_tile_chunk): only the layout that the
+    // caller's buffer was checked for is used
+    if (cp.cross_ws != cross) return LQT_ENOMEM;
     // argument check of the condensed solve before anything is launched
     st = lqt_solve_cross(&cp.Pc, &cp.cross, &cp.sc, opts, base, 0, s);
     if (st != LQT_ENOMEM) return st == LQT_OK ? LQT_EINVAL : st;
