@@ -28,7 +28,7 @@ def test_buffer_checked_with_the_sizes_used(kind):
         (lambda: lqt.lqt_condensed_workspace_bytes(P, B))
     stop = threading.Event()
     toggler = None
-    before = lqt.lqt_set_single_tile_chunk(8)
+    before = lqt.lqt_set_single_tile_chunk(16)
     try:
         small = size()
         lqt.lqt_set_single_tile_chunk(0)
@@ -48,7 +48,7 @@ def test_buffer_checked_with_the_sizes_used(kind):
         def toggle():
             while not stop.is_set():
                 lqt.lqt_set_single_tile_chunk(0)
-                lqt.lqt_set_single_tile_chunk(8)
+                lqt.lqt_set_single_tile_chunk(16)
 
         toggler = threading.Thread(target=toggle)
         toggler.start()
@@ -61,7 +61,7 @@ def test_buffer_checked_with_the_sizes_used(kind):
         toggler.join()
         torch.cuda.synchronize()
         assert bool((buf[small:] == 0x5A).all())
-        lqt.lqt_set_single_tile_chunk(8)
+        lqt.lqt_set_single_tile_chunk(16)
         assert solve() == lqt.LQT_OK
         torch.cuda.synchronize()
         compare({k: v.double().cpu().numpy() for k, v in out.items()}, oracle_solve(prob),
