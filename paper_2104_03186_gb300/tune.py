@@ -7,12 +7,15 @@ levels of Alg. 1.  Short chunks give more parallel groups and more tree
 levels; long chunks the reverse, and which wins depends on how full the GPU
 is.  The tuner times lqt_solve_batched on this GPU on a synthetic batch shaped
 like the benchmark's ragged batch (diagonal tracking, m = n / 2), choosing the
-chunk length of each (n, T-bucket) in turn with the others fixed, then times
-the three launch modes (one launch per tree level, one persistent launch per
-size, or the automatic mode, which is the per-level launches) with that table
-on the whole batch and on a small batch of the size a
-server forms, and keeps the mode that is fastest on the small batch among
-those within 1% of the best on the whole batch.  The library applies a tuned
+chunk length of each (n, T-bucket) in turn with the others fixed.  A table is
+timed on the whole batch and on its first quarter and sixteenth, and counts with
+the geometric mean: lengths chosen on the whole batch alone gained 1% there and
+lost up to 11% on a quarter of it.  The table is kept if it beats the library's own
+lengths by MIN_GAIN, otherwise the plan has no entries.  Then the two launch modes
+(one launch per run of tree levels, or one persistent launch per size; the
+automatic mode is the first) are timed on the same batches and on a small batch of
+the size a server forms, and the mode that is fastest on the small batch is kept
+among those within 1% of the best on the others.  The library applies a tuned
 length only up to the batch's total steps over the resident lane groups, so
 the small batches of a server keep their short chunks.
 
@@ -20,8 +23,8 @@ the small batches of a server keep their short chunks.
 
 writes the table as JSON (default: tuned_batch_plans.json beside this file),
 which the Python binding applies when it loads the library; --modes-only keeps
-the committed chunk lengths and re-times the launch modes alone.  The
-selection and file logic below needs no GPU.
+the file's chunk lengths, times them against the library's own, and the launch
+modes.  The selection and file logic below needs no GPU.
 """
 from __future__ import annotations
 
@@ -35,6 +38,9 @@ import numpy as np
 
 SIZES = (8, 16)
 MODES = ("per_level", "persistent", "auto")  # lqt_batch_set_tuning's launch modes
+TIMED_MODES = ("per_level", "persistent")    # those that differ: auto is per_level
+SHARES = (1, 4, 16)  # a table is timed on the whole batch, its first quarter and sixteenth
+MIN_GAIN = 0.005  # a table has to beat the untuned plan by more than runs differ
 SMALL_BATCH = 16  # problems in the small batch the launch modes are also timed on
 BUCKETS = ((64, 512), (513, 2048), (2049, 4096))  # T ranges (inclusive)
 CANDIDATES = (8, 16, 32, 64, 128, 256)
@@ -62,6 +68,12 @@ def choose_mode(mix_ms: Dict[str, float], small_ms: Dict[str, float],
     best = min(mix_ms.values())
     near = [m for m in MODES if m in mix_ms and mix_ms[m] <= best * (1.0 + rel)]
     return min(near, key=lambda m: (small_ms.get(m, float("inf")), MODES.index(m)))
+
+
+def keep_table(untuned_ms: float, tuned_ms: float) -> bool:
+    """Whether a table is worth its entries: faster than the library's own chunk
+    lengths by more than MIN_GAIN."""
+    return tuned_ms < untuned_ms * (1.0 - MIN_GAIN)
 
 
 def plan_mode(plan: dict) -> str:
@@ -101,20 +113,22 @@ def load(path: str = DEFAULT_OUT) -> dict:
 # measurement (GPU)
 # ---------------------------------------------------------------------------
 
-def _time_batch(Ps, outs, ws, reps: int) -> float:
+def _time_batch(items, ws, reps: int) -> float:
+    """Median ms of a batch given as a descriptor array (building the descriptors
+    of 4096 problems in Python takes several times as long as solving them)."""
     import torch
 
     from . import lqt
 
     stream = torch.cuda.current_stream()
     for _ in range(2):
-        lqt.lqt_solve_batched(Ps, outs, ws, stream)
+        lqt.lqt_solve_batched_array(items, ws, stream)
     ts = []
     for _ in range(reps):
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         e0.record(stream)
-        lqt.lqt_solve_batched(Ps, outs, ws, stream)
+        lqt.lqt_solve_batched_array(items, ws, stream)
         e1.record(stream)
         e1.synchronize()
         ts.append(e0.elapsed_time(e1))
@@ -125,38 +139,36 @@ def _time_batch(Ps, outs, ws, reps: int) -> float:
 
 
 def _prepared(probs):
-    import torch
-
     from . import lqt
 
     Ps = [lqt.Problem.from_inputs(p, dtype=np.float32) for p in probs]
     outs = [P.allocate_outputs() for P in Ps]
-    return Ps, outs, torch
+    return Ps, outs, np.frombuffer(lqt._items(Ps, outs), dtype=lqt.BATCH_ITEM)[:len(Ps)].copy()
 
 
-def _workspace(Ps, outs):
+def _workspace(items):
     import torch
 
     from . import lqt
 
-    nbytes = lqt.lqt_batch_workspace_bytes(Ps, outs)
+    nbytes = lqt.lqt_batch_workspace_bytes_array(items)
     if nbytes == 0:
         raise lqt.LQTError(lqt.LQT_EUNSUPPORTED, "tuning workspace")
     return torch.empty(nbytes, dtype=torch.uint8, device="cuda")
 
 
-def measure(problems: int = 4096, reps: int = 3, sizes: Sequence[int] = SIZES,
+def measure(problems: int = 4096, reps: int = 7, sizes: Sequence[int] = SIZES,
             buckets=BUCKETS, candidates: Sequence[int] = CANDIDATES, seed: int = 11,
             fixed_entries: Sequence[Tuple[int, int, int]] = ()) -> dict:
     """Tune on this GPU and return the plan.  The best chunk length of a
     bucket depends on what else the batch holds (a batch that fills the GPU
-    favours longer chunks than a small one), so every candidate is timed on
-    the whole mixed batch (the benchmark's distribution, another draw: n
-    uniform in {4, 8, 16}, T uniform in [64, 4096]): one pass of coordinate descent over
-    the (n, T-bucket) entries from the untuned chunk length (64), then the
-    launch modes with the resulting table, on the whole batch and on its first
-    SMALL_BATCH problems.  fixed_entries: keep these (n, t_max, chunk_steps)
-    and time the launch modes alone."""
+    favours longer chunks than a small one), so every candidate is timed on the
+    mixed batch and on parts of it (SHARES; the benchmark's distribution, another
+    draw: n uniform in {4, 8, 16}, T uniform in [64, 4096]): one pass of coordinate
+    descent over the (n, T-bucket) entries from chunks of 64 steps, then the launch
+    modes with the resulting table (or none, see keep_table), also on the first
+    SMALL_BATCH problems.  The plan's times are geometric means over SHARES.
+    fixed_entries: time these (n, t_max, chunk_steps) instead of a search."""
     import torch
 
     from . import inputs, lqt
@@ -173,23 +185,22 @@ def measure(problems: int = 4096, reps: int = 3, sizes: Sequence[int] = SIZES,
 
     with ThreadPoolExecutor(max_workers=os.cpu_count() or 1) as ex:
         mix = list(ex.map(one, range(problems)))
-    Ps, outs, _ = _prepared(mix)
+    Ps, outs, items = _prepared(mix)
     del mix
     table = {(n, t_hi): 64 for n in sizes for (_, t_hi) in buckets}
 
-    def run(tab, mode="per_level", Ps=Ps, outs=outs):
-        lqt.lqt_batch_set_tuning([(n, t, b) for (n, t), b in sorted(tab.items())], mode)
-        ws = _workspace(Ps, outs)
-        ms = _time_batch(Ps, outs, ws, reps)
-        del ws
-        return ms
+    parts = [items[:max(1, len(items) // k)].copy() for k in SHARES]
 
+    def run(tab, mode="per_level", batches=parts):
+        lqt.lqt_batch_set_tuning([(n, t, b) for (n, t), b in sorted(tab.items())], mode)
+        ms = [_time_batch(b, _workspace(b), reps) for b in batches]
+        return float(np.exp(np.mean(np.log(ms))))
+
+    rejected = []
     if fixed_entries:
         table = {(n, t): b for n, t, b in fixed_entries}
-        base_ms, entries = None, [{"n": n, "t_max": t, "chunk_steps": b}
-                                  for n, t, b in fixed_entries]
+        entries = [{"n": n, "t_max": t, "chunk_steps": b} for n, t, b in fixed_entries]
     else:
-        base_ms = run(table)
         timings: Dict[Tuple[int, int], Dict[int, float]] = {}
         for key in sorted(table):
             per_b = {}
@@ -202,14 +213,20 @@ def measure(problems: int = 4096, reps: int = 3, sizes: Sequence[int] = SIZES,
             timings[key] = per_b
             table[key] = min(per_b.items(), key=lambda kv: (kv[1], -kv[0]))[0]
         entries = choose(timings)
-    mix_ms = {m: run(table, m) for m in MODES}
-    small = slice(0, min(SMALL_BATCH, len(Ps)))
-    small_ms = {m: run(table, m, Ps[small], outs[small]) for m in MODES}
+    # the untuned plan and the table in turn, so that drift meets both
+    pairs = [(run({}), run(table)) for _ in range(3)]
+    base_ms, tuned_ms = (min(p[i] for p in pairs) for i in (0, 1))
+    if not keep_table(base_ms, tuned_ms):
+        rejected, entries, table = entries, [], {}
+    mix_ms = {m: run(table, m) for m in TIMED_MODES}
+    small = items[:min(SMALL_BATCH, len(Ps))].copy()
+    small_ms = {m: run(table, m, [small]) for m in TIMED_MODES}
     mode = choose_mode(mix_ms, small_ms)
     lqt.lqt_batch_set_tuning([(n, t, b) for (n, t), b in sorted(table.items())], mode)
     return {"entries": entries, "launch_mode": mode, "mix_ms": mix_ms,
             "small_batch_ms": small_ms, "small_batch": SMALL_BATCH,
-            "untuned_ms": base_ms, "gpu": torch.cuda.get_device_name(0),
+            "untuned_ms": base_ms, "tuned_ms": tuned_ms, "rejected_entries": rejected,
+            "shares": list(SHARES), "gpu": torch.cuda.get_device_name(0),
             "when": time.strftime("%Y-%m-%dT%H:%M:%SZ", time.gmtime()),
             "problems": problems, "candidates": list(candidates),
             "buckets": [list(b) for b in buckets]}
@@ -219,17 +236,13 @@ def main(argv=None) -> int:
     ap = argparse.ArgumentParser(description=__doc__.split("\n")[0])
     ap.add_argument("--out", default=DEFAULT_OUT)
     ap.add_argument("--problems", type=int, default=4096)
-    ap.add_argument("--reps", type=int, default=3)
+    ap.add_argument("--reps", type=int, default=7)
     ap.add_argument("--modes-only", action="store_true",
-                    help="keep the committed chunk lengths, time the launch modes")
+                    help="time the file's chunk lengths instead of a search")
     args = ap.parse_args(argv)
     old = load(args.out) if args.modes_only else None
     plan = measure(args.problems, args.reps,
                    fixed_entries=entries_for(old) if old else ())
-    if old:
-        # the chunk-length timings of the full tuning run stay with their entries
-        plan["entries"], plan["untuned_ms"] = old["entries"], old.get("untuned_ms")
-        plan["candidates"], plan["buckets"] = old["candidates"], old["buckets"]
     save(plan, args.out)
     print(json.dumps({"out": args.out, "launch_mode": plan["launch_mode"],
                       "entries": [(e["n"], e["t_max"], e["chunk_steps"]) for e in plan["entries"]],
