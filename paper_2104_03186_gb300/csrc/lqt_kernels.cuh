@@ -447,31 +447,22 @@ __host__ __device__ __forceinline__ constexpr int tslot(int i) {
     return i + (i >> tree_shift((int)sizeof(R)));
 }
 
-// Factor store of the top-level backward scan (k_bwd_top, modes 1 and 2):
-// the 4 N^2 map entries of each of the up-sweep's combines (combine_view<REC>),
-// then the 2 N^2 of each of the down-sweep's value applies (value_apply<REC>).
-// Entry-major: entry e of node u at e * tp + u (fewer than tp nodes per
-// sweep), so that the threads of a level, which handle consecutive nodes,
-// touch consecutive words.
-__host__ __device__ constexpr int top_fac_up(int n) { return 4 * n * n; }
-__host__ __device__ constexpr int top_fac_dn(int n) { return 2 * n * n; }
-__host__ __device__ constexpr long long top_fac_elems(int n, int tp) {
-    return (long long)tp * (top_fac_up(n) + top_fac_dn(n));
-}
-// Dynamic shared memory of k_bwd_top: the tree and the carries, plus the
-// staged factor store when it replays.
-// Staging area of the tile totals (one per thread at most), whole 16-byte units.
+// Staging area of k_bwd_top's tile totals (one per thread at most), whole 16-byte
+// units.
 __host__ __device__ constexpr long long top_stage_elems(int elem, int tp, int es) {
     return ((long long)tp * elem * es + 15) / 16 * 16 / es;
 }
+// Dynamic shared memory of k_bwd_top: the tree, the carries, the staged totals and
+// the mbarrier of the bulk copy.  maps: and six N x N maps a thread, which no kernel
+// keeps; the host layout check asks whether they would fit.
 __host__ __device__ constexpr long long top_smem_bytes(int elem, int value, int n, int tp,
-                                                       int es, bool replay) {
-    return ((long long)(elem + value) * tstride(tp, es) + (replay ? top_fac_elems(n, tp) : 0) +
+                                                       int es, bool maps) {
+    return ((long long)(elem + value) * tstride(tp, es) + (maps ? 6LL * n * n * tp : 0) +
             top_stage_elems(elem, tp, es)) *
                es +
-           16;  // the mbarrier of the bulk copies
+           16;
 }
-constexpr long long kTopSmemMax = 227 * 1024;
+constexpr long long kTopSmemMax = 227 * 1024;  // opt-in limit of a CTA
 
 template <typename R, int N, int M, int W>
 struct Smem {

@@ -106,8 +106,10 @@ static lqt_status launch_solve_inv(const Params<R>& P, const Plan& plan, cudaStr
         return cudaGetLastError() == cudaSuccess ? LQT_OK : LQT_ECUDA;
     }
     const size_t smem_up = SM::bytes(SM::UP_BIG, P.p);
-    const size_t smem_top = (size_t)top_smem_bytes(Dims<N>::ELEM, Dims<N>::VALUE, N, TP,
-                                                   (int)sizeof(R), false);
+    constexpr long long kTop = top_smem_bytes(Dims<N>::ELEM, Dims<N>::VALUE, N, TP,
+                                              (int)sizeof(R), false);
+    static_assert(kTop <= kTopSmemMax, "the top scan fits one CTA");
+    const size_t smem_top = (size_t)kTop;
     const size_t smem_down = SM::bytes(SM::DOWN_BIG, P.p);
     const size_t smem_ftop = (size_t)(Dims<N>::AFFINE + N) * tstride(TP, (int)sizeof(R)) * sizeof(R);
     const size_t smem_fdown = SM::bytes(SM::FDOWN_BIG, P.p);

@@ -716,7 +716,7 @@ __device__ bool value_apply(const R* P, const R* val, R* out, R* sh, const Team<
     return ok;
 }
 
-// f2 after f1: (F2 F1, F2 c1 + c2) into out (may be f1 or f2).  sh: 2 N^2 + N.
+// f2 after f1: (F2 F1, F2 c1 + c2) into out (may be f1 or f2).  sh: 2 N^2.
 template <int N, typename R>
 __device__ void affine_compose(const R* f1, const R* f2, R* out, R* sh, const Team<N>& g) {
     using A = DAffine<N>;
