@@ -104,7 +104,8 @@ typedef struct {
  *   u*_k = -K_k x*_k + d_k is often a small difference of large terms
  *   (tracking a slowly varying reference), so FP32 rounding of S, v and x is
  *   amplified in u*; ill-conditioned costs amplify it in every output.
- *   n <= 4 (LQT_REFINE_ON and LQT_REFINE_FULL alike): the solve runs twice,
+ *   n <= 4 (LQT_REFINE_ON, and LQT_REFINE_FULL but for (n, m) = (4, 2) with
+ *   p, pT <= 8, which takes FULL's form below): the solve runs twice,
  *   first on the problem, then on the same problem shifted by the first
  *   trajectory x^ (x = x^ + xi: r'_k = r_k - H_k x^_k,
  *   c'_k = F_k x^_k + c_k - x^_{k+1}, r'_T = r_T - H_T x^_T, x'_0 = 0), whose
@@ -128,8 +129,8 @@ typedef struct {
 enum { LQT_REFINE_OFF = 0, LQT_REFINE_ON = 1, LQT_REFINE_AUTO = 2, LQT_REFINE_FULL = 3 };
 /* method: trajectory recovery (Sec. IV-C).  LQT_METHOD_DEFAULT (0) and
  *   LQT_METHOD_1 take Method 1 (Lemma LQT_trajectory_combination: a forward
- *   scan of the closed-loop affine maps from x_0).  LQT_METHOD_2 (n = 8, 16, 32
- *   only; LQT_EUNSUPPORTED otherwise) takes Method 2 (Lemma
+ *   scan of the closed-loop affine maps from x_0).  LQT_METHOD_2 (n = 8,
+ *   16, 32, and (4, 2) with p, pT <= 8; LQT_EUNSUPPORTED otherwise) takes Method 2 (Lemma
  *   LQT_trajectory_method2): a forward scan of the same elements seeded with
  *   (0, x_0, 0, 0, 0) (Remark LQT_init2) gives V_{S->k}, and
  *   x*_k = (I + C_{S,k} S_k)^{-1} (b_{S,k} + C_{S,k} v_k) (eq. lqt_method_2);
@@ -137,8 +138,8 @@ enum { LQT_REFINE_OFF = 0, LQT_REFINE_ON = 1, LQT_REFINE_AUTO = 2, LQT_REFINE_FU
 enum { LQT_METHOD_DEFAULT = 0, LQT_METHOD_1 = 1, LQT_METHOD_2 = 2 };
 /* wait_probe_polls: diagnostic of the bounded device waits (n <= 4 sizes
  *   only; LQT_EUNSUPPORTED elsewhere).  0 (the default) does nothing.  When
- *   positive, the backward down-sweep kernel of each pass also waits on a
- *   barrier that nothing completes, giving up after this many polls: exactly
+ *   positive, the backward down-sweep kernel (a refined solve: its first pass's)
+ *   also waits on a barrier that nothing completes, giving up after this many polls: exactly
  *   what a bulk copy that never lands would cause.  The wait runs out, the
  *   kernel records LQT_ETIMEOUT in the status word and carries on, so the
  *   solve still writes its outputs and lqt_workspace_status() returns

@@ -1408,7 +1408,7 @@ __global__ void __launch_bounds__(W, 1) k_fwd_down(const Params<R> P) {
 //             u) and the offset of its forward map, the in-tile forward sweep;
 // then fwd_top and fwd_down as in the first pass.  An element pass folds 44
 // numbers a step through 4 x 4 operators of 2300 cycles a tree level; the
-// vectors take a quarter of the arithmetic and levels of 500 cycles, for 96
+// vectors take a third of the arithmetic and levels of 500 cycles, for 96
 // bytes a step of S and K to read back.
 // ===========================================================================
 template <typename R, int N, int M>
