@@ -315,22 +315,27 @@ __device__ __forceinline__ void load_cost(const Params<R>& P, long long k, const
                 }
             return;
         }
+        // two terms at a time: one waits for every load in turn, four evict one
+        // another's lines.  n = 4, p = 8, unrefined, with a scalar load per entry of H
+        // and 1 term / rows of H by 16 bytes and 1, 2, 4 terms, us: T = 100 69.3 / 57.5,
+        // 47.2, 48.7; T = 1000 481 / 341, 253, 279; T = 30000 242 / 140, 140, 141
 #pragma unroll 1
         for (int a = 0; a < p; ++a) {
             R y[N];
 #pragma unroll
             for (int j = 0; j < N; ++j) y[j] = R(0);
             R xr = R(0);
-#pragma unroll 1
+#pragma unroll 2
             for (int b = 0; b < p; ++b) {
                 const R xab = __ldg(X + a * p + b);
+                R hb[N];
+                ldg_vals<R, N>(H + b * N, P.vec & VEC_H, hb);
 #pragma unroll
-                for (int j = 0; j < N; ++j) y[j] += xab * __ldg(H + b * N + j);
+                for (int j = 0; j < N; ++j) y[j] += xab * hb[j];
                 if (r) xr += xab * __ldg(r + b);
             }
             R h[N];
-#pragma unroll
-            for (int i = 0; i < N; ++i) h[i] = __ldg(H + a * N + i);
+            ldg_vals<R, N>(H + a * N, P.vec & VEC_H, h);
 #pragma unroll
             for (int i = 0; i < N; ++i) {
                 st.q[i] += h[i] * xr;
